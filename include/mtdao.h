@@ -265,6 +265,9 @@ int mtdao_step(mtdao_handle h, const void *grads_dev, int32_t grad_dtype, double
  * grads_dev + k * grads_stride_bytes (stride 0: the same buffer for every
  * step; otherwise a multiple of 16) and uses lrs[k] (host array of count
  * doubles).  Stops at the first failing step (t counts the steps done).
+ * Steps with no average between them share one launch that reads and writes
+ * every state once (up to 64 steps): the states in memory are those of the
+ * step before only at an average and when the call's work has completed.
  */
 int mtdao_run(mtdao_handle h, const void *grads_dev, int64_t grads_stride_bytes, int32_t grad_dtype,
               const double *lrs, int32_t count);

@@ -25,6 +25,8 @@ template <int BASE>
 cudaError_t launch_step_base(int, int, bool, const StepArgs &, int, cudaStream_t);
 template <int BASE>
 cudaError_t launch_step_sync_base(int, int, bool, const StepArgs &, int, cudaStream_t);
+template <int BASE>
+cudaError_t launch_step_run_base(int, int, const RunArgs &, cudaStream_t);
 extern template cudaError_t launch_step_base<MTDAO_BASE_ADAM>(int, int, bool, const StepArgs &, int,
                                                               cudaStream_t);
 extern template cudaError_t launch_step_base<MTDAO_BASE_ADOPT>(int, int, bool, const StepArgs &, int,
@@ -37,6 +39,21 @@ extern template cudaError_t launch_step_sync_base<MTDAO_BASE_ADOPT>(int, int, bo
                                                                     int, cudaStream_t);
 extern template cudaError_t launch_step_sync_base<MTDAO_BASE_SGDM>(int, int, bool, const StepArgs &,
                                                                    int, cudaStream_t);
+extern template cudaError_t launch_step_run_base<MTDAO_BASE_ADAM>(int, int, const RunArgs &,
+                                                                  cudaStream_t);
+extern template cudaError_t launch_step_run_base<MTDAO_BASE_ADOPT>(int, int, const RunArgs &,
+                                                                   cudaStream_t);
+extern template cudaError_t launch_step_run_base<MTDAO_BASE_SGDM>(int, int, const RunArgs &,
+                                                                  cudaStream_t);
+
+cudaError_t launch_step_run(int base, int n_mom, int gdt, const RunArgs &a, cudaStream_t st) {
+    switch (base) {
+        case MTDAO_BASE_ADAM: return launch_step_run_base<MTDAO_BASE_ADAM>(n_mom, gdt, a, st);
+        case MTDAO_BASE_ADOPT: return launch_step_run_base<MTDAO_BASE_ADOPT>(n_mom, gdt, a, st);
+        case MTDAO_BASE_SGDM: return launch_step_run_base<MTDAO_BASE_SGDM>(n_mom, gdt, a, st);
+        default: return cudaErrorInvalidValue;
+    }
+}
 
 cudaError_t launch_step(int base, int n_mom, int gdt, bool clip, const StepArgs &a, int sms,
                         cudaStream_t st) {
@@ -75,7 +92,7 @@ struct mtdao_ctx {
     int num_sms = 1;
     cudaStream_t stream = nullptr;
     float *arena = nullptr;
-    float *clip_scale = nullptr;      // [M]
+    float *clip_scale = nullptr;      // [kRunMaxSteps][M] (a single step uses the first row)
     double *norm_out = nullptr;       // [M]
     double *norm_partial = nullptr;   // [M][norm_blocks]
     int norm_blocks = 1;
@@ -430,7 +447,8 @@ extern "C" int mtdao_create(const mtdao_config *cfg, int32_t M, const int64_t *n
         const char *what;
     } allocs[] = {
         {reinterpret_cast<void **>(&h->arena), arena_elems * sizeof(float), "state arena"},
-        {reinterpret_cast<void **>(&h->clip_scale), M * sizeof(float), "clip factors"},
+        {reinterpret_cast<void **>(&h->clip_scale),
+         static_cast<size_t>(kRunMaxSteps) * M * sizeof(float), "clip factors"},
         {reinterpret_cast<void **>(&h->norm_out), M * sizeof(double), "norm output"},
         {reinterpret_cast<void **>(&h->norm_partial),
          static_cast<size_t>(M) * h->norm_blocks * sizeof(double), "norm partials"},
@@ -626,6 +644,68 @@ extern "C" int mtdao_step(mtdao_handle h, const void *grads_dev, int32_t grad_dt
     return MTDAO_OK;
 }
 
+// How many of the next `count` steps one launch takes (step_run.cuh): those
+// before the next that brings an average, which is a step of its own (its
+// average is fused in).  1 also where a launch of several would not give what
+// single steps give: the first step of the original ADOPT order, gradients
+// that lie in the state arena itself (a later step is to read what an earlier
+// one wrote), a bad argument (the single step reports it).
+static int32_t run_length(const mtdao_ctx *h, const char *grads, int64_t stride, int32_t grad_dtype,
+                          const double *lrs, int32_t count) {
+    if (!aligned16(grads) || (grad_dtype != MTDAO_F32 && grad_dtype != MTDAO_BF16)) return 1;
+    if (h->cfg.base == MTDAO_BASE_ADOPT && h->cfg.adopt_prev_v && h->step == 0) return 1;
+    const int32_t most = count < kRunMaxSteps ? count : kRunMaxSteps;
+    const int64_t elems = static_cast<int64_t>(h->M) * h->n_padded;
+    const uintptr_t g0 = reinterpret_cast<uintptr_t>(grads);
+    const uintptr_t g1 = g0 + static_cast<uintptr_t>((most - 1) * stride + elems * (grad_dtype == MTDAO_F32 ? 4 : 2));
+    const uintptr_t a0 = reinterpret_cast<uintptr_t>(h->arena);
+    const uintptr_t a1 = a0 + static_cast<uintptr_t>(elems) * h->n_states * sizeof(float);
+    if (g0 < a1 && a0 < g1) return 1;
+    int32_t k = 0;
+    while (k < most) {
+        if (!std::isfinite(lrs[k]) || due_mask(&h->cfg, h->step + k) != 0u) break;
+        ++k;
+    }
+    return k < 1 ? 1 : k;
+}
+
+// `count` steps in one launch, for a count that run_length gave.
+static int enqueue_run(mtdao_ctx *h, const char *grads, int64_t stride, int32_t grad_dtype, const double *lrs,
+                       int32_t count) {
+    if (int rc = select_device(h)) return rc;
+    const mtdao_config *c = &h->cfg;
+    const bool clip = c->clip_mode == MTDAO_CLIP_GLOBAL_NORM;
+    for (int32_t k = 0; clip && k < count; ++k) {
+        cudaError_t e = launch_grad_sqnorm(grads + k * stride, grad_dtype, h->M, h->n_padded, h->norm_blocks,
+                                           h->norm_partial, h->norm_out, h->clip_scale + k * h->M, c->clip_rho,
+                                           h->stream);
+        if (e != cudaSuccess) return cuda_fail(h, e, "gradient norm launch");
+    }
+    RunArgs a;
+    std::memset(&a, 0, sizeof a);
+    a.arena = h->arena;
+    a.grads = grads;
+    a.clip_scale = clip ? h->clip_scale : nullptr;
+    a.grad_stride = stride;
+    a.n_padded = h->n_padded;
+    a.stride = static_cast<int64_t>(h->M) * h->n_padded;
+    a.M = h->M;
+    a.count = count;
+    for (int32_t k = 0; k < count; ++k) {
+        const StepScalars sc = step_scalars(c, h->step + k, lrs[k]);
+        if (k == 0) a.sc = sc;
+        RunStep &r = a.steps[k];
+        r.neg_lr = sc.neg_lr;
+        r.sv = sc.sv;
+        r.clip_c = sc.clip_c;
+        for (int j = 0; j < c->n_mom; ++j) r.k[j] = sc.k[j];
+    }
+    cudaError_t e = launch_step_run(c->base, c->n_mom, grad_dtype, a, h->stream);
+    if (e != cudaSuccess) return cuda_fail(h, e, "step launch");
+    h->step += count;
+    return MTDAO_OK;
+}
+
 extern "C" int mtdao_run(mtdao_handle h, const void *grads_dev, int64_t grads_stride_bytes,
                          int32_t grad_dtype, const double *lrs, int32_t count) {
     Range range("mtdao_run");
@@ -634,9 +714,14 @@ extern "C" int mtdao_run(mtdao_handle h, const void *grads_dev, int64_t grads_st
         return set_error(h, MTDAO_ERR_INVALID, "run: bad count or NULL arguments");
     if (grads_stride_bytes < 0 || grads_stride_bytes % 16 != 0)
         return set_error(h, MTDAO_ERR_ALIGN, "run: gradient stride must be a non-negative multiple of 16");
-    for (int32_t k = 0; k < count; ++k) {
-        const void *g = static_cast<const char *>(grads_dev) + static_cast<int64_t>(k) * grads_stride_bytes;
-        if (int rc = mtdao_step(h, g, grad_dtype, lrs[k], due_mask(&h->cfg, h->step))) return rc;
+    int32_t k = 0;
+    while (k < count) {
+        const char *g = static_cast<const char *>(grads_dev) + static_cast<int64_t>(k) * grads_stride_bytes;
+        const int32_t together = run_length(h, g, grads_stride_bytes, grad_dtype, lrs + k, count - k);
+        const int rc = together > 1 ? enqueue_run(h, g, grads_stride_bytes, grad_dtype, lrs + k, together)
+                                    : mtdao_step(h, g, grad_dtype, lrs[k], due_mask(&h->cfg, h->step));
+        if (rc != MTDAO_OK) return rc;
+        k += together;
     }
     return MTDAO_OK;
 }

@@ -49,6 +49,28 @@ struct StepArgs {
     StepScalars sc;
 };
 
+// What changes from one step to the next within one launch of several.
+struct RunStep {
+    float neg_lr, sv, clip_c;        // as in StepScalars
+    float k[MTDAO_MAX_MOM];
+};
+
+// Steps of one launch: the array travels in the kernel's parameters (4 KB).
+constexpr int kRunMaxSteps = 64;
+
+struct RunArgs {
+    float *arena;
+    const void *grads;               // step k's [M][n_padded] gradients at grads + k * grad_stride bytes
+    const float *clip_scale;         // [count][M] global-norm clip factors, or nullptr
+    int64_t grad_stride;
+    int64_t n_padded;
+    int64_t stride;
+    int32_t M;
+    int32_t count;                   // 1 .. kRunMaxSteps
+    StepScalars sc;                  // what does not change with the step
+    RunStep steps[kRunMaxSteps];
+};
+
 struct SyncArgs {
     float *arena;
     int64_t n_padded;
@@ -67,6 +89,10 @@ cudaError_t launch_step(int base, int n_mom, int grad_dtype, bool clip, const St
 // otherwise (the caller then runs launch_step followed by launch_sync).
 cudaError_t launch_step_sync(int base, int n_mom, int grad_dtype, bool clip, const StepArgs &a,
                              int num_sms, cudaStream_t stream);
+
+// count consecutive local steps with no average, the states read and written
+// once.
+cudaError_t launch_step_run(int base, int n_mom, int grad_dtype, const RunArgs &a, cudaStream_t stream);
 
 // Step 0 of the original ADOPT order: v = g^2 over count elements (all
 // replicas' v slabs, contiguous), nothing else touched.

@@ -1,6 +1,7 @@
 // step_adam.cu -- instantiates the local-step kernels of Algorithm 1 (MT-DAO-Adam).
 // One translation unit per base so that the instantiations compile in parallel.
 #include "step_kernels.cuh"
+#include "step_run.cuh"
 #include "step_sync_kernels.cuh"
 
 namespace mtdao {
@@ -9,5 +10,6 @@ template cudaError_t launch_step_base<MTDAO_BASE_ADAM>(int, int, bool, const Ste
                                                 cudaStream_t);
 template cudaError_t launch_step_sync_base<MTDAO_BASE_ADAM>(int, int, bool, const StepArgs &, int,
                                                      cudaStream_t);
+template cudaError_t launch_step_run_base<MTDAO_BASE_ADAM>(int, int, const RunArgs &, cudaStream_t);
 
 }  // namespace mtdao

@@ -93,8 +93,12 @@ __device__ __forceinline__ float step_acc_init(const StepScalars &sc, float g, f
 // would form inf - inf = NaN where beta * s is s itself (beta > 0), so an
 // infinite state stays infinite from one step to the next, as it does in
 // exact arithmetic; c = 1 (beta = 0) keeps the fma's NaN, which is 0 * inf.
+// Without GUARD an infinite s gives the NaN: for a caller that looks for NaN
+// afterwards and then repeats the work with the guard.
+template <bool GUARD = true>
 __device__ __forceinline__ float ema_decay(float c, float s) {
     const float d = fmaf(-c, s, s);
+    if constexpr (!GUARD) return d;
     return (fabsf(s) == __int_as_float(0x7f800000) && c < 1.0f) ? s : d;
 }
 
@@ -104,7 +108,7 @@ __device__ __forceinline__ float ema_decay(float c, float s) {
 // With st visited in state_order this is Algorithm 1 (Adam), 2 (ADOPT) or
 // 3 (SGDM) for the element; every EMA is beta * s + (1 - beta) * target in
 // the fma form described with StepScalars.
-template <int BASE, int N>
+template <int BASE, int N, bool GUARD = true>
 __device__ __forceinline__ void update_state(const StepScalars &sc, int st, float g, float s, float &gt,
                                              float &acc, float &cur) {
     if (st == 1 + N && BASE == MTDAO_BASE_ADOPT) {
@@ -114,9 +118,9 @@ __device__ __forceinline__ void update_state(const StepScalars &sc, int st, floa
         float gn;
         if (sc.prev_v) {
             gn = g / (sqrtf(cur) + sc.eps);
-            cur = fmaf(__fmul_rn(sc.c2, g), g, ema_decay(sc.c2, cur));
+            cur = fmaf(__fmul_rn(sc.c2, g), g, ema_decay<GUARD>(sc.c2, cur));
         } else {
-            cur = fmaf(__fmul_rn(sc.c2, g), g, ema_decay(sc.c2, cur));
+            cur = fmaf(__fmul_rn(sc.c2, g), g, ema_decay<GUARD>(sc.c2, cur));
             gn = g / (sqrtf(cur) + sc.eps);
         }
         gn = gn > sc.clip_c ? sc.clip_c : (gn < -sc.clip_c ? -sc.clip_c : gn);  // keeps NaN
@@ -125,7 +129,7 @@ __device__ __forceinline__ void update_state(const StepScalars &sc, int st, floa
     } else if (st == 1 + N) {
         // Algorithm 1: v of the raw gradient, then the denominator
         // sqrt(v / b_v) + eps of the momenta's combination.
-        cur = fmaf(__fmul_rn(sc.c2, g), g, ema_decay(sc.c2, cur));
+        cur = fmaf(__fmul_rn(sc.c2, g), g, ema_decay<GUARD>(sc.c2, cur));
         acc = acc / fmaf(sqrtf(cur), sc.sv, sc.eps);
     } else if (st == 0) {
         cur = fmaf(sc.neg_lr, acc, cur);                     // x - eta_t Delta
@@ -133,7 +137,7 @@ __device__ __forceinline__ void update_state(const StepScalars &sc, int st, floa
         // momentum u_j of clip(g) (Adam, SGDM) or of ADOPT's clamped g
         const int j = st - 1;
         const float target = BASE == MTDAO_BASE_ADOPT ? gt : __fmul_rn(g, s);
-        cur = fmaf(sc.c1[j], target, ema_decay(sc.c1[j], cur));
+        cur = fmaf(sc.c1[j], target, ema_decay<GUARD>(sc.c1[j], cur));
         acc = fmaf(sc.k[j], cur, acc);
     }
 }
