@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(kWideMaxThreads) sync_stats_wide_kernel(const 
         cp_async_wait<1>();                      // this thread's copies of `span` have landed
         __syncthreads();                         // ... and every thread's
         const float *tile = tiles + buf * M * S;
-        tile_means<FOUR>(tile, M, log2_s, S, mean);
+        tile_means<FOUR ? 4 : 1>(tile, M, log2_s, S, mean);
         __syncthreads();
         if (live) {
             float p0 = 0.0f, p1 = 0.0f, p2 = 0.0f, p3 = 0.0f;   // this thread's 4 * NV elements
@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(kWideMaxThreads) pseudo_grad_stats_wide_kernel
         __syncthreads();
         const float *tile = tiles + buf * R * S;
         const float *anc = tile + M * S;
-        tile_means<FOUR>(tile, M, log2_s, S, mean);
+        tile_means<FOUR ? 4 : 1>(tile, M, log2_s, S, mean);
         __syncthreads();
         if (live) {
             float p0 = 0.0f, p1 = 0.0f, p2 = 0.0f, p3 = 0.0f;   // this thread's 4 * NV elements

@@ -2,7 +2,7 @@
 //
 // step_sync_kernel is element-major: a lane updates the same few elements
 // of all M replicas (M <= 7) or of half of them while the other half-warp
-// holds the rest (M = 8; see FusedShape), with the update of
+// holds the rest (M = 8 on smaller states; see FusedShape), with the update of
 // step_kernels.cuh; then it writes each state due for averaging as the
 // replica mean (E_m[.] of Algorithms 1-3) instead of the local values.  The
 // average costs no HBM traffic beyond the step's own.
@@ -24,13 +24,11 @@ namespace mtdao {
 //   M = 8       : two groups (half-warps) of R = 4, V = 4: replicas 0..3 and
 //                 4..7 are the two parts of the compensated mean of
 //                 replica_mean.cuh, combined by shuffles.
-// M from 9 to 64 take the block-staged kernel of step_sync_wide.cuh (lane
-// groups went further before: M = 16 as four groups of four replicas, the
-// compensated sums handed from group to group by shuffles, ran at 4.9-5.3
-// TB/s against 5.2 for the block-staged kernel with every state due and 5.7
-// against 6.8 with x alone; M = 32 as eight groups loaded 64-byte pieces of
-// eight replica slabs and ran slower than the separate average); above 64,
-// the plain step followed by the standalone average.
+// M = 8 on large states and M from 9 to 256 take the tiled kernel of
+// step_sync_wide.cuh (lane groups went further before: M = 16 as four groups
+// of four replicas, the compensated sums handed from group to group by
+// shuffles, ran at 4.9-5.3 TB/s against 6.7-6.9); above 256, the plain step
+// followed by the standalone average.
 // The states are visited one after another (state_order); the next
 // state's loads are issued before the current state is updated and stored,
 // so two states' loads are in flight per lane within the 128-register cap.
@@ -285,8 +283,13 @@ cudaError_t launch_step_sync_m(const StepArgs &a, int num_sms, cudaStream_t st) 
         case 5: return launch_step_sync_t<BASE, N, GDT, CLIP, 5>(a, num_sms, st);
         case 6: return launch_step_sync_t<BASE, N, GDT, CLIP, 6>(a, num_sms, st);
         case 7: return launch_step_sync_t<BASE, N, GDT, CLIP, 7>(a, num_sms, st);
-        case 8: return launch_step_sync_t<BASE, N, GDT, CLIP, 8>(a, num_sms, st);
-        default: return launch_step_sync_wide<BASE, N, GDT, CLIP>(a, num_sms, st);
+        case 8:
+            // flat vectors, GB/s here / tiled: n = 200k (in L2) 3742 / 2724,
+            // 1M (Adam N = 3) 5865 / 5544, 4M (bf16) 5992 / 6245, 20M 6417-6592
+            // / 6553-6939 (Adam, ADOPT, SGDM, N = 1 to 4)
+            if (a.n_padded < int64_t{1} << 21) return launch_step_sync_t<BASE, N, GDT, CLIP, 8>(a, num_sms, st);
+            return launch_step_sync_tile<BASE, N, GDT, CLIP>(a, num_sms, st);
+        default: return launch_step_sync_tile<BASE, N, GDT, CLIP>(a, num_sms, st);
     }
 }
 

@@ -1,0 +1,88 @@
+"""The tiled fused step (step_sync_wide.cuh): the step and the averages in one
+pass give the bits of the step followed by the averages, at the edges of what
+the tile's width and threads are chosen by."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from parity_util import workload_dict
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def P():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2510_05361_gb300 as P
+    P.load()
+    return P
+
+
+def _pair(P, w, M, gdt, seed, plant=False):
+    engines = [P.MTDAO(w["opt"], M, w["shapes"]) for _ in range(2)]
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    n = engines[0].n_padded
+    for s in range(engines[0].n_states):
+        vals = torch.randn((M, n), device="cuda", generator=gen) * 0.02
+        if s == engines[0].n_states - 1:
+            vals = vals.abs()
+        if plant:
+            vals[M // 2, 5::97] = float("inf")
+            vals[M - 1, 7::89] = float("nan")
+        for e in engines:
+            e.state_view(s).copy_(vals)
+    g = torch.randn((M, n), device="cuda", generator=gen) * 0.01
+    return engines, g.to(torch.bfloat16) if gdt == "bf16" else g
+
+
+def _same(a, b):
+    for s in range(a.n_states):
+        x, y = a.state_view(s), b.state_view(s)
+        nan = torch.isnan(x)
+        assert torch.equal(nan, torch.isnan(y)), s
+        assert torch.equal(torch.where(nan, 0.0, x), torch.where(nan, 0.0, y)), s
+
+
+# (M, numel): one tile, an SM's worth of tiles, tiles of every width; M = 8 from
+# 2^21 elements on; the largest tile set that fits (M = 256, N = 4, f32); above it
+CASES = [("adam", 4, "f32", 256, 30000), ("adam", 1, "f32", 256, 512), ("sgdm", 1, "bf16", 256, 1),
+         ("adopt", 2, "bf16", 255, 5000), ("adopt", 2, "bf16", 8, 1 << 21), ("sgdm", 3, "f32", 8, (1 << 21) - 256),
+         ("adam", 2, "f32", 9, 150000), ("adopt", 1, "f32", 16, 20000), ("sgdm", 2, "bf16", 17, 10001),
+         ("adam", 3, "f32", 48, 9999), ("adam", 4, "f32", 64, 9999), ("adopt", 2, "bf16", 64, 9999),
+         ("sgdm", 4, "f32", 65, 4999), ("adam", 2, "bf16", 100, 4999), ("adam", 3, "f32", 129, 4999),
+         ("adam", 1, "bf16", 257, 3000)]
+
+
+@pytest.mark.parametrize("clip", [False, True])
+@pytest.mark.parametrize("base,N,gdt,M,numel", CASES)
+def test_fused_tiles_equal_step_then_average(P, base, N, gdt, M, numel, clip):
+    if clip and base == "adopt":
+        pytest.skip("ADOPT does not clip by norm")
+    w = workload_dict([numel], M, base=base, betas=(0.9, 0.999, 0.5, 0.99)[:N], px=1, pu=1, pv=0 if base == "sgdm" else 1,
+                      clip="global_norm" if clip else "none", rho=0.05, gdt=gdt)
+    (a, b), g = _pair(P, w, M, gdt, seed=M + N, plant=clip)
+    every = (1 << a.n_states) - 1
+    for mask in (every, 1, every & ~1, 1 << (a.n_states - 1)):
+        a.step(g, 1e-3, mask)
+        b.step(g, 1e-3, 0)
+        b.sync(mask)
+        _same(a, b)
+    if not clip:                                       # the last average, against 64 bits
+        s = a.n_states - 1
+        a.step(g, 1e-3, 0)
+        before = a.state_view(s).double()
+        a.set_params(a.state_view(0)[0].clone())       # all states but x to zero; v is put back
+        a.state_view(s).copy_(before)
+        a.t = 5
+        a.step(torch.zeros_like(g), 0.0, 1 << s)
+        beta = float(w["opt"]["beta2"]) if base != "sgdm" else float(w["opt"]["beta1"][N - 1])
+        mean = beta * before.mean(0)
+        got = a.state_view(s).double()
+        assert bool((got == got[0]).all())
+        # the decay rounds each value once (2^-24 of it), the compensated mean a few times
+        scale = before.abs().mean(0) + 1e-30
+        assert float(((got[0] - mean).abs() / scale).max()) < 4 * 2.0 ** -23
+    a.close()
+    b.close()
