@@ -98,7 +98,6 @@ struct mtdao_ctx {
     int norm_blocks = 1;
     double *stats_partial = nullptr;  // diagnostics workspace (allocated on first use)
     size_t stats_cap = 0;
-    float *stats_mean = nullptr;      // M > 8 diagnostics: [n_padded] replica mean (first use)
     float *anchor[2 + MTDAO_MAX_MOM] = {};  // per state: its value at the last average
     // host-gradient staging (mtdao_step_host)
     void *staging[2] = {nullptr, nullptr};
@@ -278,7 +277,6 @@ void release(mtdao_ctx *h) {
     if (h->norm_out) cudaFree(h->norm_out);
     if (h->norm_partial) cudaFree(h->norm_partial);
     if (h->stats_partial) cudaFree(h->stats_partial);
-    if (h->stats_mean) cudaFree(h->stats_mean);
     for (float *a : h->anchor)
         if (a) cudaFree(a);
 }
@@ -523,45 +521,22 @@ static int refresh_anchor(mtdao_ctx *h, uint32_t mask) {
     return MTDAO_OK;
 }
 
-// Diagnostics kernels hold M replicas in registers up to this M; up to
-// kWideStatsM they stage all replicas of a span in shared memory (one
-// pass); above it they take two passes through a scratch vector (for
-// M = 128 and 256 the one-pass form, whose per-element mean is a chain of
-// M / 2 compensated additions, ran 2-4x slower than the plain average; the
-// two passes take 1.4x).
+// Diagnostics kernels hold M replicas in registers up to this M; above it
+// they stage them in shared memory (stats_wide.cu).
 constexpr int kStatsRegisterM = 8;
-constexpr int kWideStatsM = 64;
-
-enum StatsPath { kStatsRegister, kStatsWide, kStatsGeneral };
-
-static StatsPath stats_path(const mtdao_ctx *h) {
-    return h->M <= kStatsRegisterM ? kStatsRegister : (h->M <= kWideStatsM ? kStatsWide : kStatsGeneral);
-}
 
 static int ensure_stats_workspace(mtdao_ctx *h) {
-    const StatsPath path = stats_path(h);
-    const bool general = path == kStatsGeneral;
-    if (h->stats_partial != nullptr && (!general || h->stats_mean != nullptr)) return MTDAO_OK;
-    if (h->stats_partial == nullptr) {
-        const size_t cap = path == kStatsGeneral ? general_stats_partial_capacity(h->num_sms, h->M)
-                           : path == kStatsWide  ? wide_stats_partial_capacity(h->num_sms, h->n_states, h->M)
-                                                 : sync_stats_partial_capacity(h->num_sms, h->n_padded, h->n_states, h->M);
-        cudaError_t e = cudaMalloc(reinterpret_cast<void **>(&h->stats_partial), cap * sizeof(double));
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            h->stats_partial = nullptr;
-            return set_error(h, MTDAO_ERR_OOM, "diagnostics workspace: %s", cudaGetErrorString(e));
-        }
-        h->stats_cap = cap;
+    if (h->stats_partial != nullptr) return MTDAO_OK;
+    const size_t cap = h->M <= kStatsRegisterM
+                           ? sync_stats_partial_capacity(h->num_sms, h->n_padded, h->n_states, h->M)
+                           : tile_stats_partial_capacity(h->num_sms, h->n_padded, h->n_states, h->M);
+    cudaError_t e = cudaMalloc(reinterpret_cast<void **>(&h->stats_partial), cap * sizeof(double));
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        h->stats_partial = nullptr;
+        return set_error(h, MTDAO_ERR_OOM, "diagnostics workspace: %s", cudaGetErrorString(e));
     }
-    if (general) {
-        cudaError_t e = cudaMalloc(reinterpret_cast<void **>(&h->stats_mean), h->n_padded * sizeof(float));
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            h->stats_mean = nullptr;
-            return set_error(h, MTDAO_ERR_OOM, "diagnostics scratch: %s", cudaGetErrorString(e));
-        }
-    }
+    h->stats_cap = cap;
     return MTDAO_OK;
 }
 
@@ -807,14 +782,9 @@ extern "C" int mtdao_sync_stats(mtdao_handle h, uint32_t mask, double *stats_dev
     a.M = h->M;
     for (int s = 0; s < h->n_states; ++s)
         if (mask & (1u << s)) a.sel[a.n_sel++] = s;
-    const StatsPath path = stats_path(h);
-    cudaError_t e =
-        path == kStatsGeneral
-            ? launch_sync_stats_general(a, h->num_sms, h->stats_mean, h->stats_partial, h->stats_cap, stats_dev,
-                                        h->stream)
-        : path == kStatsWide ? launch_sync_stats_wide(a, h->num_sms, h->stats_partial, h->stats_cap, stats_dev,
-                                                      h->stream)
-                             : launch_sync_stats(a, h->num_sms, h->stats_partial, h->stats_cap, stats_dev, h->stream);
+    cudaError_t e = h->M <= kStatsRegisterM
+                        ? launch_sync_stats(a, h->num_sms, h->stats_partial, h->stats_cap, stats_dev, h->stream)
+                        : launch_sync_stats_tile(a, h->num_sms, h->stats_partial, h->stats_cap, stats_dev, h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "sync with diagnostics launch");
     return refresh_anchor(h, mask);
 }
@@ -861,14 +831,10 @@ extern "C" int mtdao_pseudo_grad_stats(mtdao_handle h, int32_t state, double *ou
     if (int rc = select_device(h)) return rc;
     if (int rc = ensure_stats_workspace(h)) return rc;
     const float *x = h->arena + static_cast<int64_t>(state) * h->M * h->n_padded;
-    const StatsPath path = stats_path(h);
-    cudaError_t e =
-        path == kStatsGeneral
-            ? launch_pseudo_grad_stats_general(x, h->anchor[state], h->n_padded, h->M, h->num_sms, h->stats_mean,
-                                               h->stats_partial, h->stats_cap, out_dev, h->stream)
-        : path == kStatsWide ? launch_pseudo_grad_stats_wide(x, h->anchor[state], h->n_padded, h->M, h->num_sms,
-                                                             h->stats_partial, h->stats_cap, out_dev, h->stream)
-                             : launch_pseudo_grad_stats(x, h->anchor[state], h->n_padded, h->M, h->num_sms,
+    cudaError_t e = h->M <= kStatsRegisterM
+                        ? launch_pseudo_grad_stats(x, h->anchor[state], h->n_padded, h->M, h->num_sms,
+                                                   h->stats_partial, h->stats_cap, out_dev, h->stream)
+                        : launch_pseudo_grad_stats_tile(x, h->anchor[state], h->n_padded, h->M, h->num_sms,
                                                         h->stats_partial, h->stats_cap, out_dev, h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "change diagnostics launch");
     return MTDAO_OK;

@@ -110,16 +110,22 @@ size_t sync_stats_partial_capacity(int num_sms, int64_t n_padded, int n_states, 
 cudaError_t launch_sync_stats(const SyncArgs &a, int num_sms, double *partial, size_t partial_cap,
                               double *stats, cudaStream_t stream);
 
-// One-pass diagnostics for 2 <= M <= 256 (the wide layout of the fused
-// step): same outputs as launch_sync_stats / launch_pseudo_grad_stats, the
-// averaged states bit-identical to launch_sync's.  Workspace: partial needs
-// wide_stats_partial_capacity() doubles.
-size_t wide_stats_partial_capacity(int num_sms, int n_states, int M);
-cudaError_t launch_sync_stats_wide(const SyncArgs &a, int num_sms, double *partial, size_t partial_cap,
+// The diagnostics for more replicas (9 to MTDAO_MAX_REPLICAS): same outputs as
+// launch_sync_stats / launch_pseudo_grad_stats, the averaged states
+// bit-identical to launch_sync's.  Workspace: partial needs
+// tile_stats_partial_capacity() doubles.
+size_t tile_stats_partial_capacity(int num_sms, int64_t n_padded, int n_states, int M);
+cudaError_t launch_sync_stats_tile(const SyncArgs &a, int num_sms, double *partial, size_t partial_cap,
                                    double *stats, cudaStream_t stream);
-cudaError_t launch_pseudo_grad_stats_wide(const float *x, const float *anchor, int64_t n, int M, int num_sms,
+cudaError_t launch_pseudo_grad_stats_tile(const float *x, const float *anchor, int64_t n, int M, int num_sms,
                                           double *partial, size_t partial_cap, double *stats,
                                           cudaStream_t stream);
+
+// stats[row * Q + q] = the sum over blocks, in a fixed order, of
+// partial[(row * Q + q) * blocks + b] (Kahan sums, x - y); q = 0 divided by
+// divide_first when that is > 0.
+cudaError_t launch_stats_finalize(const float2 *partial, int64_t blocks, int Q, int rows, int divide_first,
+                                  double *stats, cudaStream_t stream);
 
 // Per-replica sum of squares of the gradient: partial sums into
 // partial[M][blocks_per_replica], then out[m] (double) and, when
@@ -128,18 +134,6 @@ int norm_blocks_per_replica(int num_sms, int M);
 cudaError_t launch_grad_sqnorm(const void *grads, int grad_dtype, int32_t M, int64_t n_padded,
                                int blocks_per_replica, double *partial, double *out,
                                float *clip_scale, double rho, cudaStream_t stream);
-
-// Diagnostics for any M, used above 256 (two passes per state through a
-// [n_padded] fp32 scratch that holds the replica mean; see reduce_kernels.cu).  Same
-// outputs as launch_sync_stats / launch_pseudo_grad_stats; the averaged
-// states are bit-identical to launch_sync's.  Workspace: partial needs
-// general_stats_partial_capacity() doubles.
-size_t general_stats_partial_capacity(int num_sms, int M);
-cudaError_t launch_sync_stats_general(const SyncArgs &a, int num_sms, float *mean_scratch, double *partial,
-                                      size_t partial_cap, double *stats, cudaStream_t stream);
-cudaError_t launch_pseudo_grad_stats_general(const float *x, const float *anchor, int64_t n, int M, int num_sms,
-                                             float *mean_scratch, double *partial, size_t partial_cap,
-                                             double *stats, cudaStream_t stream);
 
 // Number of NaN / +-Inf gradient values per replica into out[m] (double,
 // exact), with the grid and workspace of launch_grad_sqnorm.

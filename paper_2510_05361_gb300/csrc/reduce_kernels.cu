@@ -4,8 +4,8 @@
 // Averaging (Algorithms 1-3, E_m[.] with averaging as OuterOpt): for every
 // selected state and element, the M replica values are read once and the
 // mean (replica_mean.cuh) is written back to all M replicas.  Algorithmic traffic: 8 * M bytes
-// per element per state.  HBM-bound; grid-stride over float4 vectors, one
-// grid row (blockIdx.y) per selected state.
+// per element per state.  HBM-bound; one grid row (blockIdx.y) per selected
+// state.
 //
 // Norm: sum_i g[m][i]^2 per replica with a fixed grid and fixed reduction
 // order, so the result is bit-reproducible.  Each thread accumulates its
@@ -26,8 +26,7 @@ namespace mtdao {
 namespace {
 
 // Mean of the M replicas at float4 position e of state s, M known at run
-// time (the standalone average above 8 replicas and the two-pass
-// diagnostics): replica_mean.cuh's operations in its order, four replicas'
+// time (the standalone average above 14 replicas): replica_mean.cuh's operations in its order, four replicas'
 // loads in flight (one at a time, the average of M = 9-64 ran at 5.5-5.8
 // TB/s).
 __device__ __forceinline__ float4 replica_mean4(const float *s, int64_t n, int M, int64_t e) {
@@ -362,15 +361,20 @@ __global__ void __launch_bounds__(kThreads) sync_stats_kernel(const SyncArgs a, 
 // thread t of block (q, row) adds a contiguous run of blocks in order, then
 // block_sum adds the threads' sums in a fixed order.  q = 0 is divided by
 // divide_first (M for the variance, a mean over workers; 0 leaves it).
-__global__ void __launch_bounds__(kNormThreads) stats_finalize_kernel(const double *partial, int64_t blocks,
+// A value is a double, or a Kahan sum (x - y).
+__device__ __forceinline__ double wide_value(double v) { return v; }
+__device__ __forceinline__ double wide_value(float2 v) { return static_cast<double>(v.x) - static_cast<double>(v.y); }
+
+template <typename T>
+__global__ void __launch_bounds__(kNormThreads) stats_finalize_kernel(const T *partial, int64_t blocks,
                                                                       int Q, int divide_first, double *stats) {
     const int q = blockIdx.x, row = blockIdx.y;
-    const double *p = partial + (static_cast<int64_t>(row) * Q + q) * blocks;
+    const T *p = partial + (static_cast<int64_t>(row) * Q + q) * blocks;
     const int64_t per = (blocks + blockDim.x - 1) / blockDim.x;
     const int64_t lo = threadIdx.x * per;
     const int64_t hi = lo + per < blocks ? lo + per : blocks;
     double acc = 0.0;
-    for (int64_t b = lo; b < hi; ++b) acc += p[b];
+    for (int64_t b = lo; b < hi; ++b) acc += wide_value(p[b]);
     const double total = block_sum(acc);
     if (threadIdx.x == 0) stats[row * Q + q] = (q == 0 && divide_first > 0) ? total / divide_first : total;
 }
@@ -473,229 +477,6 @@ cudaError_t launch_pseudo_grad_stats_t(const float *x, const float *anchor, int6
     return cudaGetLastError();
 }
 
-// ---------------------------------------------------------------- diagnostics for any M
-
-// For M above the register-resident kernels' limit the diagnostics take two
-// passes over one state (a [n] fp32 scratch holds the mean between them):
-//   pass 1 (grid-stride over float4 positions): the replica mean of
-//     replica_mean.cuh (the bits mtdao_sync stores), written to the
-//     scratch, and the sums that need only the mean (and the anchor);
-//   pass 2 (grid (blocks, M)): per replica the sums against the scratch
-//     mean and, for an average, the mean written over the replica.
-// As in the one-pass kernels, each position's four elements are summed in
-// fp32, each thread accumulates its positions with Kahan compensation, and
-// warps, blocks and a finalize kernel reduce in fp64 in fixed order:
-// bit-reproducible.  (GB300's fp64 rate is far below its fp32 rate, so the
-// per-element work stays in fp32.)
-
-// Deterministic block reduction of K doubles per thread into out[0..K)
-// (written by thread 0).
-template <int K>
-__device__ void block_sum_k(const double (&v)[K], double *out) {
-    __shared__ double part[K][kNormThreads / 32];
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        const double x = warp_sum(v[k]);
-        if (l == 0) part[k][w] = x;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            double t = 0.0;
-            for (int i = 0; i < static_cast<int>(blockDim.x >> 5); ++i) t += part[k][i];
-            out[k] = t;
-        }
-    }
-}
-
-// Positions a pass-2 thread loads before it accumulates them (i, i + T,
-// i + 2T, ...: the order of a plain grid-stride loop): four for the sync
-// diagnostics (two float4 loads per position), two for the change
-// diagnostics (three per position, within 64 registers).
-constexpr int kPass2Unroll = 4;
-constexpr int kPass2UnrollChange = 2;
-
-// Pass 1 of the sync diagnostics: mean -> scratch; per block sum s_bar^2.
-__global__ void __launch_bounds__(kNormThreads, 4) sync_stats_pass1_kernel(const float *s, int64_t n, int M,
-                                                                       float *mean_out, double *partial) {
-    const int64_t nv = n / 4;
-    Kahan q;
-    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < nv;
-         i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        const int64_t e = 4 * i;
-        const float4 mv = replica_mean4(s, n, M, e);
-        *reinterpret_cast<float4 *>(mean_out + e) = mv;
-        q.add(fmaf(mv.x, mv.x, fmaf(mv.y, mv.y, fmaf(mv.z, mv.z, __fmul_rn(mv.w, mv.w)))));
-    }
-    const double v[1] = {q.value()};
-    block_sum_k<1>(v, partial + blockIdx.x);
-}
-
-// Pass 2 of the sync diagnostics, replica m = blockIdx.y: per block
-// (sum (s_m - s_bar)^2, sum s_m^2, sum s_m * s_bar); with write_mean the
-// replica is overwritten by the mean (the average itself).
-__global__ void __launch_bounds__(kNormThreads, 4) sync_stats_pass2_kernel(float *s, int64_t n, const float *mean,
-                                                                       int write_mean, double *partial) {
-    const int m = blockIdx.y;
-    const int64_t nv = n / 4;
-    const int64_t T = static_cast<int64_t>(gridDim.x) * blockDim.x;
-    float *rep = s + m * n;
-    Kahan q0, q1, q2;
-    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < nv; i += kPass2Unroll * T) {
-        float4 rv[kPass2Unroll], mv[kPass2Unroll];
-#pragma unroll
-        for (int u = 0; u < kPass2Unroll; ++u)
-            if (i + u * T < nv) {
-                rv[u] = ld_state(rep + 4 * (i + u * T));
-                mv[u] = *reinterpret_cast<const float4 *>(mean + 4 * (i + u * T));
-            }
-#pragma unroll
-        for (int u = 0; u < kPass2Unroll; ++u) {
-            if (i + u * T >= nv) break;
-            float r[4], mb[4];
-            to_array(rv[u], r);
-            to_array(mv[u], mb);
-            float p0 = 0.0f, p1 = 0.0f, p2 = 0.0f;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const float dv = r[k] - mb[k];
-                p0 = fmaf(dv, dv, p0);
-                p1 = fmaf(r[k], r[k], p1);
-                p2 = fmaf(r[k], mb[k], p2);
-            }
-            q0.add(p0);
-            q1.add(p1);
-            q2.add(p2);
-            if (write_mean) st_state(rep + 4 * (i + u * T), mv[u]);
-        }
-    }
-    const double v[3] = {q0.value(), q1.value(), q2.value()};
-    block_sum_k<3>(v, partial + 3 * (static_cast<int64_t>(m) * gridDim.x + blockIdx.x));
-}
-
-// Pass 1 of the change diagnostics: x_bar -> scratch; per block
-// (sum (x_bar - a)^2, sum a^2).
-__global__ void __launch_bounds__(kNormThreads, 4) pseudo_grad_pass1_kernel(const float *x, const float *anchor,
-                                                                        int64_t n, int M, float *mean_out,
-                                                                        double *partial) {
-    const int64_t nv = n / 4;
-    Kahan q0, q1;
-    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < nv;
-         i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        const int64_t e = 4 * i;
-        const float4 mv = replica_mean4(x, n, M, e);
-        *reinterpret_cast<float4 *>(mean_out + e) = mv;
-        float mean[4], a[4];
-        to_array(mv, mean);
-        to_array(__ldcs(reinterpret_cast<const float4 *>(anchor + e)), a);
-        float p0 = 0.0f, p1 = 0.0f;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const float glob = mean[k] - a[k];
-            p0 = fmaf(glob, glob, p0);
-            p1 = fmaf(a[k], a[k], p1);
-        }
-        q0.add(p0);
-        q1.add(p1);
-    }
-    const double v[2] = {q0.value(), q1.value()};
-    block_sum_k<2>(v, partial + 2 * static_cast<int64_t>(blockIdx.x));
-}
-
-// Pass 2 of the change diagnostics, replica m = blockIdx.y: per block
-// (sum (x_m - a)^2, sum (x_m - a)(x_bar - a)).  Read-only.
-__global__ void __launch_bounds__(kNormThreads, 4) pseudo_grad_pass2_kernel(const float *x, const float *anchor,
-                                                                        int64_t n, const float *mean,
-                                                                        double *partial) {
-    const int m = blockIdx.y;
-    const int64_t nv = n / 4;
-    const int64_t T = static_cast<int64_t>(gridDim.x) * blockDim.x;
-    const float *rep = x + m * n;
-    Kahan q0, q1;
-    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < nv; i += kPass2UnrollChange * T) {
-        float4 rv[kPass2UnrollChange], mv[kPass2UnrollChange], av[kPass2UnrollChange];
-#pragma unroll
-        for (int u = 0; u < kPass2UnrollChange; ++u)
-            if (i + u * T < nv) {
-                const int64_t e = 4 * (i + u * T);
-                rv[u] = ld_state(rep + e);
-                mv[u] = *reinterpret_cast<const float4 *>(mean + e);
-                av[u] = *reinterpret_cast<const float4 *>(anchor + e);
-            }
-#pragma unroll
-        for (int u = 0; u < kPass2UnrollChange; ++u) {
-            if (i + u * T >= nv) break;
-            float r[4], mb[4], a[4];
-            to_array(rv[u], r);
-            to_array(mv[u], mb);
-            to_array(av[u], a);
-            float p0 = 0.0f, p1 = 0.0f;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const float loc = r[k] - a[k];
-                const float glob = mb[k] - a[k];
-                p0 = fmaf(loc, loc, p0);
-                p1 = fmaf(loc, glob, p1);
-            }
-            q0.add(p0);
-            q1.add(p1);
-        }
-    }
-    const double v[2] = {q0.value(), q1.value()};
-    block_sum_k<2>(v, partial + 2 * (static_cast<int64_t>(m) * gridDim.x + blockIdx.x));
-}
-
-// Adds block partials in block order.  p1 holds K1 values per pass-1
-// block, p2 K2 values per (replica, pass-2 block).  For t < K1:
-// out[g[t]] = sum_b p1[b][t]; for t < K2 and each replica m:
-// out[r[t] + m] = sum_b p2[m][b][t], except that t_sum (if >= 0) is
-// summed over the replicas too and divided by M into out[sum_to]
-// instead.
-struct FinalizeMap {
-    int K1, K2;
-    int g[2];
-    int r[3];
-    int t_sum, sum_to;
-};
-
-__global__ void general_stats_finalize_kernel(const double *p1, int b1, const double *p2, int b2, int M,
-                                              FinalizeMap f, double *out) {
-    if (threadIdx.x == 0) {
-        for (int t = 0; t < f.K1; ++t) {
-            double acc = 0.0;
-            for (int b = 0; b < b1; ++b) acc += p1[b * f.K1 + t];
-            out[f.g[t]] = acc;
-        }
-        if (f.t_sum >= 0) {
-            double acc = 0.0;
-            for (int m = 0; m < M; ++m)
-                for (int b = 0; b < b2; ++b) acc += p2[(static_cast<int64_t>(m) * b2 + b) * f.K2 + f.t_sum];
-            out[f.sum_to] = acc / M;
-        }
-    }
-    for (int m = threadIdx.x; m < M; m += blockDim.x) {
-        for (int t = 0; t < f.K2; ++t) {
-            if (t == f.t_sum) continue;
-            double acc = 0.0;
-            for (int b = 0; b < b2; ++b) acc += p2[(static_cast<int64_t>(m) * b2 + b) * f.K2 + t];
-            out[f.r[t] + m] = acc;
-        }
-    }
-}
-
-struct GeneralGrid {
-    int b1, b2;
-};
-
-GeneralGrid general_grid(int num_sms, int M, int64_t n) {
-    const int64_t need = (n / 4 + kNormThreads - 1) / kNormThreads;
-    int64_t b1 = 4 * static_cast<int64_t>(num_sms), b2 = b1 / M;
-    if (b1 > need) b1 = need;
-    if (b2 > need) b2 = need;
-    return {static_cast<int>(b1 < 1 ? 1 : b1), static_cast<int>(b2 < 1 ? 1 : b2)};
-}
 }  // namespace
 
 cudaError_t launch_pseudo_grad_stats(const float *x, const float *anchor, int64_t n, int M, int num_sms,
@@ -792,46 +573,9 @@ cudaError_t launch_grad_sqnorm(const void *grads, int grad_dtype, int32_t M, int
 }
 
 
-size_t general_stats_partial_capacity(int num_sms, int M) {
-    const size_t b1 = 4 * static_cast<size_t>(num_sms);
-    const size_t b2 = b1 / static_cast<size_t>(M > 0 ? M : 1) + 1;
-    return 2 * b1 + 3 * b2 * static_cast<size_t>(M);
-}
-
-cudaError_t launch_sync_stats_general(const SyncArgs &a, int num_sms, float *mean_scratch, double *partial,
-                                      size_t partial_cap, double *stats, cudaStream_t stream) {
-    const int M = a.M;
-    const int Q = 2 + 2 * M;
-    const GeneralGrid g = general_grid(num_sms, M, a.n_padded);
-    if (static_cast<size_t>(g.b1) + 3 * static_cast<size_t>(g.b2) * M > partial_cap) return cudaErrorInvalidValue;
-    double *p1 = partial, *p2 = partial + g.b1;
-    // stats row: [0] variance (sum over replicas / M), [1] s_bar^2, [2 + m] s_m^2, [2 + M + m] s_m s_bar
-    FinalizeMap f = {1, 3, {1, 0}, {0, 2, 2 + M}, 0, 0};
-    for (int k = 0; k < a.n_sel; ++k) {
-        float *s = a.arena + static_cast<int64_t>(a.sel[k]) * a.stride;
-        sync_stats_pass1_kernel<<<g.b1, kNormThreads, 0, stream>>>(s, a.n_padded, M, mean_scratch, p1);
-        sync_stats_pass2_kernel<<<dim3(g.b2, M), kNormThreads, 0, stream>>>(s, a.n_padded, mean_scratch,
-                                                                            M > 1 ? 1 : 0, p2);
-        general_stats_finalize_kernel<<<1, 256, 0, stream>>>(p1, g.b1, p2, g.b2, M, f,
-                                                             stats + static_cast<int64_t>(k) * Q);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
-}
-
-cudaError_t launch_pseudo_grad_stats_general(const float *x, const float *anchor, int64_t n, int M, int num_sms,
-                                             float *mean_scratch, double *partial, size_t partial_cap,
-                                             double *stats, cudaStream_t stream) {
-    const GeneralGrid g = general_grid(num_sms, M, n);
-    if (2 * static_cast<size_t>(g.b1) + 2 * static_cast<size_t>(g.b2) * M > partial_cap)
-        return cudaErrorInvalidValue;
-    double *p1 = partial, *p2 = partial + 2 * g.b1;
-    // out: [m] (x_m - a)^2, [M + m] (x_m - a)(x_bar - a), [2M] (x_bar - a)^2, [2M + 1] a^2
-    FinalizeMap f = {2, 2, {2 * M, 2 * M + 1}, {0, M, 0}, -1, 0};
-    pseudo_grad_pass1_kernel<<<g.b1, kNormThreads, 0, stream>>>(x, anchor, n, M, mean_scratch, p1);
-    pseudo_grad_pass2_kernel<<<dim3(g.b2, M), kNormThreads, 0, stream>>>(x, anchor, n, mean_scratch, p2);
-    general_stats_finalize_kernel<<<1, 256, 0, stream>>>(p1, g.b1, p2, g.b2, M, f, stats);
+cudaError_t launch_stats_finalize(const float2 *partial, int64_t blocks, int Q, int rows, int divide_first,
+                                  double *stats, cudaStream_t stream) {
+    stats_finalize_kernel<<<dim3(Q, rows), kNormThreads, 0, stream>>>(partial, blocks, Q, divide_first, stats);
     return cudaGetLastError();
 }
 

@@ -1,373 +1,281 @@
-// stats_wide.cu -- the cross-worker diagnostics of section 4.1 in one pass
-// for 9 <= M <= 64 replicas (the kernels take up to kWideMaxM = 256; above
-// 64 the library uses the two-pass form of reduce_kernels.cu, whose
-// register-resident kernels cover M <= 8).
+// stats_wide.cu -- the cross-worker diagnostics of section 4.1 for more
+// replicas than a thread holds (9 <= M <= 1024).
 //
-// Same block layout as the wide fused step (step_sync_wide.cuh): a block
-// owns spans of S consecutive elements of all M replicas, thread (r, f)
-// copies 16 elements of replica r (four float4 positions f, f + P, ...) into
-// a shared M x S tile (double-buffered with cp.async), the
-// span's replica means are formed from the tile by tile_means (the bits of
-// the standalone average), and each thread then forms its own replica's
-// sums against the mean.  Every replica value is read from HBM once; the
-// sync diagnostics write the mean over it (the average itself), so a sync
-// with diagnostics moves the bytes of a plain sync.
+// A block takes a run of consecutive tiles, S columns of all M replicas each:
+// copies a tile to shared memory (cp.async), forms its replica means
+// (tile_means: the bits of the standalone average) and adds every replica's
+// sums against the mean; the sync diagnostics then store the mean over the
+// replicas (the average itself).  Every replica value is read from HBM once.
+// What overlaps the copies of a block is the work of the others on its SM.
 //
-// Sums are bit-reproducible: a thread's 16 elements of a span are summed in
-// fp32, each thread accumulates its spans with Kahan compensation, the P
-// threads of a replica combine in fp64 by a fixed shuffle pattern, the
-// block writes one partial row, and a finalize kernel adds the rows in
-// block order.  The grid is persistent (spans strided by the grid), so the
-// partial rows stay few.
+// Sums are bit-reproducible: a thread's elements of a tile are summed in fp32,
+// each thread accumulates its tiles with Kahan compensation, the L lanes of a
+// replica combine their compensated sums by a fixed shuffle pattern, the block
+// writes one compensated sum per quantity, and launch_stats_finalize adds the
+// blocks' in fp64 in a fixed order.
 #include <cuda_runtime.h>
 #include <cstdint>
 
 #include "kahan.cuh"
 #include "mtdao_internal.h"
-#include "replica_mean.cuh"
+#include "replica_tile.cuh"
 #include "step_kernels.cuh"
-#include "step_sync_wide.cuh"
 
 namespace mtdao {
 
 namespace {
 
-// Sum over the P lanes of one replica (aligned groups of P lanes, P a power
-// of two dividing 32): every lane of the group ends with the same value.
-__device__ __forceinline__ double replica_lanes_sum(double v, int P) {
-    for (int off = P >> 1; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+constexpr int kStatsTileThreads = 256;
+
+struct StatsTileArgs {
+    float *arena;                    // state sel[blockIdx.y] at arena + sel * stride, [M][n]
+    const float *anchor;             // change diagnostics: [n]
+    float2 *partial;                 // [state][Q][gridDim.x]: Kahan sums
+    int64_t n, stride;
+    int32_t sel[2 + MTDAO_MAX_MOM];
+    int32_t M;
+    int32_t tiles;                   // tiles of a run
+    int32_t log2_s, log2_l;          // columns of a tile, lanes of a replica
+};
+
+// Sum over the block, valid in thread 0 (fixed order).
+__device__ Kahan block_total(Kahan v) {
+    __shared__ float2 part[kStatsTileThreads / 32];
+    v = lanes_sum(v, 32);
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = make_float2(v.s, v.c);
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (int i = 1; i < static_cast<int>(blockDim.x >> 5); ++i) {
+            Kahan o;
+            o.s = part[i].x;
+            o.c = part[i].y;
+            v = v + o;
+        }
+    __syncthreads();
     return v;
 }
 
-// float4 positions per thread and span: the span is S = 4 * P * kStatsVec
-// elements (rows of 128 bytes or more for every M up to 256).
-constexpr int kStatsVec = 4;
-constexpr int kStatsVecLog2 = 2;
-
-// Copies this thread's kStatsVec float4 positions of replica r of a span
-// (src: the replica's first element of the span) into its tile row, then
-// commits the group (an empty one when the span is past the end).
-__device__ __forceinline__ void fetch_row(bool live, float *dst, const float *src, int P) {
-    if (live) {
-#pragma unroll
-        for (int j = 0; j < kStatsVec; ++j) cp_async16(dst + 4 * P * j, src + 4 * P * j);
-    }
-    cp_async_commit();
-}
-
-// Sync diagnostics of the selected state blockIdx.y, partial row per block:
+// CHANGE = false, sync diagnostics (Q = 2 + 2M):
 //   q = 0          sum_m sum_i (s_m - s_bar)^2
 //   q = 1          sum_i s_bar^2
 //   q = 2 + m      sum_i s_m^2
 //   q = 2 + M + m  sum_i s_m * s_bar
-// at partial[(blockIdx.y * gridDim.x + blockIdx.x) * Q + q], Q = 2 + 2M;
-// s_bar (the fp32 mean) is written over every replica.
-template <bool FOUR>
-__global__ void __launch_bounds__(kWideMaxThreads) sync_stats_wide_kernel(const SyncArgs a, int log2_p,
-                                                                          double *partial) {
-    extern __shared__ __align__(16) float smem[];
-    constexpr int NV = kStatsVec;
-    const int M = a.M;
-    const int P = 1 << log2_p;
-    const int log2_s = log2_p + 2 + kStatsVecLog2;
-    const int S = 1 << log2_s;
-    const int Q = 2 + 2 * M;
-    const int t = threadIdx.x;
-    const int r = t >> log2_p;
-    const int f = t & (P - 1);
-    const bool live = r < M;
-    float *base = a.arena + static_cast<int64_t>(a.sel[blockIdx.y]) * a.stride;
-    const int64_t n = a.n_padded;
-    const int64_t n_spans = n / S;
-    float *tiles = smem;                         // [2][M][S]
-    float *mean = smem + 2 * M * S;              // [S]
-    Kahan dev, sq, cross, msq;
-
-    const int64_t first = blockIdx.x;
-    fetch_row(live && first < n_spans, tiles + r * S + 4 * f, base + r * n + first * S + 4 * f, P);
-    int buf = 0;
-    for (int64_t span = first; span < n_spans; span += gridDim.x, buf ^= 1) {
-        const int64_t next = span + gridDim.x;
-        fetch_row(live && next < n_spans, tiles + ((buf ^ 1) * M + r) * S + 4 * f,
-                  base + r * n + next * S + 4 * f, P);
-        cp_async_wait<1>();                      // this thread's copies of `span` have landed
-        __syncthreads();                         // ... and every thread's
-        const float *tile = tiles + buf * M * S;
-        tile_means<FOUR ? 4 : 1>(tile, M, log2_s, S, mean);
-        __syncthreads();
-        if (live) {
-            float p0 = 0.0f, p1 = 0.0f, p2 = 0.0f, p3 = 0.0f;   // this thread's 4 * NV elements
-#pragma unroll
-            for (int j = 0; j < NV; ++j) {
-                const int c = 4 * f + 4 * P * j;
-                float x[4], mb[4];
-                to_array(*reinterpret_cast<const float4 *>(tile + r * S + c), x);
-                const float4 mv = *reinterpret_cast<const float4 *>(mean + c);
-                to_array(mv, mb);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const float dv = x[k] - mb[k];
-                    p0 = fmaf(dv, dv, p0);
-                    p1 = fmaf(x[k], x[k], p1);
-                    p2 = fmaf(x[k], mb[k], p2);
-                    p3 = fmaf(mb[k], mb[k], p3);
-                }
-                st_state(base + r * n + span * S + c, mv);
-            }
-            dev.add(p0);
-            sq.add(p1);
-            cross.add(p2);
-            if (r == 0) msq.add(p3);
-        }
-        __syncthreads();                         // this tile and the means are rewritten next
-    }
-    cp_async_wait<0>();
-
-    // Per replica: its P lanes' sums; then one row of Q values.
-    const double d = replica_lanes_sum(dev.value(), P);
-    const double s2 = replica_lanes_sum(sq.value(), P);
-    const double c2 = replica_lanes_sum(cross.value(), P);
-    const double m2 = replica_lanes_sum(msq.value(), P);   // replica 0's lanes hold sum s_bar^2
-    double *red = reinterpret_cast<double *>(smem);        // [3][M] + 1, over the (now idle) tiles
-    if (live && f == 0) {
-        red[r] = d;
-        red[M + r] = s2;
-        red[2 * M + r] = c2;
-        if (r == 0) red[3 * M] = m2;
-    }
-    __syncthreads();
-    double *row = partial + (static_cast<int64_t>(blockIdx.y) * gridDim.x + blockIdx.x) * Q;
-    for (int q = t; q < Q; q += blockDim.x) {
-        double v;
-        if (q == 0) {
-            v = 0.0;
-            for (int m = 0; m < M; ++m) v += red[m];
-        } else if (q == 1) {
-            v = red[3 * M];
-        } else if (q < 2 + M) {
-            v = red[M + (q - 2)];
-        } else {
-            v = red[2 * M + (q - 2 - M)];
-        }
-        row[q] = v;
-    }
-}
-
-// Pseudo-gradient diagnostics of x[M][n] against the anchor a[n], read-only;
-// partial row per block (Q = 2M + 2):
+// CHANGE = true, change of x against the anchor a, read-only (Q = 2M + 2):
 //   q = m          sum_i (x_m - a)^2
 //   q = M + m      sum_i (x_m - a) * (x_bar - a)
 //   q = 2M         sum_i (x_bar - a)^2
 //   q = 2M + 1     sum_i a^2
-// The anchor's span travels with replica 0's row (one more tile row).
-template <bool FOUR>
-__global__ void __launch_bounds__(kWideMaxThreads) pseudo_grad_stats_wide_kernel(const float *x,
-                                                                                 const float *anchor,
-                                                                                 int64_t n, int M, int log2_p,
-                                                                                 double *partial) {
+// Thread t takes the rows (replicas) t / L + k * blockDim / L, k < R.
+template <bool CHANGE, int R, int V>
+__global__ void __launch_bounds__(kStatsTileThreads) stats_tile_kernel(const __grid_constant__ StatsTileArgs a) {
     extern __shared__ __align__(16) float smem[];
-    constexpr int NV = kStatsVec;
-    const int P = 1 << log2_p;
-    const int log2_s = log2_p + 2 + kStatsVecLog2;
-    const int S = 1 << log2_s;
-    const int Q = 2 * M + 2;
+    const int M = a.M;
+    const int S = 1 << a.log2_s;
+    const int log2_p = a.log2_s - 2;
+    const int L = 1 << a.log2_l;
+    const int items = M << log2_p;
     const int t = threadIdx.x;
-    const int r = t >> log2_p;
-    const int f = t & (P - 1);
-    const bool live = r < M;
-    const int64_t n_spans = n / S;
-    const int R = M + 1;                         // tile rows: the replicas, then the anchor
-    float *tiles = smem;                         // [2][M + 1][S]
-    float *mean = smem + 2 * R * S;              // [S]
-    Kahan loc2, cross, glob2, a2;
+    const int lane = t & (L - 1);
+    const int row0 = t >> a.log2_l;
+    const int row_step = static_cast<int>(blockDim.x) >> a.log2_l;
+    const int64_t n = a.n;
+    float *base = a.arena + static_cast<int64_t>(a.sel[blockIdx.y]) * a.stride;
+    float *tile = smem;                          // [M][S]
+    float *mean = smem + M * S;                  // [S]
+    float *anc = mean + S;                       // [S] (CHANGE)
+    Kahan own[R], cross[R];                      // s_m^2 and s_m s_bar, or (x_m - a)^2 and (x_m - a)(x_bar - a)
+    Kahan all, ref;                              // (s_m - s_bar)^2 and s_bar^2, or (x_bar - a)^2 and a^2
 
-    auto fetch = [&](int64_t span, int b) {
-        const bool ok = live && span < n_spans;
-        if (ok && r == 0) {
-#pragma unroll
-            for (int j = 0; j < NV; ++j)
-                cp_async16(tiles + (b * R + M) * S + 4 * f + 4 * P * j, anchor + span * S + 4 * f + 4 * P * j);
-        }
-        fetch_row(ok, tiles + (b * R + r) * S + 4 * f, x + r * n + span * S + 4 * f, P);
-    };
-    fetch(blockIdx.x, 0);
-    int buf = 0;
-    for (int64_t span = blockIdx.x; span < n_spans; span += gridDim.x, buf ^= 1) {
-        fetch(span + gridDim.x, buf ^ 1);
-        cp_async_wait<1>();
+    const int64_t n_tiles = n >> a.log2_s;
+    const int64_t first = static_cast<int64_t>(blockIdx.x) * a.tiles;
+    const int64_t last = first + a.tiles < n_tiles ? first + a.tiles : n_tiles;
+    for (int64_t k = first; k < last; ++k) {
+        const int64_t col0 = k << a.log2_s;
+        for (int i = t; i < items; i += static_cast<int>(blockDim.x))
+            cp_async16(tile + 4 * i, base + (i >> log2_p) * n + col0 + 4 * (i & ((1 << log2_p) - 1)));
+        if (CHANGE && t < (1 << log2_p)) cp_async16(anc + 4 * t, a.anchor + col0 + 4 * t);
+        cp_async_commit();
+        cp_async_wait<0>();                      // this thread's copies have landed
+        __syncthreads();                         // ... and every thread's
+        tile_means<V>(tile, M, a.log2_s, S, mean);
         __syncthreads();
-        const float *tile = tiles + buf * R * S;
-        const float *anc = tile + M * S;
-        tile_means<FOUR ? 4 : 1>(tile, M, log2_s, S, mean);
-        __syncthreads();
-        if (live) {
-            float p0 = 0.0f, p1 = 0.0f, p2 = 0.0f, p3 = 0.0f;   // this thread's 4 * NV elements
 #pragma unroll
-            for (int j = 0; j < NV; ++j) {
-                const int c = 4 * f + 4 * P * j;
-                float xv[4], mb[4], aj[4];
-                to_array(*reinterpret_cast<const float4 *>(tile + r * S + c), xv);
+        for (int j = 0; j < R; ++j) {
+            const int r = row0 + j * row_step;
+            if (r >= M) break;
+            float p0 = 0.0f, p1 = 0.0f, p2 = 0.0f, p3 = 0.0f;
+            for (int c = 4 * lane; c < S; c += 4 * L) {
+                float x[4], mb[4];
+                to_array(*reinterpret_cast<const float4 *>(tile + r * S + c), x);
                 to_array(*reinterpret_cast<const float4 *>(mean + c), mb);
-                to_array(*reinterpret_cast<const float4 *>(anc + c), aj);
+                if constexpr (CHANGE) {
+                    float av[4];
+                    to_array(*reinterpret_cast<const float4 *>(anc + c), av);
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const float loc = xv[k] - aj[k];
-                    const float glob = mb[k] - aj[k];
-                    p0 = fmaf(loc, loc, p0);
-                    p1 = fmaf(loc, glob, p1);
-                    p2 = fmaf(glob, glob, p2);
-                    p3 = fmaf(aj[k], aj[k], p3);
+                    for (int q = 0; q < 4; ++q) {
+                        const float loc = x[q] - av[q], glob = mb[q] - av[q];
+                        p0 = fmaf(loc, loc, p0);
+                        p1 = fmaf(loc, glob, p1);
+                        p2 = fmaf(glob, glob, p2);
+                        p3 = fmaf(av[q], av[q], p3);
+                    }
+                } else {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const float dv = x[q] - mb[q];
+                        p0 = fmaf(x[q], x[q], p0);
+                        p1 = fmaf(x[q], mb[q], p1);
+                        p2 = fmaf(dv, dv, p2);
+                        p3 = fmaf(mb[q], mb[q], p3);
+                    }
                 }
             }
-            loc2.add(p0);
-            cross.add(p1);
-            if (r == 0) {
-                glob2.add(p2);
-                a2.add(p3);
+            own[j].add(p0);
+            cross[j].add(p1);
+            if (!CHANGE || r == 0) all.add(p2);
+            if (r == 0) ref.add(p3);
+        }
+        if constexpr (!CHANGE) {
+            for (int i = t; i < items; i += static_cast<int>(blockDim.x)) {
+                const int f = i & ((1 << log2_p) - 1);
+                st_state(base + (i >> log2_p) * n + col0 + 4 * f, *reinterpret_cast<const float4 *>(mean + 4 * f));
             }
         }
-        __syncthreads();
+        __syncthreads();                         // the tile and the means are rewritten next
     }
-    cp_async_wait<0>();
 
-    const double l2 = replica_lanes_sum(loc2.value(), P);
-    const double c2 = replica_lanes_sum(cross.value(), P);
-    const double g2 = replica_lanes_sum(glob2.value(), P);
-    const double aa = replica_lanes_sum(a2.value(), P);
-    double *red = reinterpret_cast<double *>(smem);        // [2][M] + 2
-    if (live && f == 0) {
-        red[r] = l2;
-        red[M + r] = c2;
-        if (r == 0) {
-            red[2 * M] = g2;
-            red[2 * M + 1] = aa;
+    const int Q = 2 + 2 * M;
+    float2 *out = a.partial + static_cast<int64_t>(blockIdx.y) * Q * gridDim.x + blockIdx.x;
+    auto put = [&](int q, const Kahan &v) { out[static_cast<int64_t>(q) * gridDim.x] = make_float2(v.s, v.c); };
+    const int own_at = CHANGE ? 0 : 2;
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+        const int r = row0 + j * row_step;
+        const Kahan v0 = lanes_sum(own[j], L);
+        const Kahan v1 = lanes_sum(cross[j], L);
+        if (r < M && lane == 0) {
+            put(own_at + r, v0);
+            put(own_at + M + r, v1);
         }
     }
-    __syncthreads();
-    double *row = partial + static_cast<int64_t>(blockIdx.x) * Q;
-    for (int q = t; q < Q; q += blockDim.x) row[q] = red[q];
+    const Kahan all_sum = block_total(all);
+    const Kahan ref_sum = block_total(ref);
+    if (t == 0) {
+        put(CHANGE ? 2 * M : 0, all_sum);
+        put(CHANGE ? 2 * M + 1 : 1, ref_sum);
+    }
 }
 
-// out[row * Q + q] = sum over blocks b (in order) of partial[(row * blocks + b) * Q + q];
-// q = 0 divided by divide_first when that is > 0.
-__global__ void wide_stats_finalize_kernel(const double *partial, int blocks, int Q, int divide_first,
-                                           double *out) {
-    const int row = blockIdx.y;
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= Q) return;
-    double total = 0.0;
-    for (int b = 0; b < blocks; ++b) total += partial[(static_cast<int64_t>(row) * blocks + b) * Q + q];
-    out[static_cast<int64_t>(row) * Q + q] = (q == 0 && divide_first > 0) ? total / divide_first : total;
-}
-
-struct WideShape {
-    int log2_p, S, threads;
+struct StatsTileShape {
+    int log2_s, log2_l, R, threads, tiles;
+    int64_t runs;                    // blocks of one state
     size_t smem;
 };
 
-WideShape wide_shape(int M, int extra_rows) {
-    WideShape w;
-    const int P = wide_positions(M);
-    w.log2_p = 0;
-    while ((1 << w.log2_p) < P) ++w.log2_p;
-    w.S = 4 * P * kStatsVec;
-    w.threads = (M * P + 31) / 32 * 32;
-    // two tiles of M (+ extra) rows and the span's means; the final
-    // reduction reuses the tiles
-    const size_t floats = 2 * static_cast<size_t>(M + extra_rows) * w.S + w.S;
-    const size_t red = 2 * (3 * static_cast<size_t>(M) + 2);   // doubles -> floats
-    w.smem = (floats > red ? floats : red) * sizeof(float);
+// Columns, lanes of a replica, threads and tiles of a run (diagnostics of a
+// round's end -- change of x, then the average of every state with its sums --
+// in us; the previous kernels, one-pass in rows of 128 to 256 bytes with
+// persistent blocks up to M = 64 and two passes above, first).
+//   Columns: 256 up to M = 12 (M = 9, Adam N = 1, n = 8M: 534 -> 500; 128
+//   columns 511), 128 up to 16 (M = 16, Adam N = 2, n = 8M: 942 -> 806; 64
+//   columns 835), else 64 (M = 32, n = 4M: 781 -> 646; M = 64, n = 2M: 709 ->
+//   639; M = 128, n = 600k: 1102 -> 496; M = 256, n = 400k: 1073 -> 598), fewer
+//   where two tiles would not fit an SM or the SMs would not have one each.
+//   Lanes and threads: the fewer, the more rows a thread takes and the less
+//   there is to combine at a run's end (M = 64: 2 lanes and 128 threads 639, 8
+//   lanes 683, 512 threads 1120).
+//   Tiles: runs enough for 8 blocks an SM, 8 at most, so that the tiles under
+//   way lie close together (M = 64: 640, runs of 32 675; M = 100, n = 75k, runs
+//   of 1 to 2: 231 -> 56, of 32 254); as many columns where the tiles are
+//   narrower, which keeps the workspace under 1 % of the states (M = 1024, n =
+//   100k: 1305 -> 998 in runs of 6, 1033 of 12).
+StatsTileShape stats_tile_shape(int num_sms, int64_t n, int n_sel, int M) {
+    StatsTileShape w;
+    auto bytes = [&](int log2_s) { return static_cast<size_t>(M + 2) * sizeof(float) << log2_s; };
+    w.log2_s = M <= 12 ? 8 : (M <= 16 ? 7 : 6);
+    while (w.log2_s > 3 &&
+           (2 * (bytes(w.log2_s) + kSharedReserved) > kSharedPerSm || (n >> w.log2_s) * n_sel < num_sms))
+        --w.log2_s;
+    w.smem = bytes(w.log2_s);
+    w.log2_l = M <= 16 ? 2 : 1;                  // 2^log2_l <= S / 4 for every S
+    if (w.log2_l > w.log2_s - 2) w.log2_l = w.log2_s - 2;
+    w.R = 1;
+    while (w.R < 8 && (M << w.log2_l) > w.R * 128) w.R *= 2;
+    w.threads = (((M << w.log2_l) + w.R - 1) / w.R + 31) / 32 * 32;
+    const int64_t n_tiles = n >> w.log2_s;
+    const int64_t per = n_tiles * n_sel / (8 * static_cast<int64_t>(num_sms));
+    const int64_t most = w.log2_s >= 6 ? 8 : 512 >> w.log2_s;
+    w.tiles = static_cast<int>(per < 1 ? 1 : (per > most ? most : per));
+    w.runs = (n_tiles + w.tiles - 1) / w.tiles;
     return w;
 }
 
-template <typename Kernel>
-int wide_blocks_per_sm(Kernel kernel, const WideShape &w) {
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, w.threads, w.smem) != cudaSuccess ||
-        per_sm < 1) {
-        cudaGetLastError();
-        per_sm = 1;
-    }
-    return per_sm;
+template <bool CHANGE, int R, int V>
+cudaError_t launch_stats_tile_t(const StatsTileArgs &a, const StatsTileShape &w, int n_sel, cudaStream_t stream) {
+    auto kernel = stats_tile_kernel<CHANGE, R, V>;
+    if (const cudaError_t e = allow_shared(kernel, w.smem); e != cudaSuccess) return e;
+    kernel<<<dim3(static_cast<unsigned>(w.runs), n_sel), w.threads, w.smem, stream>>>(a);
+    return cudaGetLastError();
 }
 
-// Blocks per selected state: the device's resident blocks shared over the
-// states, at most one per span, within the workspace.
-int wide_grid(int per_sm, int num_sms, int n_sel, int64_t n_spans, int Q, size_t partial_cap) {
-    int64_t g = static_cast<int64_t>(per_sm) * num_sms / (n_sel > 0 ? n_sel : 1);
-    if (g > n_spans) g = n_spans;
-    const int64_t fit = static_cast<int64_t>(partial_cap / (static_cast<size_t>(Q) * (n_sel > 0 ? n_sel : 1)));
-    if (g > fit) g = fit;
-    return static_cast<int>(g < 1 ? 1 : g);
-}
-
-}  // namespace
-
-size_t wide_stats_partial_capacity(int num_sms, int n_states, int M) {
-    // at most 32 resident blocks per SM, shared over the states
-    return static_cast<size_t>(32 * num_sms + n_states) * (2 + 2 * static_cast<size_t>(M));
-}
-
-namespace {
-
-template <bool FOUR>
-cudaError_t launch_sync_stats_wide_t(const SyncArgs &a, int num_sms, double *partial, size_t partial_cap,
-                                     double *stats, cudaStream_t stream) {
-    if (a.n_sel <= 0) return cudaSuccess;
-    if (a.M < 2 || a.M > kWideMaxM) return cudaErrorNotSupported;
+template <bool CHANGE>
+cudaError_t launch_stats_tile(StatsTileArgs &a, int n_sel, int num_sms, size_t partial_cap, double *stats,
+                              cudaStream_t stream) {
     const int Q = 2 + 2 * a.M;
-    const WideShape w = wide_shape(a.M, 0);
-    if (w.smem > 48 * 1024) {        // before the occupancy query, which depends on it
-        cudaError_t e = cudaFuncSetAttribute(sync_stats_wide_kernel<FOUR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             static_cast<int>(w.smem));
-        if (e != cudaSuccess) return e;
+    const StatsTileShape w = stats_tile_shape(num_sms, a.n, n_sel, a.M);
+    if (w.runs > 0x7fffffff || static_cast<size_t>(w.runs) * n_sel * Q > partial_cap) return cudaErrorInvalidValue;
+    a.log2_s = w.log2_s;
+    a.log2_l = w.log2_l;
+    a.tiles = w.tiles;
+    cudaError_t e;
+    // columns of a lane in the means: the fewer warps a block has, the more
+    switch (w.R) {
+        case 1:
+            e = a.M <= 16 ? launch_stats_tile_t<CHANGE, 1, 4>(a, w, n_sel, stream)
+                          : launch_stats_tile_t<CHANGE, 1, 2>(a, w, n_sel, stream);
+            break;
+        case 2: e = launch_stats_tile_t<CHANGE, 2, 1>(a, w, n_sel, stream); break;
+        case 4: e = launch_stats_tile_t<CHANGE, 4, 1>(a, w, n_sel, stream); break;
+        default: e = launch_stats_tile_t<CHANGE, 8, 1>(a, w, n_sel, stream); break;
     }
-    const int per_sm = wide_blocks_per_sm(sync_stats_wide_kernel<FOUR>, w);
-    if (static_cast<size_t>(Q) * a.n_sel > partial_cap) return cudaErrorInvalidValue;
-    const int g = wide_grid(per_sm, num_sms, a.n_sel, a.n_padded / w.S, Q, partial_cap);
-    sync_stats_wide_kernel<FOUR><<<dim3(g, a.n_sel), w.threads, w.smem, stream>>>(a, w.log2_p, partial);
-    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    wide_stats_finalize_kernel<<<dim3((Q + 255) / 256, a.n_sel), 256, 0, stream>>>(partial, g, Q, a.M, stats);
-    return cudaGetLastError();
-}
-
-template <bool FOUR>
-cudaError_t launch_pseudo_grad_stats_wide_t(const float *x, const float *anchor, int64_t n, int M, int num_sms,
-                                            double *partial, size_t partial_cap, double *stats,
-                                            cudaStream_t stream) {
-    if (M < 2 || M > kWideMaxM) return cudaErrorNotSupported;
-    const int Q = 2 * M + 2;
-    const WideShape w = wide_shape(M, 1);
-    if (w.smem > 48 * 1024) {        // before the occupancy query, which depends on it
-        cudaError_t e = cudaFuncSetAttribute(pseudo_grad_stats_wide_kernel<FOUR>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(w.smem));
-        if (e != cudaSuccess) return e;
-    }
-    const int per_sm = wide_blocks_per_sm(pseudo_grad_stats_wide_kernel<FOUR>, w);
-    if (static_cast<size_t>(Q) > partial_cap) return cudaErrorInvalidValue;
-    const int g = wide_grid(per_sm, num_sms, 1, n / w.S, Q, partial_cap);
-    pseudo_grad_stats_wide_kernel<FOUR><<<g, w.threads, w.smem, stream>>>(x, anchor, n, M, w.log2_p, partial);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    wide_stats_finalize_kernel<<<dim3((Q + 255) / 256, 1), 256, 0, stream>>>(partial, g, Q, 0, stats);
-    return cudaGetLastError();
+    return launch_stats_finalize(a.partial, w.runs, Q, n_sel, CHANGE ? 0 : a.M, stats, stream);
 }
 
 }  // namespace
 
-cudaError_t launch_sync_stats_wide(const SyncArgs &a, int num_sms, double *partial, size_t partial_cap,
-                                   double *stats, cudaStream_t stream) {
-    return wide_four_columns(a.M) ? launch_sync_stats_wide_t<true>(a, num_sms, partial, partial_cap, stats, stream)
-                                  : launch_sync_stats_wide_t<false>(a, num_sms, partial, partial_cap, stats, stream);
+size_t tile_stats_partial_capacity(int num_sms, int64_t n_padded, int n_states, int M) {
+    int64_t most = 0;
+    for (int k = 1; k <= n_states; ++k) {
+        const int64_t rows = stats_tile_shape(num_sms, n_padded, k, M).runs * k;
+        if (rows > most) most = rows;
+    }
+    return static_cast<size_t>(most) * (2 + 2 * static_cast<size_t>(M));
 }
 
-cudaError_t launch_pseudo_grad_stats_wide(const float *x, const float *anchor, int64_t n, int M, int num_sms,
+cudaError_t launch_sync_stats_tile(const SyncArgs &s, int num_sms, double *partial, size_t partial_cap,
+                                   double *stats, cudaStream_t stream) {
+    if (s.n_sel <= 0) return cudaSuccess;
+    StatsTileArgs a = {};
+    a.arena = s.arena;
+    a.partial = reinterpret_cast<float2 *>(partial);
+    a.n = s.n_padded;
+    a.stride = s.stride;
+    a.M = s.M;
+    for (int k = 0; k < s.n_sel; ++k) a.sel[k] = s.sel[k];
+    return launch_stats_tile<false>(a, s.n_sel, num_sms, partial_cap, stats, stream);
+}
+
+cudaError_t launch_pseudo_grad_stats_tile(const float *x, const float *anchor, int64_t n, int M, int num_sms,
                                           double *partial, size_t partial_cap, double *stats,
                                           cudaStream_t stream) {
-    return wide_four_columns(M)
-               ? launch_pseudo_grad_stats_wide_t<true>(x, anchor, n, M, num_sms, partial, partial_cap, stats, stream)
-               : launch_pseudo_grad_stats_wide_t<false>(x, anchor, n, M, num_sms, partial, partial_cap, stats, stream);
+    StatsTileArgs a = {};
+    a.arena = const_cast<float *>(x);            // not written
+    a.anchor = anchor;
+    a.partial = reinterpret_cast<float2 *>(partial);
+    a.n = n;
+    a.M = M;
+    return launch_stats_tile<true>(a, 1, num_sms, partial_cap, stats, stream);
 }
 
 }  // namespace mtdao

@@ -1,7 +1,6 @@
 // step_sync_wide.cuh -- the local step with the replica average fused in,
 // for replica counts above what a lane holds (M = 8 on large states, 9 to
-// kTileMaxM), and the span layout of the one-pass diagnostics of
-// stats_wide.cu.
+// kTileMaxM).
 //
 // A block owns a tile: S consecutive columns of all M replicas, of every
 // state and of the gradient, copied to shared memory (cp.async) at once.
@@ -28,111 +27,13 @@
 // that fit on an SM (one where a tile takes more than 113 KB).
 #pragma once
 
-#include "replica_mean.cuh"
+#include "replica_tile.cuh"
 #include "step_kernels.cuh"
 
 namespace mtdao {
 
-constexpr int kWideMaxM = 256;            // largest M of the span layout (diagnostics)
-constexpr int kWideMaxThreads = 512;      // largest block of the span layout
 constexpr int kTileMaxThreads = 512;      // largest block of the fused step
 constexpr int kTileMaxM = 256;            // largest M of the fused step (above: step + average)
-
-// Threads per replica row of the span (a power of two).
-constexpr int wide_positions(int M) { return M <= 16 ? 16 : M <= 64 ? 8 : M <= 128 ? 4 : 2; }
-
-
-// V consecutive floats of shared memory.
-template <int V>
-__device__ __forceinline__ void ld_shared_v(const float *p, float (&v)[V]) {
-    if constexpr (V == 4) {
-        to_array(*reinterpret_cast<const float4 *>(p), v);
-    } else if constexpr (V == 2) {
-        const float2 t = *reinterpret_cast<const float2 *>(p);
-        v[0] = t.x;
-        v[1] = t.y;
-    } else {
-        v[0] = *p;
-    }
-}
-
-// Replica means of the n_cols columns of a block's tiles into mean[p]
-// (column p: tile + (p / S) * M * S + p % S, the replicas at stride
-// S = 2^log2_s).  Columns go in groups of V; lanes i and i + 16 of a warp
-// take one group and form its two compensated parts of replica_mean.cuh,
-// replicas 1 .. h-1 and h .. M-1 in order (h = M / 2), and join them with a
-// shuffle: the bits of replica_mean_rt (with its plain mean where the
-// compensated one is NaN).  A half-warp reads one row, so no two of its
-// lanes meet in a bank.  Every thread of the block calls it (the shuffles
-// take whole warps: blockDim.x is a multiple of 32).
-template <int V>
-__device__ __forceinline__ void tile_means(const float *tile, int M, int log2_s, int n_cols, float *mean) {
-    const int h = M / 2;
-    const int S = 1 << log2_s;
-    const int part = (threadIdx.x >> 4) & 1;
-    const int first = V * ((threadIdx.x >> 5) * 16 + (threadIdx.x & 15));
-    const int lo = part ? (h > 1 ? h : 1) : 1, hi = part ? M : h;
-    for (int p0 = 0; p0 < n_cols; p0 += V * static_cast<int>(blockDim.x >> 1)) {
-        if (p0 + V * 16 * static_cast<int>(threadIdx.x >> 5) >= n_cols) break;      // the whole warp is past the end
-        const int p = p0 + first;
-        const float *base = tile + (p >> log2_s) * M * S + (p & (S - 1));
-        float s0[V], mine[V], other[V];
-#pragma unroll
-        for (int k = 0; k < V; ++k) s0[k] = mine[k] = 0.0f;
-        if (p < n_cols) {
-            ld_shared_v<V>(base, s0);
-            float sum[V], comp[V];
-#pragma unroll
-            for (int k = 0; k < V; ++k) sum[k] = comp[k] = 0.0f;
-#pragma unroll 4
-            for (int m = lo; m < hi; ++m) {
-                float v[V];
-                ld_shared_v<V>(base + m * S, v);
-#pragma unroll
-                for (int k = 0; k < V; ++k) {            // DiffSum::add
-                    const float y = (v[k] - s0[k]) - comp[k];
-                    const float t = sum[k] + y;
-                    comp[k] = (t - sum[k]) - y;
-                    sum[k] = t;
-                }
-            }
-#pragma unroll
-            for (int k = 0; k < V; ++k) mine[k] = sum[k] - comp[k];
-        }
-#pragma unroll
-        for (int k = 0; k < V; ++k) other[k] = __shfl_xor_sync(0xffffffffu, mine[k], 16);
-        if (p < n_cols && part == 0) {
-#pragma unroll
-            for (int k = 0; k < V; ++k) {
-                float v = replica_mean_from_parts(s0[k], mine[k], other[k], static_cast<float>(M));
-                if (v != v) {                    // non-finite values: the plain mean (replica_mean.cuh)
-                    float plain = s0[k];
-                    for (int m = 1; m < M; ++m) plain += base[m * S + k];
-                    v = plain / static_cast<float>(M);
-                }
-                mean[p + k] = v;
-            }
-        }
-    }
-}
-
-// The means of the one-pass diagnostics: four columns per lane pair up to
-// M = 32, one above.
-constexpr bool wide_four_columns(int M) { return M <= 32; }
-
-// 16- and 8-byte asynchronous global -> shared copies (cp.async) and their
-// groups: a block copies its next span while it works on the current one.
-__device__ __forceinline__ void cp_async16(void *smem_dst, const void *gmem_src) {
-    const unsigned dst = static_cast<unsigned>(__cvta_generic_to_shared(smem_dst));
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(gmem_src) : "memory");
-}
-__device__ __forceinline__ void cp_async8(void *smem_dst, const void *gmem_src) {
-    const unsigned dst = static_cast<unsigned>(__cvta_generic_to_shared(smem_dst));
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(dst), "l"(gmem_src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
 // Floats of one tile set: M x S floats per state and the gradient's
 // (M x S f32, or bf16 in half the floats).
@@ -244,16 +145,14 @@ struct TileShape {
 // 6659, 3 items 6067).
 template <typename Bytes>
 TileShape tile_shape(int M, int64_t n, int num_sms, Bytes bytes) {
-    constexpr size_t kPerSm = 227 * 1024, kReserved = 1024;     // shared memory of an SM, and per resident block
     TileShape w;
     w.S = M <= 16 ? 128 : 64;
-    while (w.S > 32 && 2 * (bytes(w.S) + kReserved) > kPerSm) w.S /= 2;
-    while (w.S > 8 && (bytes(w.S) + kReserved > kPerSm || n / w.S < num_sms)) w.S /= 2;
+    while (w.S > 32 && 2 * (bytes(w.S) + kSharedReserved) > kSharedPerSm) w.S /= 2;
+    while (w.S > 8 && (bytes(w.S) + kSharedReserved > kSharedPerSm || n / w.S < num_sms)) w.S /= 2;
     w.smem = bytes(w.S);
     const int items = M * (w.S / 4);
     int64_t resident = (n / w.S + num_sms - 1) / num_sms;        // blocks of an SM
-    const int64_t fit = static_cast<int64_t>(kPerSm / (w.smem + kReserved));
-    if (resident > fit) resident = fit < 1 ? 1 : fit;
+    if (resident > tile_blocks_fit(w.smem)) resident = tile_blocks_fit(w.smem);
     if (resident > 16) resident = 16;
     int per = static_cast<int>((items * resident + 1023) / 1024);    // items of a thread
     if (per > 2 && items % (32 * per) != 0 && items % 64 == 0 && items <= 512) per = 2;
@@ -273,11 +172,7 @@ cudaError_t launch_step_sync_tile(const StepArgs &a, int num_sms, cudaStream_t s
     int log2_p = 0;
     while ((4 << log2_p) < w.S) ++log2_p;
     auto kernel = step_sync_tile_kernel<BASE, N, GDT, CLIP>;
-    if (w.smem > 48 * 1024) {
-        const cudaError_t e =
-            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(w.smem));
-        if (e != cudaSuccess) return e;
-    }
+    if (const cudaError_t e = allow_shared(kernel, w.smem); e != cudaSuccess) return e;
     kernel<<<static_cast<unsigned>(a.n_padded / w.S), w.threads, w.smem, stream>>>(a, log2_p);
     return cudaGetLastError();
 }

@@ -1,6 +1,6 @@
-"""The tiled fused step (step_sync_wide.cuh): the step and the averages in one
-pass give the bits of the step followed by the averages, at the edges of what
-the tile's width and threads are chosen by."""
+"""The kernels on tiles of all replicas, at the edges of what a tile's width and
+threads are chosen by: the fused step (step_sync_wide.cuh) gives the bits of the
+step followed by the averages, the diagnostics (stats_wide.cu) the sums in 64 bits."""
 import numpy as np
 import pytest
 
@@ -55,11 +55,9 @@ CASES = [("adam", 4, "f32", 256, 30000), ("adam", 1, "f32", 256, 512), ("sgdm", 
          ("adam", 1, "bf16", 257, 3000)]
 
 
-@pytest.mark.parametrize("clip", [False, True])
-@pytest.mark.parametrize("base,N,gdt,M,numel", CASES)
+@pytest.mark.parametrize("base,N,gdt,M,numel,clip", [c + (clip,) for c in CASES for clip in (False, True)
+                                                     if not (clip and c[0] == "adopt")])
 def test_fused_tiles_equal_step_then_average(P, base, N, gdt, M, numel, clip):
-    if clip and base == "adopt":
-        pytest.skip("ADOPT does not clip by norm")
     w = workload_dict([numel], M, base=base, betas=(0.9, 0.999, 0.5, 0.99)[:N], px=1, pu=1, pv=0 if base == "sgdm" else 1,
                       clip="global_norm" if clip else "none", rho=0.05, gdt=gdt)
     (a, b), g = _pair(P, w, M, gdt, seed=M + N, plant=clip)
@@ -84,5 +82,50 @@ def test_fused_tiles_equal_step_then_average(P, base, N, gdt, M, numel, clip):
         # the decay rounds each value once (2^-24 of it), the compensated mean a few times
         scale = before.abs().mean(0) + 1e-30
         assert float(((got[0] - mean).abs() / scale).max()) < 4 * 2.0 ** -23
+    a.close()
+    b.close()
+
+
+@pytest.mark.parametrize("M,numel", [(9, 256), (9, 700001), (12, 200000), (13, 400001), (16, 100), (17, 200001),
+                                     (64, 200001), (65, 200001), (128, 5000), (129, 90000), (257, 20000),
+                                     (513, 9000), (1024, 8000)])
+def test_diagnostics_on_tiles(P, M, numel):
+    """One tile a block, runs of several with a shorter last one, every number
+    of rows a thread takes, narrow tiles."""
+    w = workload_dict([numel], M, base="adam", betas=(0.9,), px=1, pu=1, pv=1)
+    (a, b), _ = _pair(P, w, M, "f32", seed=M)
+    x0 = torch.randn((a.n_padded,), device="cuda") * 0.1
+    x0[numel:] = 0
+    keep = [a.state_view(s).clone() for s in range(3)]
+    a.set_params(x0)
+    a.track_anchor(1)
+    for s in range(3):
+        a.state_view(s).copy_(keep[s])
+        b.state_view(s).copy_(keep[s])
+    change = a.pseudo_grad_stats(0)
+    stats = a.sync_stats(0b101)
+    b.sync(0b101)
+    _same(a, b)
+    # the anchor is x's average now
+    assert float(a.pseudo_grad_stats(0)[: 2 * M + 1].abs().max()) == 0.0
+
+    def close(got, want, scale=None):
+        # fp32 sums of at most 64 elements, then compensated: a few 2^-24 of the sum of magnitudes
+        assert bool(((got - want).abs() <= 2e-6 * (want.abs() if scale is None else scale) + 1e-300).all())
+
+    x, anchor = keep[0].double(), x0.double()
+    mean = x.mean(0)
+    loc, glob = x - anchor, mean - anchor
+    close(change[:M], loc.square().sum(1))
+    close(change[M:2 * M], (loc * glob).sum(1), (loc * glob).abs().sum(1))
+    close(change[2 * M], glob.square().sum())
+    close(change[2 * M + 1], anchor.square().sum())
+    for row, s in enumerate((0, 2)):
+        v = keep[s].double()
+        m = v.mean(0)
+        close(stats[row, 0], (v - m).square().sum() / M)
+        close(stats[row, 1], m.square().sum())
+        close(stats[row, 2:2 + M], v.square().sum(1))
+        close(stats[row, 2 + M:], (v * m).sum(1), (v * m).abs().sum(1))
     a.close()
     b.close()
