@@ -19,96 +19,98 @@
 #include "mtdao_internal.h"
 #include "kahan.cuh"
 #include "replica_mean.cuh"
+#include "replica_tile.cuh"
 #include "step_kernels.cuh"
 
 namespace mtdao {
 
 namespace {
 
-// Mean of the M replicas at float4 position e of state s, M known at run
-// time (the standalone average above 14 replicas): replica_mean.cuh's operations in its order, four replicas'
-// loads in flight (one at a time, the average of M = 9-64 ran at 5.5-5.8
-// TB/s).
-__device__ __forceinline__ float4 replica_mean4(const float *s, int64_t n, int M, int64_t e) {
-    float s0[4];
-    to_array(ld_state(s + e), s0);
-    DiffSum pa[4] = {DiffSum(s0[0]), DiffSum(s0[1]), DiffSum(s0[2]), DiffSum(s0[3])};
-    DiffSum pb[4] = {DiffSum(s0[0]), DiffSum(s0[1]), DiffSum(s0[2]), DiffSum(s0[3])};
-    float plain[4] = {s0[0], s0[1], s0[2], s0[3]};
-    const int h = M / 2;
-    for (int m = 1; m < M; m += 4) {          // four replicas' loads in flight, added in order
-        float r[4][4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (m + u < M) to_array(ld_state(s + (m + u) * n + e), r[u]);
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            if (m + u >= M) break;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                if (m + u < h) pa[k].add(r[u][k]);
-                else pb[k].add(r[u][k]);
-                plain[k] += r[u][k];
-            }
-        }
-    }
-    float mean[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-        mean[k] = mean_or_plain(
-            replica_mean_from_parts(s0[k], pa[k].partial(), pb[k].partial(), static_cast<float>(M)), plain[k],
-            static_cast<float>(M));
-    return from_array(mean);
-}
-
-template <int MT>
+// One float4 position of one state per thread, the replicas in registers.
+template <int M>
 __global__ void __launch_bounds__(kThreads) sync_kernel(const SyncArgs a) {
-    const int M = MT > 0 ? MT : a.M;
     float *base = a.arena + static_cast<int64_t>(a.sel[blockIdx.y]) * a.stride;
     const int64_t n = a.n_padded;
     const int64_t nv = n / 4;
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < nv;
          i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
         const int64_t e = 4 * i;
-        float mean[4];
-        if constexpr (MT > 0) {
-            float r[MT][4];
+        float r[M][4], mean[4];
 #pragma unroll
-            for (int m = 0; m < MT; ++m) to_array(ld_state(base + m * n + e), r[m]);
+        for (int m = 0; m < M; ++m) to_array(ld_state(base + m * n + e), r[m]);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) mean[k] = replica_mean<MT>([&](int m) { return r[m][k]; });
-        } else {
-            // streamed: replicas 1 .. h-1 feed part A, h .. M-1 part B (replica_mean.cuh)
-            to_array(replica_mean4(base, n, M, e), mean);
-        }
+        for (int k = 0; k < 4; ++k) mean[k] = replica_mean<M>([&](int m) { return r[m][k]; });
         const float4 mv = from_array(mean);
+#pragma unroll
         for (int m = 0; m < M; ++m) st_state(base + m * n + e, mv);
     }
 }
 
-template <int MT>
-cudaError_t launch_sync_t(const SyncArgs &a, int num_sms, cudaStream_t stream) {
-    // M = 2 .. 14 (replicas held in registers): one float4 position per
-    // thread, like the local step's stream_grid (flat 2^27, all states, GB/s
-    // against the persistent grid: M = 2 6342 -> 7098, M = 4 6447 -> 7025,
-    // M = 8 6546 -> 6941; flat 2^30 replica-elements against the streamed
-    // loop: M = 3 4588 -> 6336, 5-7 5069 -> 6609-6658, 9-14 5564 -> 6343-6784).
-    // At 15 and 16 the replicas take 151-176 registers (M = 16: 5086 against
-    // 5796 streamed).  The streamed runtime-M loop (M > 14) keeps the
-    // persistent grid (one position per thread: 3-7 % slower at M = 9-64).
-    const int64_t nv = a.n_padded / 4;
-    const int64_t need = (nv + kThreads - 1) / kThreads;
-    int64_t gx;
-    if constexpr (MT > 0) {
-        gx = need > 0x7fffffff ? 0x7fffffff : need;
-    } else {
-        static const int per_sm = blocks_per_sm(sync_kernel<MT>);
-        gx = static_cast<int64_t>(per_sm) * num_sms / (a.n_sel > 0 ? a.n_sel : 1);
-        if (gx > need) gx = need;
-    }
-    if (gx < 1) gx = 1;
+template <int M>
+cudaError_t launch_sync_t(const SyncArgs &a, cudaStream_t stream) {
+    // M = 2 .. 14: one float4 position per thread, like the local step's
+    // stream_grid (flat 2^27, all states, GB/s against a persistent grid:
+    // M = 2 6342 -> 7098, M = 4 6447 -> 7025, M = 8 6546 -> 6941).  At 15 and
+    // 16 the replicas take 151-176 registers.
+    const int64_t need = (a.n_padded / 4 + kThreads - 1) / kThreads;
+    const int64_t gx = need > 0x7fffffff ? 0x7fffffff : need;
     dim3 grid(static_cast<unsigned>(gx), static_cast<unsigned>(a.n_sel));
-    sync_kernel<MT><<<grid, kThreads, 0, stream>>>(a);
+    sync_kernel<M><<<grid, kThreads, 0, stream>>>(a);
+    return cudaGetLastError();
+}
+
+constexpr int kSyncTileThreads = 128;
+
+// The average on one tile of S = 4 * 2^log2_p columns of all replicas per
+// block: copied to shared memory, the means formed there, stored to every
+// replica; the blocks start in index order.  Takes M > 14, where a thread
+// that streams the replicas of its position (four loads in flight, persistent
+// grid) has one long chain of loads behind its sums.  That one -> this, us:
+// M = 16, n = 8M, one state 179 -> 152; M = 32, n = 5M, 3 states 620 -> 552
+// (6.96 TB/s); M = 64, n = 2M 504 -> 448; M = 256, n = 400k 423 -> 366; M =
+// 1024, n = 100k, 2 states 520 -> 378; M = 256, n = 1000 65.5 -> 6.2.  Bound by
+// HBM; above M = 256 by the tiles of 16 to 32 columns (64 to 128 bytes a row)
+// that two of them fit on an SM with.
+template <int V>
+__global__ void __launch_bounds__(kSyncTileThreads) sync_tile_kernel(const __grid_constant__ SyncArgs a, int log2_p) {
+    extern __shared__ __align__(16) float smem[];
+    const int M = a.M;
+    const int S = 4 << log2_p;
+    const int items = M << log2_p;
+    const int64_t n = a.n_padded;
+    float *base = a.arena + static_cast<int64_t>(a.sel[blockIdx.y]) * a.stride + static_cast<int64_t>(blockIdx.x) * S;
+    float *mean = smem + M * S;
+    for (int i = threadIdx.x; i < items; i += static_cast<int>(blockDim.x))
+        cp_async16(smem + 4 * i, base + (i >> log2_p) * n + 4 * (i & ((1 << log2_p) - 1)));
+    cp_async_commit();
+    cp_async_wait<0>();
+    __syncthreads();
+    tile_means<V>(smem, M, log2_p + 2, S, mean);
+    __syncthreads();
+    for (int i = threadIdx.x; i < items; i += static_cast<int>(blockDim.x)) {
+        const int f = i & ((1 << log2_p) - 1);
+        st_state(base + (i >> log2_p) * n + 4 * f, *reinterpret_cast<const float4 *>(mean + 4 * f));
+    }
+}
+
+cudaError_t launch_sync_tile(const SyncArgs &a, int num_sms, cudaStream_t stream) {
+    auto bytes = [&](int log2_p) { return (static_cast<size_t>(a.M + 1) * 4 * sizeof(float)) << log2_p; };
+    // Columns: 128 up to M = 32 (M = 16: 152 us, 64 columns 195), 64 above (M =
+    // 64: 448, 128 columns 451), fewer where two tiles would not fit an SM or
+    // the SMs would not have one each.  128 threads: M = 32 552 us, 256 560-580,
+    // 512 824-863.
+    int log2_p = a.M <= 32 ? 5 : 4;
+    while (log2_p > 1 && (2 * (bytes(log2_p) + kSharedReserved) > kSharedPerSm ||
+                          (a.n_padded >> (log2_p + 2)) * a.n_sel < num_sms))
+        --log2_p;
+    const size_t smem = bytes(log2_p);
+    // one column per lane in the means above M = 32 (M = 256: 366 us, four 401)
+    auto kernel = a.M <= 32 ? sync_tile_kernel<4> : sync_tile_kernel<1>;
+    if (const cudaError_t e = allow_shared(kernel, smem); e != cudaSuccess) return e;
+    const int64_t gx = a.n_padded >> (log2_p + 2);
+    if (gx > 0x7fffffff) return cudaErrorInvalidValue;
+    kernel<<<dim3(static_cast<unsigned>(gx), static_cast<unsigned>(a.n_sel)), kSyncTileThreads, smem, stream>>>(
+        a, log2_p);
     return cudaGetLastError();
 }
 
@@ -522,20 +524,20 @@ cudaError_t launch_sync_stats(const SyncArgs &a, int num_sms, double *partial, s
 cudaError_t launch_sync(const SyncArgs &a, int num_sms, cudaStream_t stream) {
     if (a.n_sel <= 0 || a.M <= 1) return cudaSuccess;
     switch (a.M) {
-        case 2: return launch_sync_t<2>(a, num_sms, stream);
-        case 3: return launch_sync_t<3>(a, num_sms, stream);
-        case 4: return launch_sync_t<4>(a, num_sms, stream);
-        case 5: return launch_sync_t<5>(a, num_sms, stream);
-        case 6: return launch_sync_t<6>(a, num_sms, stream);
-        case 7: return launch_sync_t<7>(a, num_sms, stream);
-        case 8: return launch_sync_t<8>(a, num_sms, stream);
-        case 9: return launch_sync_t<9>(a, num_sms, stream);
-        case 10: return launch_sync_t<10>(a, num_sms, stream);
-        case 11: return launch_sync_t<11>(a, num_sms, stream);
-        case 12: return launch_sync_t<12>(a, num_sms, stream);
-        case 13: return launch_sync_t<13>(a, num_sms, stream);
-        case 14: return launch_sync_t<14>(a, num_sms, stream);
-        default: return launch_sync_t<0>(a, num_sms, stream);
+        case 2: return launch_sync_t<2>(a, stream);
+        case 3: return launch_sync_t<3>(a, stream);
+        case 4: return launch_sync_t<4>(a, stream);
+        case 5: return launch_sync_t<5>(a, stream);
+        case 6: return launch_sync_t<6>(a, stream);
+        case 7: return launch_sync_t<7>(a, stream);
+        case 8: return launch_sync_t<8>(a, stream);
+        case 9: return launch_sync_t<9>(a, stream);
+        case 10: return launch_sync_t<10>(a, stream);
+        case 11: return launch_sync_t<11>(a, stream);
+        case 12: return launch_sync_t<12>(a, stream);
+        case 13: return launch_sync_t<13>(a, stream);
+        case 14: return launch_sync_t<14>(a, stream);
+        default: return launch_sync_tile(a, num_sms, stream);
     }
 }
 

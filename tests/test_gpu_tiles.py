@@ -1,6 +1,7 @@
 """The kernels on tiles of all replicas, at the edges of what a tile's width and
 threads are chosen by: the fused step (step_sync_wide.cuh) gives the bits of the
-step followed by the averages, the diagnostics (stats_wide.cu) the sums in 64 bits."""
+step followed by the averages, the average (reduce_kernels.cu) those of
+replica_mean.cuh's sums, the diagnostics (stats_wide.cu) the sums in 64 bits."""
 import numpy as np
 import pytest
 
@@ -82,6 +83,47 @@ def test_fused_tiles_equal_step_then_average(P, base, N, gdt, M, numel, clip):
         # the decay rounds each value once (2^-24 of it), the compensated mean a few times
         scale = before.abs().mean(0) + 1e-30
         assert float(((got[0] - mean).abs() / scale).max()) < 4 * 2.0 ** -23
+    a.close()
+    b.close()
+
+
+def _mean32(s):
+    """replica_mean.cuh in numpy, fp32: [M][n] -> [n]."""
+    M, s0 = s.shape[0], s[0]
+    parts = []
+    for lo, hi in ((1, M // 2), (max(M // 2, 1), M)):
+        total = np.zeros_like(s0)
+        comp = np.zeros_like(s0)
+        for m in range(lo, hi):
+            y = (s[m] - s0) - comp
+            t = total + y
+            comp = (t - total) - y
+            total = t
+        parts.append(total - comp)
+    q = (parts[0] + parts[1]) / np.float32(M)
+    mean = np.where(q == 0, s0, s0 + q)
+    plain = s0.copy()
+    for m in range(1, M):
+        plain = plain + s[m]
+    return np.where(np.isnan(mean), plain / np.float32(M), mean)
+
+
+@pytest.mark.parametrize("M,numel", [(14, 3000), (15, 3000), (16, 40000), (32, 20001), (33, 20001), (64, 300),
+                                     (100, 3000), (256, 1), (257, 9000), (441, 6000), (1024, 700), (1024, 12000)])
+def test_average_on_tiles(P, M, numel):
+    w = workload_dict([numel], M, base="sgdm", betas=(0.9,), px=1, pu=1, pv=0)
+    (a, b), _ = _pair(P, w, M, "f32", seed=M, plant=True)
+    ref = [a.state_view(s).cpu().numpy() for s in range(2)]
+    with np.errstate(invalid="ignore", over="ignore"):
+        ref = [_mean32(r) for r in ref]
+    a.sync(0b11)
+    b.sync(0b10)
+    for s in range(2):
+        got = a.state_view(s).cpu().numpy()
+        nan = np.isnan(ref[s])
+        assert np.array_equal(np.isnan(got), np.broadcast_to(nan, got.shape)), s
+        assert np.array_equal(got[:, ~nan], np.broadcast_to(ref[s][~nan], got[:, ~nan].shape)), s
+    assert torch.equal(torch.nan_to_num(a.state_view(1)), torch.nan_to_num(b.state_view(1)))
     a.close()
     b.close()
 
