@@ -508,8 +508,9 @@ extern "C" int mtdao_set_params(mtdao_handle h, const float *x0_dev) {
 
 // ====================================================================== hot path
 
-// After a step or sync that averaged the states in mask, each tracked
-// anchor among them becomes the averaged value (replica 0's copy).
+// After a step that averaged the states in mask in its own pass (and with one
+// replica), each tracked anchor among them becomes the averaged value (replica
+// 0's copy); the averaging kernels store the anchors themselves.
 static int refresh_anchor(mtdao_ctx *h, uint32_t mask) {
     for (int s = 0; s < h->n_states; ++s) {
         if (h->anchor[s] == nullptr || ((mask >> s) & 1u) == 0) continue;
@@ -540,7 +541,7 @@ static int ensure_stats_workspace(mtdao_ctx *h) {
     return MTDAO_OK;
 }
 
-static int enqueue_sync(mtdao_ctx *h, uint32_t mask) {
+static SyncArgs sync_args(const mtdao_ctx *h, uint32_t mask) {
     SyncArgs a;
     std::memset(&a, 0, sizeof a);
     a.arena = h->arena;
@@ -548,7 +549,16 @@ static int enqueue_sync(mtdao_ctx *h, uint32_t mask) {
     a.stride = static_cast<int64_t>(h->M) * h->n_padded;
     a.M = h->M;
     for (int s = 0; s < h->n_states; ++s)
-        if (mask & (1u << s)) a.sel[a.n_sel++] = s;
+        if (mask & (1u << s)) {
+            a.anchor[a.n_sel] = h->anchor[s];
+            a.sel[a.n_sel++] = s;
+        }
+    return a;
+}
+
+// The average of the states in mask (M > 1) and of their anchors.
+static int enqueue_sync(mtdao_ctx *h, uint32_t mask) {
+    const SyncArgs a = sync_args(h, mask);
     cudaError_t e = launch_sync(a, h->num_sms, h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "sync launch");
     return MTDAO_OK;
@@ -576,9 +586,7 @@ extern "C" int mtdao_step(mtdao_handle h, const void *grads_dev, int32_t grad_dt
         cudaError_t e = launch_adopt_init_v(v, grads_dev, grad_dtype, static_cast<int64_t>(h->M) * h->n_padded,
                                             h->stream);
         if (e != cudaSuccess) return cuda_fail(h, e, "ADOPT initial second-moment launch");
-        if (avg_mask != 0)
-            if (int rc = enqueue_sync(h, avg_mask)) return rc;
-        if (int rc = refresh_anchor(h, sync_mask)) return rc;
+        if (int rc = avg_mask != 0 ? enqueue_sync(h, avg_mask) : refresh_anchor(h, sync_mask)) return rc;
         ++h->step;
         return MTDAO_OK;
     }
@@ -601,6 +609,7 @@ extern "C" int mtdao_step(mtdao_handle h, const void *grads_dev, int32_t grad_dt
     a.sc = step_scalars(c, h->step, lr);
 
     cudaError_t e;
+    uint32_t copy_mask = sync_mask;          // anchors that no averaging kernel stores
     if (a.sync_mask != 0) {
         e = launch_step_sync(c->base, c->n_mom, grad_dtype, clip, a, h->num_sms, h->stream);
         if (e == cudaErrorNotSupported) {
@@ -608,13 +617,14 @@ extern "C" int mtdao_step(mtdao_handle h, const void *grads_dev, int32_t grad_dt
             e = launch_step(c->base, c->n_mom, grad_dtype, clip, a, h->num_sms, h->stream);
             if (e != cudaSuccess) return cuda_fail(h, e, "step launch");
             if (int rc = enqueue_sync(h, a.sync_mask)) return rc;
+            copy_mask = 0;
             e = cudaSuccess;
         }
     } else {
         e = launch_step(c->base, c->n_mom, grad_dtype, clip, a, h->num_sms, h->stream);
     }
     if (e != cudaSuccess) return cuda_fail(h, e, "step launch");
-    if (int rc = refresh_anchor(h, sync_mask)) return rc;
+    if (int rc = refresh_anchor(h, copy_mask)) return rc;
     ++h->step;
     return MTDAO_OK;
 }
@@ -759,9 +769,7 @@ extern "C" int mtdao_sync(mtdao_handle h, uint32_t mask) {
                                               "the %d states", mask, h->n_states);
     if (mask == 0) return MTDAO_OK;
     if (int rc = select_device(h)) return rc;
-    if (h->M > 1)
-        if (int rc = enqueue_sync(h, mask)) return rc;
-    return refresh_anchor(h, mask);
+    return h->M > 1 ? enqueue_sync(h, mask) : refresh_anchor(h, mask);
 }
 
 extern "C" int mtdao_sync_stats(mtdao_handle h, uint32_t mask, double *stats_dev) {
@@ -774,19 +782,12 @@ extern "C" int mtdao_sync_stats(mtdao_handle h, uint32_t mask, double *stats_dev
     if (mask == 0) return MTDAO_OK;
     if (int rc = select_device(h)) return rc;
     if (int rc = ensure_stats_workspace(h)) return rc;
-    SyncArgs a;
-    std::memset(&a, 0, sizeof a);
-    a.arena = h->arena;
-    a.n_padded = h->n_padded;
-    a.stride = static_cast<int64_t>(h->M) * h->n_padded;
-    a.M = h->M;
-    for (int s = 0; s < h->n_states; ++s)
-        if (mask & (1u << s)) a.sel[a.n_sel++] = s;
+    const SyncArgs a = sync_args(h, mask);
     cudaError_t e = h->M <= kStatsRegisterM
                         ? launch_sync_stats(a, h->num_sms, h->stats_partial, h->stats_cap, stats_dev, h->stream)
                         : launch_sync_stats_tile(a, h->num_sms, h->stats_partial, h->stats_cap, stats_dev, h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "sync with diagnostics launch");
-    return refresh_anchor(h, mask);
+    return h->M > 1 ? MTDAO_OK : refresh_anchor(h, mask);
 }
 
 extern "C" int mtdao_track_anchor(mtdao_handle h, uint32_t state_mask) {

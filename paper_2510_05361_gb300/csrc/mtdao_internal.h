@@ -78,6 +78,7 @@ struct SyncArgs {
     int32_t M;
     int32_t n_sel;                   // number of states to average
     int32_t sel[2 + MTDAO_MAX_MOM];  // their indices
+    float *anchor[2 + MTDAO_MAX_MOM];    // [n_padded] copy of the mean of the k-th selected state, or nullptr
 };
 
 // Local step over all replicas (one pass).  Returns the launch error.

@@ -28,7 +28,7 @@ namespace {
 
 // One float4 position of one state per thread, the replicas in registers.
 template <int M>
-__global__ void __launch_bounds__(kThreads) sync_kernel(const SyncArgs a) {
+__global__ void __launch_bounds__(kThreads) sync_kernel(const __grid_constant__ SyncArgs a) {
     float *base = a.arena + static_cast<int64_t>(a.sel[blockIdx.y]) * a.stride;
     const int64_t n = a.n_padded;
     const int64_t nv = n / 4;
@@ -43,6 +43,7 @@ __global__ void __launch_bounds__(kThreads) sync_kernel(const SyncArgs a) {
         const float4 mv = from_array(mean);
 #pragma unroll
         for (int m = 0; m < M; ++m) st_state(base + m * n + e, mv);
+        if (a.anchor[blockIdx.y] != nullptr) st_state(a.anchor[blockIdx.y] + e, mv);
     }
 }
 
@@ -91,6 +92,10 @@ __global__ void __launch_bounds__(kSyncTileThreads) sync_tile_kernel(const __gri
         const int f = i & ((1 << log2_p) - 1);
         st_state(base + (i >> log2_p) * n + 4 * f, *reinterpret_cast<const float4 *>(mean + 4 * f));
     }
+    float *anchor = a.anchor[blockIdx.y];
+    if (anchor != nullptr && threadIdx.x < (1 << log2_p))
+        st_state(anchor + static_cast<int64_t>(blockIdx.x) * S + 4 * threadIdx.x,
+                 *reinterpret_cast<const float4 *>(mean + 4 * threadIdx.x));
 }
 
 cudaError_t launch_sync_tile(const SyncArgs &a, int num_sms, cudaStream_t stream) {
@@ -302,10 +307,12 @@ constexpr int kSyncStatsTile = 128;
 //   q = 2 + m      s_m^2
 //   q = 2 + M + m  s_m * s_bar
 // written to partial[(sel * Q + q) * gridDim.x + block], Q = 2 + 2M.  s_bar
-// is the fp32 mean that is stored.  With M = 1 nothing is stored (there is
-// nothing to average) but the sums are still formed.
+// is the fp32 mean that is stored, to the state's anchor too where it has one
+// (a copy of replica 0 after the pass took 176 us of the ~124M list's 2942 at
+// a round's end).  With M = 1 nothing is stored (there is nothing to average)
+// but the sums are still formed.
 template <int M>
-__global__ void __launch_bounds__(kThreads) sync_stats_kernel(const SyncArgs a, double *partial) {
+__global__ void __launch_bounds__(kThreads) sync_stats_kernel(const __grid_constant__ SyncArgs a, double *partial) {
     constexpr int Q = 2 + 2 * M;
     float *base = a.arena + static_cast<int64_t>(a.sel[blockIdx.y]) * a.stride;
     const int64_t n = a.n_padded;
@@ -342,6 +349,7 @@ __global__ void __launch_bounds__(kThreads) sync_stats_kernel(const SyncArgs a, 
             const float4 mv = from_array(mean);
 #pragma unroll
             for (int m = 0; m < M; ++m) st_state(base + m * n + e, mv);
+            if (a.anchor[blockIdx.y] != nullptr) st_state(a.anchor[blockIdx.y] + e, mv);
         }
     }
     __shared__ double part[Q][kThreads / 32];

@@ -30,6 +30,7 @@ constexpr int kStatsTileThreads = 256;
 struct StatsTileArgs {
     float *arena;                    // state sel[blockIdx.y] at arena + sel * stride, [M][n]
     const float *anchor;             // change diagnostics: [n]
+    float *new_anchor[2 + MTDAO_MAX_MOM];    // sync diagnostics: [n] copy of the mean, or nullptr
     float2 *partial;                 // [state][Q][gridDim.x]: Kahan sums
     int64_t n, stride;
     int32_t sel[2 + MTDAO_MAX_MOM];
@@ -140,6 +141,9 @@ __global__ void __launch_bounds__(kStatsTileThreads) stats_tile_kernel(const __g
                 const int f = i & ((1 << log2_p) - 1);
                 st_state(base + (i >> log2_p) * n + col0 + 4 * f, *reinterpret_cast<const float4 *>(mean + 4 * f));
             }
+            float *to = a.new_anchor[blockIdx.y];
+            if (to != nullptr && t < (1 << log2_p))
+                st_state(to + col0 + 4 * t, *reinterpret_cast<const float4 *>(mean + 4 * t));
         }
         __syncthreads();                         // the tile and the means are rewritten next
     }
@@ -262,7 +266,10 @@ cudaError_t launch_sync_stats_tile(const SyncArgs &s, int num_sms, double *parti
     a.n = s.n_padded;
     a.stride = s.stride;
     a.M = s.M;
-    for (int k = 0; k < s.n_sel; ++k) a.sel[k] = s.sel[k];
+    for (int k = 0; k < s.n_sel; ++k) {
+        a.sel[k] = s.sel[k];
+        a.new_anchor[k] = s.anchor[k];
+    }
     return launch_stats_tile<false>(a, s.n_sel, num_sms, partial_cap, stats, stream);
 }
 

@@ -198,3 +198,34 @@ def test_pseudo_grad_stats_needs_an_anchor(P):
         P.mtdao_track_anchor(eng.h, 1 << 5)
     assert e.value.code == P.ERR_INVALID
     eng.close()
+
+
+@pytest.mark.parametrize("M", [1, 2, 8, 14, 15, 40, 257])
+@pytest.mark.parametrize("how", ["sync", "sync_stats", "step", "adopt_first_step"])
+def test_anchors_follow_every_average(P, M, how):
+    """The averaging kernels store the anchors of the states they average; the
+    others keep theirs."""
+    w = workload_dict([3000, 11], M, base="adopt", betas=(0.9, 0.99), px=4, pu=[4, 4], pv=4)
+    w["opt"]["adopt_prev_v"] = how == "adopt_first_step"
+    eng = P.MTDAO(w["opt"], M, w["shapes"])
+    n = eng.n_padded
+    gen = torch.Generator(device="cuda").manual_seed(M)
+    eng.track_anchor(0b1011)                          # x, u1 and v
+    for s in range(4):
+        eng.state_view(s).copy_(torch.rand((M, n), device="cuda", generator=gen) + 0.5)
+    if how != "adopt_first_step":
+        eng.t = 7
+    mask = 0b1101
+    if how == "sync":
+        eng.sync(mask)
+    elif how == "sync_stats":
+        eng.sync_stats(mask)
+    else:
+        eng.step(torch.randn((M, n), device="cuda", generator=gen) * 0.01, 1e-3, mask)
+    for s in (0, 3):                                  # averaged: nothing has changed since
+        assert float(eng.pseudo_grad_stats(s)[:2 * M + 1].abs().max()) == 0.0, s
+    assert float(eng.pseudo_grad_stats(1)[:M].min()) > 0.0       # not averaged: still against zero
+    assert float(eng.pseudo_grad_stats(1)[2 * M + 1]) == 0.0
+    with pytest.raises(P.MTDAOError):
+        eng.pseudo_grad_stats(2)
+    eng.close()
