@@ -285,20 +285,23 @@ __global__ void __launch_bounds__(kNormThreads) sqnorm_finalize_kernel(const dou
 
 // ---------------------------------------------------------------- sync + diagnostics
 
-// Float4 positions a thread of sync_stats_kernel takes, consecutive for its
-// block: block b covers positions [b * tile * 256, (b + 1) * tile * 256).
-// One block per tile, started in index order as earlier blocks retire;
-// every block leaves one row of sums for stats_finalize_kernel, so the sums
-// do not depend on the SM count.  A block's fixed cost is that row (2M + 2
-// warp and block reductions in fp64), so the tile must be long.  On the ~1B
-// and ~350M workloads this launch took the sync with diagnostics from
-// 6426 / 6335 GB/s (persistent grid: occupancy x SMs blocks, grid-stride)
-// to 6712 / 6696.  On flat 2^30-element sets (GB/s at M = 4 / 8):
-// persistent 5943 / 6139; tiles of 2: 1621 / 1795, 8: 5638 / 4590,
-// 32: 6152 / 6275, 128: 6121 / 6308, 512: 6051 / 6173.  The read-only
-// pseudo-gradient pass keeps the persistent grid: with tiles of 512 it ran
-// 6212 / 5908 GB/s on the two workloads against 7153 / 6237.
-constexpr int kSyncStatsTile = 128;
+// The block's sums of Q values per thread, value j to out[j * gridDim.x].
+template <int Q>
+__device__ __forceinline__ void block_sums(const Kahan (&acc)[Q], float2 *out) {
+    __shared__ float2 part[Q][kThreads / 32];
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+#pragma unroll
+    for (int j = 0; j < Q; ++j) {
+        const Kahan v = lanes_sum(acc[j], 32);
+        if (l == 0) part[j][w] = make_float2(v.s, v.c);
+    }
+    __syncthreads();
+    if (threadIdx.x < Q) {
+        Kahan total;
+        for (int i = 0; i < kThreads / 32; ++i) total = total + Kahan{part[threadIdx.x][i].x, part[threadIdx.x][i].y};
+        out[static_cast<int64_t>(threadIdx.x) * gridDim.x] = make_float2(total.s, total.c);
+    }
+}
 
 // Replica average of the selected states (exactly as sync_kernel) plus, in
 // the same pass over the M replicas, per state and block the partial sums of
@@ -309,17 +312,17 @@ constexpr int kSyncStatsTile = 128;
 // written to partial[(sel * Q + q) * gridDim.x + block], Q = 2 + 2M.  s_bar
 // is the fp32 mean that is stored, to the state's anchor too where it has one
 // (a copy of replica 0 after the pass took 176 us of the ~124M list's 2942 at
-// a round's end).  With M = 1 nothing is stored (there is nothing to average)
+// a round's end).  The sums travel as compensated fp32 pairs.  With M = 1 nothing is stored (there is nothing to average)
 // but the sums are still formed.
 template <int M>
-__global__ void __launch_bounds__(kThreads) sync_stats_kernel(const __grid_constant__ SyncArgs a, double *partial) {
+__global__ void __launch_bounds__(kThreads) sync_stats_kernel(const __grid_constant__ SyncArgs a, int tile, float2 *partial) {
     constexpr int Q = 2 + 2 * M;
     float *base = a.arena + static_cast<int64_t>(a.sel[blockIdx.y]) * a.stride;
     const int64_t n = a.n_padded;
     const int64_t nv = n / 4;
     Kahan acc[Q];
-    const int64_t first = static_cast<int64_t>(blockIdx.x) * kSyncStatsTile * blockDim.x + threadIdx.x;
-    for (int k = 0; k < kSyncStatsTile; ++k) {
+    const int64_t first = static_cast<int64_t>(blockIdx.x) * tile * blockDim.x + threadIdx.x;
+    for (int k = 0; k < tile; ++k) {
         const int64_t i = first + static_cast<int64_t>(k) * blockDim.x;
         if (i >= nv) break;
         const int64_t e = 4 * i;
@@ -352,45 +355,35 @@ __global__ void __launch_bounds__(kThreads) sync_stats_kernel(const __grid_const
             if (a.anchor[blockIdx.y] != nullptr) st_state(a.anchor[blockIdx.y] + e, mv);
         }
     }
-    __shared__ double part[Q][kThreads / 32];
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-#pragma unroll
-    for (int j = 0; j < Q; ++j) {
-        const double v = warp_sum(acc[j].value());
-        if (l == 0) part[j][w] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < Q) {
-        double total = 0.0;
-        for (int i = 0; i < static_cast<int>(blockDim.x >> 5); ++i) total += part[threadIdx.x][i];
-        partial[(static_cast<int64_t>(blockIdx.y) * Q + threadIdx.x) * gridDim.x + blockIdx.x] = total;
-    }
+    block_sums<Q>(acc, partial + static_cast<int64_t>(blockIdx.y) * Q * gridDim.x + blockIdx.x);
 }
 
-// stats[row * Q + q] = the sum over blocks of partial[(row * Q + q) * blocks + b]:
-// thread t of block (q, row) adds a contiguous run of blocks in order, then
-// block_sum adds the threads' sums in a fixed order.  q = 0 is divided by
+// stats[row * Q + q] = the sum over blocks of partial[(row * Q + q) * blocks + b]
+// (Kahan sums): thread t of block (q, row) adds blocks t, t + 256, ... in
+// order, then lanes and warps combine in a fixed order.  q = 0 is divided by
 // divide_first (M for the variance, a mean over workers; 0 leaves it).
-// A value is a double, or a Kahan sum (x - y).
-__device__ __forceinline__ double wide_value(double v) { return v; }
-__device__ __forceinline__ double wide_value(float2 v) { return static_cast<double>(v.x) - static_cast<double>(v.y); }
-
-template <typename T>
-__global__ void __launch_bounds__(kNormThreads) stats_finalize_kernel(const T *partial, int64_t blocks,
-                                                                      int Q, int divide_first, double *stats) {
+__global__ void __launch_bounds__(kNormThreads) stats_finalize_kernel(const float2 *partial, int64_t blocks, int Q,
+                                                                      int divide_first, double *stats) {
     const int q = blockIdx.x, row = blockIdx.y;
-    const T *p = partial + (static_cast<int64_t>(row) * Q + q) * blocks;
-    const int64_t per = (blocks + blockDim.x - 1) / blockDim.x;
-    const int64_t lo = threadIdx.x * per;
-    const int64_t hi = lo + per < blocks ? lo + per : blocks;
-    double acc = 0.0;
-    for (int64_t b = lo; b < hi; ++b) acc += wide_value(p[b]);
-    const double total = block_sum(acc);
-    if (threadIdx.x == 0) stats[row * Q + q] = (q == 0 && divide_first > 0) ? total / divide_first : total;
+    const float2 *p = partial + (static_cast<int64_t>(row) * Q + q) * blocks;
+    Kahan acc;
+#pragma unroll 4
+    for (int64_t b = threadIdx.x; b < blocks; b += kNormThreads) {
+        const float2 v = p[b];
+        acc = acc + Kahan{v.x, v.y};
+    }
+    __shared__ float2 part[kNormThreads / 32];
+    acc = lanes_sum(acc, 32);
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = make_float2(acc.s, acc.c);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double total = 0.0;
+        for (int i = 0; i < kNormThreads / 32; ++i)
+            total += static_cast<double>(part[i].x) - static_cast<double>(part[i].y);
+        stats[row * Q + q] = (q == 0 && divide_first > 0) ? total / divide_first : total;
+    }
 }
 
-// Blocks of a register-resident diagnostics kernel per state: each covers
-// `tile` consecutive float4 positions per thread.
 int64_t stats_blocks(int64_t n_padded, int tile) {
     const int64_t nv = n_padded / 4;
     const int64_t per_block = static_cast<int64_t>(tile) * kThreads;
@@ -398,17 +391,39 @@ int64_t stats_blocks(int64_t n_padded, int tile) {
     return b < 1 ? 1 : b;
 }
 
+// Float4 positions a thread of sync_stats_kernel takes, consecutive for its
+// block: block b covers positions [b * tile * 256, (b + 1) * tile * 256) of a
+// state.  One block per tile, started in index order as earlier blocks retire;
+// every block leaves one row of sums for stats_finalize_kernel, so the sums
+// do not depend on the SM count.  A short tile keeps the addresses under way
+// close together; what it pays for is the row at its end (2M + 2 block
+// reductions, as compensated fp32 pairs: in fp64, at 16 issue cycles an
+// instruction, only tiles of 128 and more paid).  The average of 4 states with
+// its sums, us, with tiles of 128 and fp64 rows -> of 16, here (in brackets 4,
+// 8, 32, 128): M = 2, n = 60M 716 -> 611 (639, 612, 615, 656); M = 4, n = 60M
+// 1291 -> 1173 (1156, 1172, 1179, 1232; 6.57 TB/s); M = 8, n = 30M 1311 -> 1164
+// (1190, 1166, 1173, 1266); M = 1 401 -> 388 (494, 414, 375, 387).  Smaller
+// states take shorter tiles, down to two positions, for 256 blocks: M = 4,
+// n = 1M 89 -> 25, n = 100k 61 -> 14 (tiles of 16 19).
+int sync_stats_tile(int64_t n_padded) {
+    int tile = 16;
+    while (tile > 2 && stats_blocks(n_padded, tile) < 256) tile /= 2;
+    return tile;
+}
+
 template <int M>
 cudaError_t launch_sync_stats_t(const SyncArgs &a, double *partial, size_t partial_cap, double *stats,
                                 cudaStream_t stream) {
     constexpr int Q = 2 + 2 * M;
-    const int64_t gx = stats_blocks(a.n_padded, kSyncStatsTile);
+    const int tile = sync_stats_tile(a.n_padded);
+    const int64_t gx = stats_blocks(a.n_padded, tile);
     if (static_cast<size_t>(gx) * a.n_sel * Q > partial_cap || gx > 0x7fffffff) return cudaErrorInvalidValue;
     dim3 grid(static_cast<unsigned>(gx), static_cast<unsigned>(a.n_sel));
-    sync_stats_kernel<M><<<grid, kThreads, 0, stream>>>(a, partial);
+    float2 *sums = reinterpret_cast<float2 *>(partial);
+    sync_stats_kernel<M><<<grid, kThreads, 0, stream>>>(a, tile, sums);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    stats_finalize_kernel<<<dim3(Q, a.n_sel), kNormThreads, 0, stream>>>(partial, gx, Q, M, stats);
+    stats_finalize_kernel<<<dim3(Q, a.n_sel), kNormThreads, 0, stream>>>(sums, gx, Q, M, stats);
     return cudaGetLastError();
 }
 
@@ -420,10 +435,12 @@ cudaError_t launch_sync_stats_t(const SyncArgs &a, double *partial, size_t parti
 //   q = 2M         (x_bar - a)^2
 //   q = 2M + 1     a^2
 // x_bar is the replica mean of replica_mean.cuh (the value an average would
-// store now).
+// store now).  Blocks in index order with 16 positions a thread, as the sync
+// diagnostics have them, took 186 us where this takes 176 (M = 4, n = 60M: 6.8
+// TB/s; 197 with fp64 rows).
 template <int M>
 __global__ void __launch_bounds__(kThreads) pseudo_grad_stats_kernel(const float *x, const float *anchor,
-                                                                     int64_t n, double *partial) {
+                                                                     int64_t n, float2 *partial) {
     constexpr int Q = 2 * M + 2;
     const int64_t nv = n / 4;
     Kahan acc[Q];
@@ -453,19 +470,7 @@ __global__ void __launch_bounds__(kThreads) pseudo_grad_stats_kernel(const float
 #pragma unroll
         for (int j = 0; j < Q; ++j) acc[j].add(q[j]);
     }
-    __shared__ double part[Q][kThreads / 32];
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-#pragma unroll
-    for (int j = 0; j < Q; ++j) {
-        const double v = warp_sum(acc[j].value());
-        if (l == 0) part[j][w] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < Q) {
-        double total = 0.0;
-        for (int i = 0; i < static_cast<int>(blockDim.x >> 5); ++i) total += part[threadIdx.x][i];
-        partial[static_cast<int64_t>(threadIdx.x) * gridDim.x + blockIdx.x] = total;
-    }
+    block_sums<Q>(acc, partial + blockIdx.x);
 }
 
 template <int M>
@@ -479,11 +484,12 @@ cudaError_t launch_pseudo_grad_stats_t(const float *x, const float *anchor, int6
     if (gx > need) gx = need;
     if (gx < 1) gx = 1;
     if (static_cast<size_t>(gx) * Q > partial_cap) return cudaErrorInvalidValue;
-    pseudo_grad_stats_kernel<M><<<static_cast<unsigned>(gx), kThreads, 0, stream>>>(x, anchor, n, partial);
+    float2 *sums = reinterpret_cast<float2 *>(partial);
+    pseudo_grad_stats_kernel<M><<<static_cast<unsigned>(gx), kThreads, 0, stream>>>(x, anchor, n, sums);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     // the same fixed-order finalisation as the sync diagnostics, with no division
-    stats_finalize_kernel<<<dim3(Q, 1), kNormThreads, 0, stream>>>(partial, gx, Q, 0, stats);
+    stats_finalize_kernel<<<dim3(Q, 1), kNormThreads, 0, stream>>>(sums, gx, Q, 0, stats);
     return cudaGetLastError();
 }
 
@@ -508,7 +514,7 @@ cudaError_t launch_pseudo_grad_stats(const float *x, const float *anchor, int64_
 size_t sync_stats_partial_capacity(int num_sms, int64_t n_padded, int n_states, int M) {
     // one row of 2 + 2M sums per block and state, or per persistent block
     // of the pseudo-gradient pass (at most 16 resident blocks per SM)
-    const size_t sync = static_cast<size_t>(stats_blocks(n_padded, kSyncStatsTile)) * n_states;
+    const size_t sync = static_cast<size_t>(stats_blocks(n_padded, sync_stats_tile(n_padded))) * n_states;
     const size_t change = static_cast<size_t>(16) * num_sms;
     return (sync > change ? sync : change) * (2 + 2 * static_cast<size_t>(M));
 }

@@ -171,3 +171,9 @@ def test_diagnostics_on_tiles(P, M, numel):
         close(stats[row, 2 + M:], (v * m).sum(1), (v * m).abs().sum(1))
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("M,numel", [(1, 5), (2, 1024), (3, 2049), (4, 600000), (5, 1100001), (8, 2200003), (7, 4200000)])
+def test_register_diagnostics_tiles(P, M, numel):
+    """Tiles of 2 to 16 positions per thread, the last one partly filled."""
+    test_diagnostics_on_tiles(P, M, numel)
