@@ -24,7 +24,7 @@ namespace mtdao {
 //   M = 8       : two groups (half-warps) of R = 4, V = 4: replicas 0..3 and
 //                 4..7 are the two parts of the compensated mean of
 //                 replica_mean.cuh, combined by shuffles.
-// M = 8 on large states and M from 9 to 256 take the tiled kernel of
+// M = 6 to 8 on large states (fused_tile_from) and M from 9 to 256 take the tiled kernel of
 // step_sync_wide.cuh (lane groups went further before: M = 16 as four groups
 // of four replicas, the compensated sums handed from group to group by
 // shuffles, ran at 4.9-5.3 TB/s against 6.7-6.9); above 256, the plain step
@@ -139,8 +139,37 @@ __device__ __forceinline__ void load_replicas(const float *state, int64_t n_padd
     for (int r = 0; r < S::R; ++r) ld_v<S::V>(state + (grp * S::R + r) * n_padded + e, val[r]);
 }
 
+// Blocks of an SM that the registers are cut for: two (128 registers), three
+// (80) where that ran faster on flat 20M vectors with every state due (us, two
+// -> three): M = 5 Adam N = 1 to 4 500 -> 428, 604 -> 552, 754 -> 680, 865 ->
+// 835, ADOPT 499 -> 437, 621 -> 551, 879 -> 822, bf16 ADOPT N = 3 770 -> 651;
+// M = 6 ADOPT N = 1 to 3 569 -> 527, 709 -> 681, 877 -> 814 (N = 4 1008 -> 1050,
+// Adam N = 3 874 -> 894); M = 4 Adam N = 3 783 -> 820, M = 7 Adam N = 2 785 -> 925.
+template <int BASE, int N, int M>
+constexpr int fused_blocks_per_sm() {
+    return M == 5 || (M == 6 && BASE == MTDAO_BASE_ADOPT && N <= 3) ? 3 : 2;
+}
+
+// Smallest n that the tiled kernel of step_sync_wide.cuh takes for M = 6, 7
+// and 8 (0: none); us here -> tiled, every state due.
+//   n = 4M, M = 6: Adam N = 2, 3 149 -> 152, 187 -> 174, SGDM 79 -> 78; M = 7:
+//   Adam 141 -> 137, SGDM N = 2 124 -> 121, ADOPT N = 4 251 -> 246.
+//   M = 8: n = 200k (in L2) 12.0 -> 16.4, 1M (Adam N = 3) 60 -> 63, 2M (ADOPT,
+//   bf16) 98 -> 100, 4M (bf16) 224 -> 215, 20M 3 to 7 % faster (Adam, ADOPT, SGDM, N = 1 to 4).
+//   n = 20M, M = 6: Adam N = 1 to 4 570 -> 529, 690 -> 691, 874 -> 799, 989 ->
+//   923, SGDM N = 1, 2, 4 363 -> 344, 506 -> 453, 814 -> 767, ADOPT N = 4 1008
+//   -> 964 (N = 2 681 -> 737); M = 7: Adam N = 1, 3, 4 639 -> 621, 984 -> 982,
+//   1138 -> 1078 (N = 2 785 -> 798), SGDM 429 -> 401, 566 -> 547, 938 -> 904,
+//   ADOPT N = 3, 4 1004 -> 964, 1181 -> 1136 (N = 2 801 -> 853).
+template <int BASE, int N>
+constexpr int64_t fused_tile_from(int M) {
+    constexpr bool adopt = BASE == MTDAO_BASE_ADOPT, adam = BASE == MTDAO_BASE_ADAM;
+    const bool faster = M == 8 || ((M == 6 || M == 7) && (adopt ? N >= 10 - M : !(adam && N == 2)));
+    return faster ? int64_t{1} << 22 : 0;
+}
+
 template <int BASE, int N, int GDT, bool CLIP, int M>
-__global__ void __launch_bounds__(kThreads, 2) step_sync_kernel(const StepArgs a) {
+__global__ void __launch_bounds__(kThreads, (fused_blocks_per_sm<BASE, N, M>())) step_sync_kernel(const StepArgs a) {
     using S = FusedShape<M>;
     constexpr int R = S::R;
     constexpr int V = S::V;
@@ -261,10 +290,11 @@ cudaError_t launch_step_sync_t(const StepArgs &a, int num_sms, cudaStream_t stre
     // M = 4 N = 2..4 6.6 -> 6.9-7.0 TB/s, SGDM N = 1 6487 -> 7061, but Adam
     // N = 1 6713 -> 6460 (M = 2), 6725 -> 6120 (M = 4), 6108 -> 5346 (M = 3)
     // and ADOPT N = 1 6447 -> 6248.  The 64-element chunks of M >= 5 keep
-    // the persistent grid (M = 8, ~350M workload: 6504 -> 6409).
+    // the persistent grid (M = 8, ~350M workload: 6504 -> 6409), but for M =
+    // 5's SGDM (n = 20M, N = 1, 4: 310 -> 288, 693 -> 666 us).
     auto kernel = step_sync_kernel<BASE, N, GDT, CLIP, M>;
     int grid;
-    if constexpr (FusedShape<M>::kChunk >= 128 && (N >= 2 || BASE == MTDAO_BASE_SGDM)) {
+    if constexpr (M <= 5 && (BASE == MTDAO_BASE_SGDM || (N >= 2 && M <= 4))) {
         grid = stream_grid(a.n_padded / FusedShape<M>::kChunk);
     } else {
         static const int per_sm = blocks_per_sm(kernel);
@@ -276,6 +306,8 @@ cudaError_t launch_step_sync_t(const StepArgs &a, int num_sms, cudaStream_t stre
 
 template <int BASE, int N, int GDT, bool CLIP>
 cudaError_t launch_step_sync_m(const StepArgs &a, int num_sms, cudaStream_t st) {
+    const int64_t from = fused_tile_from<BASE, N>(a.M);
+    if (from > 0 && a.n_padded >= from) return launch_step_sync_tile<BASE, N, GDT, CLIP>(a, num_sms, st);
     switch (a.M) {
         case 2: return launch_step_sync_t<BASE, N, GDT, CLIP, 2>(a, num_sms, st);
         case 3: return launch_step_sync_t<BASE, N, GDT, CLIP, 3>(a, num_sms, st);
@@ -283,12 +315,7 @@ cudaError_t launch_step_sync_m(const StepArgs &a, int num_sms, cudaStream_t st) 
         case 5: return launch_step_sync_t<BASE, N, GDT, CLIP, 5>(a, num_sms, st);
         case 6: return launch_step_sync_t<BASE, N, GDT, CLIP, 6>(a, num_sms, st);
         case 7: return launch_step_sync_t<BASE, N, GDT, CLIP, 7>(a, num_sms, st);
-        case 8:
-            // flat vectors, GB/s here / tiled: n = 200k (in L2) 3742 / 2724,
-            // 1M (Adam N = 3) 5865 / 5544, 4M (bf16) 5992 / 6245, 20M 6417-6592
-            // / 6553-6939 (Adam, ADOPT, SGDM, N = 1 to 4)
-            if (a.n_padded < int64_t{1} << 21) return launch_step_sync_t<BASE, N, GDT, CLIP, 8>(a, num_sms, st);
-            return launch_step_sync_tile<BASE, N, GDT, CLIP>(a, num_sms, st);
+        case 8: return launch_step_sync_t<BASE, N, GDT, CLIP, 8>(a, num_sms, st);
         default: return launch_step_sync_tile<BASE, N, GDT, CLIP>(a, num_sms, st);
     }
 }

@@ -1,6 +1,6 @@
 // step_sync_wide.cuh -- the local step with the replica average fused in,
-// for replica counts above what a lane holds (M = 8 on large states, 9 to
-// kTileMaxM).
+// for replica counts above what a lane holds (M = 6 to 8 on large states, 9
+// to kTileMaxM).
 //
 // A block owns a tile: S consecutive columns of all M replicas, of every
 // state and of the gradient, copied to shared memory (cp.async) at once.
