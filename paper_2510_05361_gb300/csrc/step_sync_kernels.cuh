@@ -145,31 +145,35 @@ __device__ __forceinline__ void load_replicas(const float *state, int64_t n_padd
 // 835, ADOPT 499 -> 437, 621 -> 551, 879 -> 822, bf16 ADOPT N = 3 770 -> 651;
 // M = 6 ADOPT N = 1 to 3 569 -> 527, 709 -> 681, 877 -> 814 (N = 4 1008 -> 1050,
 // Adam N = 3 874 -> 894); M = 4 Adam N = 3 783 -> 820, M = 7 Adam N = 2 785 -> 925.
+// Below kFusedThreeFrom elements the SMs have no third block to take (M = 5,
+// ADOPT N = 4, n = 20k, where 80 registers spill: 8.5 us with two, 10.3).
 template <int BASE, int N, int M>
-constexpr int fused_blocks_per_sm() {
-    return M == 5 || (M == 6 && BASE == MTDAO_BASE_ADOPT && N <= 3) ? 3 : 2;
-}
+constexpr int kFusedBlocksPerSm = M == 5 || (M == 6 && BASE == MTDAO_BASE_ADOPT && N <= 3) ? 3 : 2;
+constexpr int64_t kFusedThreeFrom = int64_t{1} << 16;
 
 // Smallest n that the tiled kernel of step_sync_wide.cuh takes for M = 6, 7
 // and 8 (0: none); us here -> tiled, every state due.
 //   n = 4M, M = 6: Adam N = 2, 3 149 -> 152, 187 -> 174, SGDM 79 -> 78; M = 7:
 //   Adam 141 -> 137, SGDM N = 2 124 -> 121, ADOPT N = 4 251 -> 246.
 //   M = 8: n = 200k (in L2) 12.0 -> 16.4, 1M (Adam N = 3) 60 -> 63, 2M (ADOPT,
-//   bf16) 98 -> 100, 4M (bf16) 224 -> 215, 20M 3 to 7 % faster (Adam, ADOPT, SGDM, N = 1 to 4).
+//   bf16) 98 -> 100, 4M (bf16) 224 -> 215, 20M 3 to 7 % faster (Adam, ADOPT,
+//   SGDM, N = 1 to 4) but for ADOPT's N = 3 and 4 with f32 gradients (n = 5M
+//   298 -> 308, 348 -> 354, 20M 1086 -> 1110, 1282 -> 1276; bf16 353 -> 352).
 //   n = 20M, M = 6: Adam N = 1 to 4 570 -> 529, 690 -> 691, 874 -> 799, 989 ->
 //   923, SGDM N = 1, 2, 4 363 -> 344, 506 -> 453, 814 -> 767, ADOPT N = 4 1008
 //   -> 964 (N = 2 681 -> 737); M = 7: Adam N = 1, 3, 4 639 -> 621, 984 -> 982,
 //   1138 -> 1078 (N = 2 785 -> 798), SGDM 429 -> 401, 566 -> 547, 938 -> 904,
 //   ADOPT N = 3, 4 1004 -> 964, 1181 -> 1136 (N = 2 801 -> 853).
-template <int BASE, int N>
+template <int BASE, int N, int GDT>
 constexpr int64_t fused_tile_from(int M) {
     constexpr bool adopt = BASE == MTDAO_BASE_ADOPT, adam = BASE == MTDAO_BASE_ADAM;
-    const bool faster = M == 8 || ((M == 6 || M == 7) && (adopt ? N >= 10 - M : !(adam && N == 2)));
+    const bool faster = (M == 8 && !(adopt && N >= 3 && GDT == MTDAO_F32)) ||
+                        ((M == 6 || M == 7) && (adopt ? N >= 10 - M : !(adam && N == 2)));
     return faster ? int64_t{1} << 22 : 0;
 }
 
-template <int BASE, int N, int GDT, bool CLIP, int M>
-__global__ void __launch_bounds__(kThreads, (fused_blocks_per_sm<BASE, N, M>())) step_sync_kernel(const StepArgs a) {
+template <int BASE, int N, int GDT, bool CLIP, int M, int BLOCKS>
+__global__ void __launch_bounds__(kThreads, BLOCKS) step_sync_kernel(const StepArgs a) {
     using S = FusedShape<M>;
     constexpr int R = S::R;
     constexpr int V = S::V;
@@ -281,8 +285,8 @@ __global__ void __launch_bounds__(kThreads, (fused_blocks_per_sm<BASE, N, M>()))
 
 // ---------------------------------------------------------------- launch helpers
 
-template <int BASE, int N, int GDT, bool CLIP, int M>
-cudaError_t launch_step_sync_t(const StepArgs &a, int num_sms, cudaStream_t stream) {
+template <int BASE, int N, int GDT, bool CLIP, int M, int BLOCKS>
+cudaError_t launch_step_sync_b(const StepArgs &a, int num_sms, cudaStream_t stream) {
     // One chunk per warp (stream_grid) where a warp's chunk spans 128
     // elements or more (M <= 4), except for Adam and ADOPT with a single
     // momentum.  Measured on flat 2^27 cases (GB/s, persistent -> one chunk
@@ -292,7 +296,7 @@ cudaError_t launch_step_sync_t(const StepArgs &a, int num_sms, cudaStream_t stre
     // and ADOPT N = 1 6447 -> 6248.  The 64-element chunks of M >= 5 keep
     // the persistent grid (M = 8, ~350M workload: 6504 -> 6409), but for M =
     // 5's SGDM (n = 20M, N = 1, 4: 310 -> 288, 693 -> 666 us).
-    auto kernel = step_sync_kernel<BASE, N, GDT, CLIP, M>;
+    auto kernel = step_sync_kernel<BASE, N, GDT, CLIP, M, BLOCKS>;
     int grid;
     if constexpr (M <= 5 && (BASE == MTDAO_BASE_SGDM || (N >= 2 && M <= 4))) {
         grid = stream_grid(a.n_padded / FusedShape<M>::kChunk);
@@ -304,9 +308,17 @@ cudaError_t launch_step_sync_t(const StepArgs &a, int num_sms, cudaStream_t stre
     return cudaGetLastError();
 }
 
+template <int BASE, int N, int GDT, bool CLIP, int M>
+cudaError_t launch_step_sync_t(const StepArgs &a, int num_sms, cudaStream_t stream) {
+    constexpr int kBlocks = kFusedBlocksPerSm<BASE, N, M>;
+    if (kBlocks > 2 && a.n_padded >= kFusedThreeFrom)
+        return launch_step_sync_b<BASE, N, GDT, CLIP, M, kBlocks>(a, num_sms, stream);
+    return launch_step_sync_b<BASE, N, GDT, CLIP, M, 2>(a, num_sms, stream);
+}
+
 template <int BASE, int N, int GDT, bool CLIP>
 cudaError_t launch_step_sync_m(const StepArgs &a, int num_sms, cudaStream_t st) {
-    const int64_t from = fused_tile_from<BASE, N>(a.M);
+    const int64_t from = fused_tile_from<BASE, N, GDT>(a.M);
     if (from > 0 && a.n_padded >= from) return launch_step_sync_tile<BASE, N, GDT, CLIP>(a, num_sms, st);
     switch (a.M) {
         case 2: return launch_step_sync_t<BASE, N, GDT, CLIP, 2>(a, num_sms, st);

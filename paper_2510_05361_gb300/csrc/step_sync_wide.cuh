@@ -49,7 +49,7 @@ __host__ __device__ constexpr int tile_set_floats(int M, int S) {
 // first (in state index order), so the means read them as one
 // [n_due][M][S] array; a due state's updated values are written back over
 // its own tile, a state that is not due goes straight to HBM.
-template <int BASE, int N, int GDT, bool CLIP>
+template <int BASE, int N, int GDT, bool CLIP, int V>
 __global__ void __launch_bounds__(kTileMaxThreads) step_sync_tile_kernel(const StepArgs a, int log2_p) {
     extern __shared__ __align__(16) float smem[];
     constexpr int kStates = kNumStates<BASE, N>;
@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(kTileMaxThreads) step_sync_tile_kernel(const S
         }
     }
     __syncthreads();
-    tile_means<4>(smem, M, log2_p + 2, n_due * S, mean);
+    tile_means<V>(smem, M, log2_p + 2, n_due * S, mean);
     __syncthreads();
     for (int i = threadIdx.x; i < items; i += static_cast<int>(blockDim.x)) {
         const int f = i & ((1 << log2_p) - 1);
@@ -136,8 +136,13 @@ struct TileShape {
 // Adam N = 3: 6915, 64 columns 5874, 256 5866), else 64 (M = 32: 6864, 128
 // columns 5970; M = 64, SGDM 6730, 128 columns 6541); 32 where two blocks of
 // 64 would not fit an SM (M = 64, Adam N = 4: 5928, 64 columns 4583; M = 100,
-// Adam N = 2: 5998, 16 columns 3711); fewer where the SMs would not have a
-// tile each (M = 256, n = 512, 8 columns 8.2 us, 32 columns 12.3).
+// Adam N = 2: 5998, 16 columns 3711).  Small states, where rows count less (L2)
+// and the SMs are to have tiles enough, take fewer: the half while an SM would
+// get fewer tiles than tile_min of them (us: M = 16, n = 200k, ADOPT N = 3 128
+// columns 27.8, 64 26.6; M = 47, n = 149k, ADOPT N = 2 64 columns 53.1, 32
+// 48.1, 16 48.0; M = 64, n = 60k, Adam N = 2 28.7, 23.0, 23.8; M = 24, n = 500k
+// 72.3, 71.8, 73.4; M = 44, n = 10k, ADOPT N = 3 11.3, 9.3, 8.2; M = 100, n =
+// 4k 32 columns 8.2, 16 6.2, 8 8.2; M = 256, n = 512 32 columns 12.3, 8 8.2).
 // Threads: about 1024 per SM over the blocks that fit, with 2 to 4 items each
 // (M = 48, Adam N = 3: 3 items 6740, 2 items 6169; M = 9: 2 items 6508, 3
 // items 6126, 1 item 4803); two items where that deals them out evenly to 256
@@ -148,7 +153,9 @@ TileShape tile_shape(int M, int64_t n, int num_sms, Bytes bytes) {
     TileShape w;
     w.S = M <= 16 ? 128 : 64;
     while (w.S > 32 && 2 * (bytes(w.S) + kSharedReserved) > kSharedPerSm) w.S /= 2;
-    while (w.S > 8 && (bytes(w.S) + kSharedReserved > kSharedPerSm || n / w.S < num_sms)) w.S /= 2;
+    auto tile_min = [](int S) { return S == 128 ? 11 : S == 64 ? 16 : S == 32 ? 3 : 1; };
+    while (w.S > 8 && (bytes(w.S) + kSharedReserved > kSharedPerSm || n / w.S < int64_t{num_sms} * tile_min(w.S)))
+        w.S /= 2;
     w.smem = bytes(w.S);
     const int items = M * (w.S / 4);
     int64_t resident = (n / w.S + num_sms - 1) / num_sms;        // blocks of an SM
@@ -171,7 +178,13 @@ cudaError_t launch_step_sync_tile(const StepArgs &a, int num_sms, cudaStream_t s
     });
     int log2_p = 0;
     while ((4 << log2_p) < w.S) ++log2_p;
-    auto kernel = step_sync_tile_kernel<BASE, N, GDT, CLIP>;
+    // One column per lane in the means where the block then has a lane for
+    // each chain, four where it has not: the chains of narrow tiles are what
+    // the block waits for (us, four -> one: M = 39, n = 11k 8.2 -> 6.2; M = 66,
+    // n = 10k 10.3 -> 8.2; M = 177, n = 96k 116 -> 110; but M = 47, n = 149k
+    // 48.1 -> 49.1, M = 32, n = 100k 22.6 -> 24.6).
+    auto kernel = 2 * n_due * w.S <= w.threads ? step_sync_tile_kernel<BASE, N, GDT, CLIP, 1>
+                                               : step_sync_tile_kernel<BASE, N, GDT, CLIP, 4>;
     if (const cudaError_t e = allow_shared(kernel, w.smem); e != cudaSuccess) return e;
     kernel<<<static_cast<unsigned>(a.n_padded / w.S), w.threads, w.smem, stream>>>(a, log2_p);
     return cudaGetLastError();
