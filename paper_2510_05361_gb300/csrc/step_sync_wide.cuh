@@ -142,7 +142,8 @@ struct TileShape {
 // columns 27.8, 64 26.6; M = 47, n = 149k, ADOPT N = 2 64 columns 53.1, 32
 // 48.1, 16 48.0; M = 64, n = 60k, Adam N = 2 28.7, 23.0, 23.8; M = 24, n = 500k
 // 72.3, 71.8, 73.4; M = 44, n = 10k, ADOPT N = 3 11.3, 9.3, 8.2; M = 100, n =
-// 4k 32 columns 8.2, 16 6.2, 8 8.2; M = 256, n = 512 32 columns 12.3, 8 8.2).
+// 4k 32 columns 8.2, 16 6.2, 8 8.2; M = 256, n = 512 32 columns 12.3, 8 8.2;
+// M = 11, n = 111k, SGDM N = 4 128 columns 8.3, 32 11.8).
 // Threads: about 1024 per SM over the blocks that fit, with 2 to 4 items each
 // (M = 48, Adam N = 3: 3 items 6740, 2 items 6169; M = 9: 2 items 6508, 3
 // items 6126, 1 item 4803); two items where that deals them out evenly to 256
@@ -153,7 +154,10 @@ TileShape tile_shape(int M, int64_t n, int num_sms, Bytes bytes) {
     TileShape w;
     w.S = M <= 16 ? 128 : 64;
     while (w.S > 32 && 2 * (bytes(w.S) + kSharedReserved) > kSharedPerSm) w.S /= 2;
-    auto tile_min = [](int S) { return S == 128 ? 11 : S == 64 ? 16 : S == 32 ? 3 : 1; };
+    auto tile_min = [&](int S) {
+        if (M * (S / 8) >= 256 && S >= 64) return S == 128 ? 11 : 16;      // the half still has items enough
+        return S >= 32 ? 3 : 1;
+    };
     while (w.S > 8 && (bytes(w.S) + kSharedReserved > kSharedPerSm || n / w.S < int64_t{num_sms} * tile_min(w.S)))
         w.S /= 2;
     w.smem = bytes(w.S);
