@@ -191,6 +191,39 @@ __global__ void __launch_bounds__(kThreads) step_kernel(const StepArgs a) {
     }
 }
 
+// The step on states so small that every warp runs at once: a warp's time is
+// then that of its loads one after another, so all states' loads go out before
+// any arithmetic, on four elements a lane and blocks of two warps that spread
+// over the SMs.  Back to back (from Python, host-bound below 4.8 us), step_kernel
+// -> this: Adam N = 2, M = 4, n = 5k 6.1 -> 5.0 us; ADOPT N = 4, n = 20k 6.2 ->
+// 4.8; Adam N = 3, n = 60k 6.1 -> 4.9; n = 200k (41 warps an SM) 6.2 -> 6.0.
+constexpr int kSmallThreads = 64;
+constexpr int64_t kSmallWarps = 64;      // warps an SM takes at once
+constexpr int kSmallChunk = 128;         // elements of one warp
+
+template <int BASE, int N, int GDT, bool CLIP>
+__global__ void __launch_bounds__(kSmallThreads) step_small_kernel(const StepArgs a) {
+    constexpr int kStates = kNumStates<BASE, N>;
+    const int64_t chunk = (static_cast<int64_t>(blockIdx.x) * kSmallThreads + threadIdx.x) >> 5;
+    if (chunk * kSmallChunk >= a.stride) return;
+    const int64_t e = chunk * kSmallChunk + 4 * (threadIdx.x & 31);
+    float g[4], cur[kStates][4], gt[4], acc[4];
+    to_array(ld_grad<GDT>(a.grads, e), g);
+#pragma unroll
+    for (int st = 0; st < kStates; ++st) to_array(ld_state(a.arena + st * a.stride + e), cur[st]);
+    float s = 1.0f;
+    if constexpr (CLIP) s = __ldg(a.clip_scale + (chunk * kSmallChunk) / a.n_padded);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) acc[k] = step_acc_init<BASE>(a.sc, g[k], s);
+#pragma unroll
+    for (int i = 0; i < kStates; ++i) {
+        const int st = state_order<BASE, N>(i);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) update_state<BASE, N>(a.sc, st, g[k], s, gt[k], acc[k], cur[st][k]);
+        st_state(a.arena + st * a.stride + e, from_array(cur[st]));
+    }
+}
+
 // ---------------------------------------------------------------- launch helpers
 
 // Persistent grid: as many blocks as fit on the device at once, but never
@@ -228,8 +261,13 @@ inline int stream_grid(int64_t n_warp_items) {
 
 template <int BASE, int N, int GDT, bool CLIP>
 cudaError_t launch_step_t(const StepArgs &a, int num_sms, cudaStream_t stream) {
+    if (a.stride <= kSmallWarps * num_sms * kSmallChunk) {
+        const int64_t threads = a.stride / kSmallChunk * 32;
+        step_small_kernel<BASE, N, GDT, CLIP>
+            <<<static_cast<unsigned>((threads + kSmallThreads - 1) / kSmallThreads), kSmallThreads, 0, stream>>>(a);
+        return cudaGetLastError();
+    }
     auto kernel = step_kernel<BASE, N, GDT, CLIP>;
-    (void)num_sms;
     const int grid = stream_grid(a.stride / kChunk);
     kernel<<<grid, kThreads, 0, stream>>>(a);
     return cudaGetLastError();

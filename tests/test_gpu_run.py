@@ -139,3 +139,32 @@ def test_run_stops_at_a_bad_rate(P):
     _same(a, b)                                    # t counts the steps done
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("base,N,gdt,clip", [(base, N, gdt, clip) for base in ("adam", "adopt", "sgdm") for N in (1, 2, 3, 4)
+                                             for gdt in ("f32", "bf16") for clip in (False, True)
+                                             if not (clip and base == "adopt")])
+def test_small_and_large_steps_agree(P, base, N, gdt, clip):
+    """Workers together take the step kernel of large states, each of them alone
+    that of small ones (up to 64 warps of 128 elements per SM)."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    most = 64 * 128 * sms
+    M, numel = 3, most // 2
+    w = workload_dict([numel], M, base=base, betas=(0.9, 0.999, 0.5, 0.99)[:N], px=0, pu=[0] * N, pv=0,
+                      clip="global_norm" if clip else "none", rho=0.05, gdt=gdt)
+    (a, _), g = _pair(P, w, M, gdt, 1, seed=N)
+    _.close()
+    assert a.n_padded <= most < M * a.n_padded
+    small = []
+    for m in range(M):
+        e = P.MTDAO(w["opt"], 1, w["shapes"])
+        for s in range(a.n_states):
+            e.state_view(s).copy_(a.state_view(s)[m:m + 1])
+        e.step(g[0, m:m + 1], 1e-3)
+        small.append(e)
+    a.step(g[0], 1e-3)
+    for s in range(a.n_states):
+        for m in range(M):
+            assert torch.equal(a.state_view(s)[m], small[m].state_view(s)[0]), (s, m)
+    for e in small + [a]:
+        e.close()
