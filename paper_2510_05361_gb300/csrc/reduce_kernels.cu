@@ -67,9 +67,10 @@ constexpr int kSyncTileThreads = 128;
 // replica; the blocks start in index order.  Takes M > 14, where a thread
 // that streams the replicas of its position (four loads in flight, persistent
 // grid) has one long chain of loads behind its sums.  That one -> this, us:
-// M = 16, n = 8M, one state 179 -> 152; M = 32, n = 5M, 3 states 620 -> 552
-// (6.96 TB/s); M = 64, n = 2M 504 -> 448; M = 256, n = 400k 423 -> 366; M =
-// 1024, n = 100k, 2 states 520 -> 378; M = 256, n = 1000 65.5 -> 6.2.  Bound by
+// M = 16, n = 8M, one state 179 -> 152, n = 20k 8.2 -> 4.1; M = 32, n = 5M, 3
+// states 620 -> 552 (6.96 TB/s), n = 200k 14.4 -> 8.2; M = 64, n = 2M 504 ->
+// 448; M = 256, n = 400k 423 -> 366; M = 1024, n = 100k, 2 states 520 -> 378; M
+// = 256, n = 1000 65.5 -> 6.2.  Bound by
 // HBM; above M = 256 by the tiles of 16 to 32 columns (64 to 128 bytes a row)
 // that two of them fit on an SM with.
 template <int V>
@@ -86,7 +87,7 @@ __global__ void __launch_bounds__(kSyncTileThreads) sync_tile_kernel(const __gri
     cp_async_commit();
     cp_async_wait<0>();
     __syncthreads();
-    tile_means<V>(smem, M, log2_p + 2, S, mean);
+    tile_means<V>(smem, M, log2_p + 2, mean);
     __syncthreads();
     for (int i = threadIdx.x; i < items; i += static_cast<int>(blockDim.x)) {
         const int f = i & ((1 << log2_p) - 1);
@@ -109,8 +110,7 @@ cudaError_t launch_sync_tile(const SyncArgs &a, int num_sms, cudaStream_t stream
                           (a.n_padded >> (log2_p + 2)) * a.n_sel < num_sms))
         --log2_p;
     const size_t smem = bytes(log2_p);
-    // one column per lane in the means above M = 32 (M = 256: 366 us, four 401)
-    auto kernel = a.M <= 32 ? sync_tile_kernel<4> : sync_tile_kernel<1>;
+    auto kernel = a.M < kSplitMeansM ? sync_tile_kernel<1> : sync_tile_kernel<0>;
     if (const cudaError_t e = allow_shared(kernel, smem); e != cudaSuccess) return e;
     const int64_t gx = a.n_padded >> (log2_p + 2);
     if (gx > 0x7fffffff) return cudaErrorInvalidValue;

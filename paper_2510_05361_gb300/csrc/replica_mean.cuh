@@ -32,6 +32,7 @@ namespace mtdao {
 struct DiffSum {
     float s0, sum, comp;
 
+    DiffSum() = default;
     __device__ __forceinline__ explicit DiffSum(float ref) : s0(ref), sum(0.0f), comp(0.0f) {}
 
     __device__ __forceinline__ void add(float sm) {

@@ -29,64 +29,104 @@ __device__ __forceinline__ void ld_shared_v(const float *p, float (&v)[V]) {
     }
 }
 
-// Replica means of the n_cols columns of a block's tiles into mean[p]
-// (column p: tile + (p / S) * M * S + p % S, the replicas at stride
-// S = 2^log2_s).  Columns go in groups of V; lanes i and i + 16 of a warp
-// take one group and form its two compensated parts of replica_mean.cuh,
-// replicas 1 .. h-1 and h .. M-1 in order (h = M / 2), and join them with a
-// shuffle: the bits of replica_mean_rt (with its plain mean where the
-// compensated one is NaN).  A half-warp reads one row, so no two of its
-// lanes meet in a bank.  Every thread of the block calls it (the shuffles
-// take whole warps: blockDim.x is a multiple of 32).
-template <int V>
-__device__ __forceinline__ void tile_means(const float *tile, int M, int log2_s, int n_cols, float *mean) {
-    const int h = M / 2;
+// Replica means of the n_cols columns of a block's tiles into mean[p], column
+// p = k * S + c being column c of the k-th tile: tile_of(k) is where that tile
+// [M][S] begins; the bits of replica_mean.cuh (with its plain mean where the
+// compensated one is NaN).
+//
+// V > 0: a lane takes V neighbouring columns and runs both compensated parts
+// over the replicas in order (1 .. h-1 and h .. M-1, h = M / 2), one replica of
+// each part a step, so that the two chains overlap.  Against a pair of lanes
+// per four columns (a part each, joined by shuffles; most of the fused step's
+// time above HBM's was its instructions: 52 of 177 an element at M = 8), fused
+// step, us, pair -> here with V = 1 (V = 4): M = 8, n = 20M, ADOPT N = 2, bf16
+// 832 -> 785 (793), Adam N = 3 1051 -> 1014 (1010); M = 9, n = 2^23 511 -> 483
+// (483); M = 16, ADOPT 686 -> 659 (671); M = 12 529 -> 511 (496); M = 64, n = 1M
+// 346 -> 326 (439).  (Half of it is the item loops of step_sync_wide.cuh.)
+// V = 0: a pair of half-warps takes a column a lane, one part each, joined by a
+// shuffle: twice the lanes on chains that are long and tiles that are narrow
+// (average, M = 256, n = 400k 370 -> 367 us, n = 1000 8.0 -> 6.2, M = 1024, n =
+// 100k 452 -> 378; fused, M = 100 359 -> 353).  kSplitMeansM: M from which.
+constexpr int kSplitMeansM = 65;
+
+template <int V, typename TileOf>
+__device__ __forceinline__ void tile_means(TileOf tile_of, int M, int log2_s, int n_cols, float *mean) {
     const int S = 1 << log2_s;
-    const int part = (threadIdx.x >> 4) & 1;
-    const int first = V * ((threadIdx.x >> 5) * 16 + (threadIdx.x & 15));
-    const int lo = part ? (h > 1 ? h : 1) : 1, hi = part ? M : h;
-    for (int p0 = 0; p0 < n_cols; p0 += V * static_cast<int>(blockDim.x >> 1)) {
-        if (p0 + V * 16 * static_cast<int>(threadIdx.x >> 5) >= n_cols) break;      // the whole warp is past the end
-        const int p = p0 + first;
-        const float *base = tile + (p >> log2_s) * M * S + (p & (S - 1));
-        float s0[V], mine[V], other[V];
-#pragma unroll
-        for (int k = 0; k < V; ++k) s0[k] = mine[k] = 0.0f;
-        if (p < n_cols) {
-            ld_shared_v<V>(base, s0);
-            float sum[V], comp[V];
-#pragma unroll
-            for (int k = 0; k < V; ++k) sum[k] = comp[k] = 0.0f;
+    const int h = M / 2;
+    const float fM = static_cast<float>(M);
+    auto column = [&](int p) { return tile_of(p >> log2_s) + (p & (S - 1)); };
+    if constexpr (V == 0) {
+        const int part = (threadIdx.x >> 4) & 1;
+        const int lo = part ? (h > 1 ? h : 1) : 1, hi = part ? M : h;
+        // every lane of a warp with a column left goes round (the shuffle)
+        for (int p0 = static_cast<int>(threadIdx.x >> 5) * 16; p0 < n_cols; p0 += static_cast<int>(blockDim.x >> 1)) {
+            const int p = p0 + static_cast<int>(threadIdx.x & 15);
+            const float *base = column(p < n_cols ? p : n_cols - 1);
+            const float s0 = *base;
+            DiffSum sum(s0);
 #pragma unroll 4
-            for (int m = lo; m < hi; ++m) {
-                float v[V];
+            for (int m = lo; m < hi; ++m) sum.add(base[m * S]);
+            const float mine = sum.partial();
+            const float other = __shfl_xor_sync(0xffffffffu, mine, 16);
+            if (p < n_cols && part == 0) {
+                float v = replica_mean_from_parts(s0, mine, other, fM);
+                if (v != v) {                    // non-finite values: the plain mean
+                    float plain = s0;
+                    for (int m = 1; m < M; ++m) plain += base[m * S];
+                    v = plain / fM;
+                }
+                mean[p] = v;
+            }
+        }
+    } else {
+        for (int p = V * static_cast<int>(threadIdx.x); p < n_cols; p += V * static_cast<int>(blockDim.x)) {
+            const float *base = column(p);
+            float s0[V], v[V], w[V];
+            ld_shared_v<V>(base, s0);
+            DiffSum pa[V], pb[V];
+#pragma unroll
+            for (int k = 0; k < V; ++k) pa[k] = pb[k] = DiffSum(s0[k]);
+            const float *at = base + S;              // replica 1 + j of part A, h + j of part B
+            const int to_b = (h - 1) * S;
+#pragma unroll 2
+            for (int j = 1; j < h; ++j, at += S) {
+                ld_shared_v<V>(at, v);
+                ld_shared_v<V>(at + to_b, w);
+#pragma unroll
+                for (int k = 0; k < V; ++k) {
+                    pa[k].add(v[k]);
+                    pb[k].add(w[k]);
+                }
+            }
+            for (int m = h > 1 ? 2 * h - 1 : 1; m < M; ++m) {        // part B's last one or two
                 ld_shared_v<V>(base + m * S, v);
 #pragma unroll
-                for (int k = 0; k < V; ++k) {            // DiffSum::add
-                    const float y = (v[k] - s0[k]) - comp[k];
-                    const float t = sum[k] + y;
-                    comp[k] = (t - sum[k]) - y;
-                    sum[k] = t;
-                }
+                for (int k = 0; k < V; ++k) pb[k].add(v[k]);
             }
-#pragma unroll
-            for (int k = 0; k < V; ++k) mine[k] = sum[k] - comp[k];
-        }
-#pragma unroll
-        for (int k = 0; k < V; ++k) other[k] = __shfl_xor_sync(0xffffffffu, mine[k], 16);
-        if (p < n_cols && part == 0) {
+            bool nan = false;
 #pragma unroll
             for (int k = 0; k < V; ++k) {
-                float v = replica_mean_from_parts(s0[k], mine[k], other[k], static_cast<float>(M));
-                if (v != v) {                    // non-finite values: the plain mean (replica_mean.cuh)
+                v[k] = replica_mean_from_parts(s0[k], pa[k].partial(), pb[k].partial(), fM);
+                nan = nan || v[k] != v[k];
+            }
+            if (nan) {                               // non-finite values: the plain mean (replica_mean.cuh)
+#pragma unroll
+                for (int k = 0; k < V; ++k) {
                     float plain = s0[k];
                     for (int m = 1; m < M; ++m) plain += base[m * S + k];
-                    v = plain / static_cast<float>(M);
+                    v[k] = mean_or_plain(v[k], plain, fM);
                 }
-                mean[p + k] = v;
             }
+#pragma unroll
+            for (int k = 0; k < V; ++k) mean[p + k] = v[k];
         }
     }
+}
+
+// The means of one tile.
+template <int V>
+__device__ __forceinline__ void tile_means(const float *tile, int M, int log2_s, float *mean) {
+    tile_means<V>([=](int) { return tile; }, M, log2_s, 1 << log2_s, mean);
 }
 
 // 16- and 8-byte asynchronous global -> shared copies (cp.async) and their

@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(kStatsTileThreads) stats_tile_kernel(const __g
         cp_async_commit();
         cp_async_wait<0>();                      // this thread's copies have landed
         __syncthreads();                         // ... and every thread's
-        tile_means<V>(tile, M, a.log2_s, S, mean);
+        tile_means<V>(tile, M, a.log2_s, mean);
         __syncthreads();
 #pragma unroll
         for (int j = 0; j < R; ++j) {
@@ -180,14 +180,13 @@ struct StatsTileShape {
 // round's end -- change of x, then the average of every state with its sums --
 // in us; the previous kernels, one-pass in rows of 128 to 256 bytes with
 // persistent blocks up to M = 64 and two passes above, first).
-//   Columns: 256 up to M = 12 (M = 9, Adam N = 1, n = 8M: 534 -> 500; 128
-//   columns 511), 128 up to 16 (M = 16, Adam N = 2, n = 8M: 942 -> 806; 64
-//   columns 835), else 64 (M = 32, n = 4M: 781 -> 646; M = 64, n = 2M: 709 ->
-//   639; M = 128, n = 600k: 1102 -> 496; M = 256, n = 400k: 1073 -> 598), fewer
+//   Columns: 256 up to M = 12 (M = 9, Adam N = 1, n = 8M: 534 -> 380), 128 up
+//   to 16 (M = 16, Adam N = 2, n = 8M: 942 -> 747), else 64 (M = 32, n = 4M: 781
+//   -> 607; M = 64, n = 2M: 709 -> 616; M = 128, n = 600k: 1102 -> 496; M = 256, n = 400k: 1073 -> 598), fewer
 //   where two tiles would not fit an SM or the SMs would not have one each.
 //   Lanes and threads: the fewer, the more rows a thread takes and the less
-//   there is to combine at a run's end (M = 64: 2 lanes and 128 threads 639, 8
-//   lanes 683, 512 threads 1120).
+//   there is to combine at a run's end (M = 64, means by lane pairs: 2 lanes and
+//   128 threads 639, 8 lanes 683, 512 threads 1120).
 //   Tiles: runs enough for 8 blocks an SM, 8 at most, so that the tiles under
 //   way lie close together (M = 64: 640, runs of 32 675; M = 100, n = 75k, runs
 //   of 1 to 2: 231 -> 56, of 32 254); as many columns where the tiles are
@@ -232,15 +231,16 @@ cudaError_t launch_stats_tile(StatsTileArgs &a, int n_sel, int num_sms, size_t p
     a.log2_l = w.log2_l;
     a.tiles = w.tiles;
     cudaError_t e;
-    // columns of a lane in the means: the fewer warps a block has, the more
+    // R = 1 is M <= 64 (tile_means: M = 9 380 us with two columns a lane, 402
+    // with one, 392 with four; M = 64 616 with one, 651 with two)
     switch (w.R) {
         case 1:
-            e = a.M <= 16 ? launch_stats_tile_t<CHANGE, 1, 4>(a, w, n_sel, stream)
-                          : launch_stats_tile_t<CHANGE, 1, 2>(a, w, n_sel, stream);
+            e = a.M <= 16 ? launch_stats_tile_t<CHANGE, 1, 2>(a, w, n_sel, stream)
+                          : launch_stats_tile_t<CHANGE, 1, 1>(a, w, n_sel, stream);
             break;
-        case 2: e = launch_stats_tile_t<CHANGE, 2, 1>(a, w, n_sel, stream); break;
-        case 4: e = launch_stats_tile_t<CHANGE, 4, 1>(a, w, n_sel, stream); break;
-        default: e = launch_stats_tile_t<CHANGE, 8, 1>(a, w, n_sel, stream); break;
+        case 2: e = launch_stats_tile_t<CHANGE, 2, 0>(a, w, n_sel, stream); break;
+        case 4: e = launch_stats_tile_t<CHANGE, 4, 0>(a, w, n_sel, stream); break;
+        default: e = launch_stats_tile_t<CHANGE, 8, 0>(a, w, n_sel, stream); break;
     }
     if (e != cudaSuccess) return e;
     return launch_stats_finalize(a.partial, w.runs, Q, n_sel, CHANGE ? 0 : a.M, stats, stream);

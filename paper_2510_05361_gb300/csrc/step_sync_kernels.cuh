@@ -143,33 +143,33 @@ __device__ __forceinline__ void load_replicas(const float *state, int64_t n_padd
 // (80) where that ran faster on flat 20M vectors with every state due (us, two
 // -> three): M = 5 Adam N = 1 to 4 500 -> 428, 604 -> 552, 754 -> 680, 865 ->
 // 835, ADOPT 499 -> 437, 621 -> 551, 879 -> 822, bf16 ADOPT N = 3 770 -> 651;
-// M = 6 ADOPT N = 1 to 3 569 -> 527, 709 -> 681, 877 -> 814 (N = 4 1008 -> 1050,
-// Adam N = 3 874 -> 894); M = 4 Adam N = 3 783 -> 820, M = 7 Adam N = 2 785 -> 925.
+// M = 6 ADOPT N = 1, 2 569 -> 527, 709 -> 681 (N = 4 1008 -> 1050, Adam N = 3
+// 874 -> 894); M = 4 Adam N = 3 783 -> 820, M = 7 Adam N = 2 785 -> 925.
 // Below kFusedThreeFrom elements the SMs have no third block to take (M = 5,
 // ADOPT N = 4, n = 20k, where 80 registers spill: 8.5 us with two, 10.3).
 template <int BASE, int N, int M>
-constexpr int kFusedBlocksPerSm = M == 5 || (M == 6 && BASE == MTDAO_BASE_ADOPT && N <= 3) ? 3 : 2;
+constexpr int kFusedBlocksPerSm = M == 5 || (M == 6 && BASE == MTDAO_BASE_ADOPT && N <= 2) ? 3 : 2;
 constexpr int64_t kFusedThreeFrom = int64_t{1} << 16;
 
 // Smallest n that the tiled kernel of step_sync_wide.cuh takes for M = 6, 7
-// and 8 (0: none); us here -> tiled, every state due.
-//   n = 4M, M = 6: Adam N = 2, 3 149 -> 152, 187 -> 174, SGDM 79 -> 78; M = 7:
-//   Adam 141 -> 137, SGDM N = 2 124 -> 121, ADOPT N = 4 251 -> 246.
-//   M = 8: n = 200k (in L2) 12.0 -> 16.4, 1M (Adam N = 3) 60 -> 63, 2M (ADOPT,
-//   bf16) 98 -> 100, 4M (bf16) 224 -> 215, 20M 3 to 7 % faster (Adam, ADOPT,
-//   SGDM, N = 1 to 4) but for ADOPT's N = 3 and 4 with f32 gradients (n = 5M
-//   298 -> 308, 348 -> 354, 20M 1086 -> 1110, 1282 -> 1276; bf16 353 -> 352).
-//   n = 20M, M = 6: Adam N = 1 to 4 570 -> 529, 690 -> 691, 874 -> 799, 989 ->
-//   923, SGDM N = 1, 2, 4 363 -> 344, 506 -> 453, 814 -> 767, ADOPT N = 4 1008
-//   -> 964 (N = 2 681 -> 737); M = 7: Adam N = 1, 3, 4 639 -> 621, 984 -> 982,
-//   1138 -> 1078 (N = 2 785 -> 798), SGDM 429 -> 401, 566 -> 547, 938 -> 904,
-//   ADOPT N = 3, 4 1004 -> 964, 1181 -> 1136 (N = 2 801 -> 853).
+// and 8 (0: none).  us here -> tiled, every state due, flat vectors:
+//   M = 8, n = 20M: Adam N = 1 to 4 695 -> 643, 877 -> 832, 1070 -> 1015, 1272
+//   -> 1201, ADOPT 701 -> 648, 882 -> 846, 1084 -> 1023, 1285 -> 1228, SGDM N =
+//   1, 4 497 -> 455, 1085 -> 1012; n = 2M Adam N = 2 95 -> 91, N = 4 133 -> 131;
+//   n = 1M 51 -> 49, 69 -> 71; n = 400k (in L2) 18 -> 21.
+//   M = 7, n = 20M: Adam 639 -> 568, 785 -> 736, 984 -> 891, 1140 -> 1053, ADOPT
+//   641 -> 605, 800 -> 783, 995 -> 909, 1181 -> 1085, SGDM 432 -> 400; n = 2M 86
+//   -> 84, 121 -> 116; n = 1M 47 -> 47; n = 400k 18 -> 21.
+//   M = 6, n = 20M: Adam 571 -> 514, 689 -> 687 (bf16 680 -> 659), 873 -> 794,
+//   989 -> 948, SGDM N = 1, 2, 4 363 -> 343, 506 -> 451, 814 -> 769, ADOPT N =
+//   3, 4 847 -> 830, 1007 -> 994 (N = 1, 2 529 -> 549, 680 -> 739); n = 4M Adam
+//   N = 2, 4 149 -> 152, 210 -> 207; n = 2M 76 -> 80, 107 -> 106.
+// M = 5 stays here (n = 20M, Adam N = 2 554 -> 600, ADOPT 552 -> 649), M = 4 too
+// (Adam N = 3 524 -> 598).
 template <int BASE, int N, int GDT>
 constexpr int64_t fused_tile_from(int M) {
-    constexpr bool adopt = BASE == MTDAO_BASE_ADOPT, adam = BASE == MTDAO_BASE_ADAM;
-    const bool faster = (M == 8 && !(adopt && N >= 3 && GDT == MTDAO_F32)) ||
-                        ((M == 6 || M == 7) && (adopt ? N >= 10 - M : !(adam && N == 2)));
-    return faster ? int64_t{1} << 22 : 0;
+    constexpr bool not6 = BASE == MTDAO_BASE_ADOPT ? N <= 2 : BASE == MTDAO_BASE_ADAM && N == 2 && GDT == MTDAO_F32;
+    return M >= 7 ? int64_t{1} << 21 : (M == 6 && !not6) ? int64_t{1} << 22 : 0;
 }
 
 template <int BASE, int N, int GDT, bool CLIP, int M, int BLOCKS>

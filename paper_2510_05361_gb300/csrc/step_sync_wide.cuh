@@ -7,20 +7,18 @@
 // Its threads update the tile with update_state; a state that is not due is
 // stored from registers, a due state's new values go back over its tile.
 // After one barrier the replica mean of every (due state, column) pair is
-// formed by two threads, each running one of the two compensated parts of
-// replica_mean.cuh over the replicas in order; after a second barrier the
-// means are stored to every replica.  The parts are the ones the standalone
-// average forms, in the same order, so fused and separate averaging give
-// identical bits for every M.
+// formed (tile_means of replica_tile.cuh: the standalone average's sums in the
+// same order, so fused and separate averaging give identical bits for every
+// M); after a second barrier the means are stored to every replica.
 //
 // One tile per block, the blocks started in index order as earlier ones
 // retire; what overlaps the copies of one block is the work of the others on
 // its SM.  Against persistent blocks that copied their next span (of half
 // the columns, for the same shared memory) while they worked on the current
-// one: M = 16, n = 2^23, Adam N = 3, f32 5872 -> 6879 GB/s; M = 32 5706 ->
-// 6850; M = 64, n = 1.9M, SGDM, bf16 4683 -> 6720; M = 100, n = 600k, Adam
-// N = 2 (step and average apart before) 3423 -> 5890, M = 256 3406 -> 3871,
-// SGDM 3384 -> 5010; M = 256, n = 512 63.5 -> 8.2 us.  Both halves count: a
+// one: M = 16, n = 2^23, Adam N = 3, f32 5872 -> 6970 GB/s; M = 32 5706 ->
+// 6850; M = 64, n = 1.9M, SGDM, bf16 4683 -> 6740; M = 100, n = 600k, Adam
+// N = 2 (step and average apart before) 3423 -> 6120, M = 256 3406 -> 3871,
+// SGDM 3384 -> 5340; M = 256, n = 512 63.5 -> 8.2 us.  Both halves count: a
 // plain copy of such tiles runs at 6.7-6.9 TB/s with rows of 256 bytes or
 // more in index order, 6.1-6.3 persistent, and 5.5-5.9 / 5.1-5.3 with rows of
 // 128 bytes.  Bound by HBM up to M = 64; above, by the two or three blocks
@@ -42,13 +40,18 @@ __host__ __device__ constexpr int tile_set_floats(int M, int S) {
     return kNumStates<BASE, N> * M * S + (GDT == MTDAO_F32 ? M * S : M * S / 2);
 }
 
+// Index of the k-th set bit of mask (k counts from 0 and is in range).
+__device__ __forceinline__ int nth_set_bit(uint32_t mask, int k) {
+    for (; k > 0; --k) mask &= mask - 1u;
+    return __ffs(static_cast<int>(mask)) - 1;
+}
+
 // The fused step on one tile of S = 4 * 2^log2_p columns of all replicas per
 // block.  Item i of the tile is float4 position i % 2^log2_p of replica
-// i / 2^log2_p; a thread copies, updates and stores the same items, so the
-// only barriers are those around the means.  The due states' tiles come
-// first (in state index order), so the means read them as one
-// [n_due][M][S] array; a due state's updated values are written back over
-// its own tile, a state that is not due goes straight to HBM.
+// i / 2^log2_p; a thread copies, updates and stores the same items (always the
+// same position, as 2^log2_p divides the block), so the only barriers are those
+// around the means.  A due state's updated values are written back over its
+// own tile, a state that is not due goes straight to HBM.
 template <int BASE, int N, int GDT, bool CLIP, int V>
 __global__ void __launch_bounds__(kTileMaxThreads) step_sync_tile_kernel(const StepArgs a, int log2_p) {
     extern __shared__ __align__(16) float smem[];
@@ -56,72 +59,79 @@ __global__ void __launch_bounds__(kTileMaxThreads) step_sync_tile_kernel(const S
     const int M = a.M;
     const int S = 4 << log2_p;
     const int tile = M * S;
-    const int items = M << log2_p;
     const int64_t n = a.n_padded;
-    const int64_t col0 = static_cast<int64_t>(blockIdx.x) * S;
+    const int64_t stride = a.stride;
     const uint32_t mask = a.sync_mask;
-    const int n_due = __popc(mask);
     float *mean = smem + tile_set_floats<BASE, N, GDT>(M, S);   // [n_due][S]
-    // tile of state st: the due states first
-    auto slot = [&](int st) {
-        const uint32_t below = (1u << st) - 1u;
-        return ((mask >> st) & 1u) ? __popc(mask & below) : n_due + __popc(~mask & below);
-    };
 
-    for (int i = threadIdx.x; i < items; i += static_cast<int>(blockDim.x)) {
-        const int64_t src = (i >> log2_p) * n + col0 + 4 * (i & ((1 << log2_p) - 1));
+    // The thread's items: replicas r, r + rows, ...; e: the element of item r.
+    const int f = static_cast<int>(threadIdx.x) & ((1 << log2_p) - 1);
+    const int r0 = static_cast<int>(threadIdx.x) >> log2_p;
+    const int rows = static_cast<int>(blockDim.x) >> log2_p;
+    const int64_t e0 = r0 * n + static_cast<int64_t>(blockIdx.x) * S + 4 * f;
+    const int64_t e_step = rows * n;
+    const int at0 = r0 * S + 4 * f, at_step = rows * S;          // in a tile
+
+    {
+        int64_t e = e0;
+        int at = at0;
+        for (int r = r0; r < M; r += rows, e += e_step, at += at_step) {
 #pragma unroll
-        for (int st = 0; st < kStates; ++st) cp_async16(smem + slot(st) * tile + 4 * i, a.arena + st * a.stride + src);
-        if constexpr (GDT == MTDAO_F32)
-            cp_async16(smem + kStates * tile + 4 * i, static_cast<const float *>(a.grads) + src);
-        else
-            cp_async8(reinterpret_cast<uint16_t *>(smem + kStates * tile) + 4 * i,
-                      static_cast<const uint16_t *>(a.grads) + src);
+            for (int st = 0; st < kStates; ++st) cp_async16(smem + st * tile + at, a.arena + st * stride + e);
+            if constexpr (GDT == MTDAO_F32)
+                cp_async16(smem + kStates * tile + at, static_cast<const float *>(a.grads) + e);
+            else
+                cp_async8(reinterpret_cast<uint16_t *>(smem + kStates * tile) + at,
+                          static_cast<const uint16_t *>(a.grads) + e);
+        }
     }
     cp_async_commit();
     cp_async_wait<0>();                          // a thread reads what it copied itself
 
-    for (int i = threadIdx.x; i < items; i += static_cast<int>(blockDim.x)) {
-        const int r = i >> log2_p;
-        const int64_t e = r * n + col0 + 4 * (i & ((1 << log2_p) - 1));
-        const float s = CLIP ? __ldg(a.clip_scale + r) : 1.0f;
-        float g[4], gt[4], acc[4];
-        if constexpr (GDT == MTDAO_F32) {
-            to_array(*reinterpret_cast<const float4 *>(smem + kStates * tile + 4 * i), g);
-        } else {
-            const uint2 w =
-                *reinterpret_cast<const uint2 *>(reinterpret_cast<const uint16_t *>(smem + kStates * tile) + 4 * i);
-            g[0] = __uint_as_float(w.x << 16);
-            g[1] = __uint_as_float(w.x & 0xffff0000u);
-            g[2] = __uint_as_float(w.y << 16);
-            g[3] = __uint_as_float(w.y & 0xffff0000u);
-        }
+    {
+        int64_t e = e0;
+        int at = at0;
+        for (int r = r0; r < M; r += rows, e += e_step, at += at_step) {
+            const float s = CLIP ? __ldg(a.clip_scale + r) : 1.0f;
+            float g[4], gt[4], acc[4];
+            if constexpr (GDT == MTDAO_F32) {
+                to_array(*reinterpret_cast<const float4 *>(smem + kStates * tile + at), g);
+            } else {
+                const uint2 w =
+                    *reinterpret_cast<const uint2 *>(reinterpret_cast<const uint16_t *>(smem + kStates * tile) + at);
+                g[0] = __uint_as_float(w.x << 16);
+                g[1] = __uint_as_float(w.x & 0xffff0000u);
+                g[2] = __uint_as_float(w.y << 16);
+                g[3] = __uint_as_float(w.y & 0xffff0000u);
+            }
 #pragma unroll
-        for (int k = 0; k < 4; ++k) acc[k] = step_acc_init<BASE>(a.sc, g[k], s);
+            for (int k = 0; k < 4; ++k) acc[k] = step_acc_init<BASE>(a.sc, g[k], s);
 #pragma unroll
-        for (int o = 0; o < kStates; ++o) {
-            const int st = state_order<BASE, N>(o);
-            float *cell = smem + slot(st) * tile + 4 * i;
-            float cur[4];
-            to_array(*reinterpret_cast<const float4 *>(cell), cur);
+            for (int o = 0; o < kStates; ++o) {
+                const int st = state_order<BASE, N>(o);
+                float *cell = smem + st * tile + at;
+                float cur[4];
+                to_array(*reinterpret_cast<const float4 *>(cell), cur);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) update_state<BASE, N>(a.sc, st, g[k], s, gt[k], acc[k], cur[k]);
-            if ((mask >> st) & 1u)
-                *reinterpret_cast<float4 *>(cell) = from_array(cur);
-            else
-                st_state(a.arena + st * a.stride + e, from_array(cur));
+                for (int k = 0; k < 4; ++k) update_state<BASE, N>(a.sc, st, g[k], s, gt[k], acc[k], cur[k]);
+                if ((mask >> st) & 1u)
+                    *reinterpret_cast<float4 *>(cell) = from_array(cur);
+                else
+                    st_state(a.arena + st * stride + e, from_array(cur));
+            }
         }
     }
     __syncthreads();
-    tile_means<V>(smem, M, log2_p + 2, n_due * S, mean);
+    tile_means<V>([=](int k) { return smem + nth_set_bit(mask, k) * tile; }, M, log2_p + 2, __popc(mask) * S, mean);
     __syncthreads();
-    for (int i = threadIdx.x; i < items; i += static_cast<int>(blockDim.x)) {
-        const int f = i & ((1 << log2_p) - 1);
-        const int64_t e = (i >> log2_p) * n + col0 + 4 * f;
+    const float *from = mean + 4 * f;
 #pragma unroll
-        for (int st = 0; st < kStates; ++st)
-            if ((mask >> st) & 1u)
-                st_state(a.arena + st * a.stride + e, *reinterpret_cast<const float4 *>(mean + slot(st) * S + 4 * f));
+    for (int st = 0; st < kStates; ++st) {
+        if (((mask >> st) & 1u) == 0) continue;
+        const float4 m4 = *reinterpret_cast<const float4 *>(from);
+        from += S;
+        float *to = a.arena + st * stride + e0;
+        for (int r = r0; r < M; r += rows, to += e_step) st_state(to, m4);
     }
 }
 
@@ -182,13 +192,8 @@ cudaError_t launch_step_sync_tile(const StepArgs &a, int num_sms, cudaStream_t s
     });
     int log2_p = 0;
     while ((4 << log2_p) < w.S) ++log2_p;
-    // One column per lane in the means where the block then has a lane for
-    // each chain, four where it has not: the chains of narrow tiles are what
-    // the block waits for (us, four -> one: M = 39, n = 11k 8.2 -> 6.2; M = 66,
-    // n = 10k 10.3 -> 8.2; M = 177, n = 96k 116 -> 110; but M = 47, n = 149k
-    // 48.1 -> 49.1, M = 32, n = 100k 22.6 -> 24.6).
-    auto kernel = 2 * n_due * w.S <= w.threads ? step_sync_tile_kernel<BASE, N, GDT, CLIP, 1>
-                                               : step_sync_tile_kernel<BASE, N, GDT, CLIP, 4>;
+    auto kernel = a.M < kSplitMeansM ? step_sync_tile_kernel<BASE, N, GDT, CLIP, 1>
+                                     : step_sync_tile_kernel<BASE, N, GDT, CLIP, 0>;
     if (const cudaError_t e = allow_shared(kernel, w.smem); e != cudaSuccess) return e;
     kernel<<<static_cast<unsigned>(a.n_padded / w.S), w.threads, w.smem, stream>>>(a, log2_p);
     return cudaGetLastError();
