@@ -115,14 +115,17 @@ def _load():
 
 
 class _LazyLib:
-    """Loads libmtdao.so on first attribute access."""
+    """Loads libmtdao.so on first attribute access; each function is looked up
+    once and then an attribute of its own."""
 
     _handle = None
 
     def __getattr__(self, name):
         if _LazyLib._handle is None:
             _LazyLib._handle = _load()
-        return getattr(_LazyLib._handle, name)
+        f = getattr(_LazyLib._handle, name)
+        setattr(self, name, f)
+        return f
 
 
 lib = _LazyLib()
@@ -345,6 +348,10 @@ class MTDAO:
         self.offsets = lay["offsets"]
         self.numels = [int(k) for k in numels]
         self.n_mom = int(opt["n_mom"])
+        # what step() checks its gradients against, made once: a step of a small
+        # model is bound by the Python and launch time of its call
+        self._grad_shape = (self.M, self.n_padded)
+        self._grad_codes = {torch.float32: F32, torch.bfloat16: BF16}
 
     def close(self) -> None:
         if getattr(self, "h", None) is not None and self.h.value:
@@ -374,7 +381,7 @@ class MTDAO:
             raise ValueError("%s: dtype %s not supported" % (what, t.dtype))
         if not t.is_contiguous():
             raise ValueError("%s must be contiguous" % what)
-        if (t.device.type == "cuda") != (device == "cuda"):
+        if t.is_cuda != (device == "cuda"):
             raise ValueError("%s must be in %s memory" % (what, "device" if device == "cuda" else "host"))
 
     def _grad_dtypes(self):
@@ -404,7 +411,12 @@ class MTDAO:
         Returns the sync mask that was applied."""
         if sync_mask is None:
             sync_mask = mtdao_sync_due(self.h)
-        self._check_tensor(grads, "grads", (self.M, self.n_padded), self._grad_dtypes(), "cuda")
+        code = None if isinstance(grads, int) else self._grad_codes.get(grads.dtype)
+        if (code is not None and dtype is None and grads.shape == self._grad_shape and grads.is_cuda
+                and grads.is_contiguous()):
+            _check(lib.mtdao_step(self.h, grads.data_ptr(), code, float(lr), sync_mask), self.h)
+            return sync_mask
+        self._check_tensor(grads, "grads", self._grad_shape, self._grad_dtypes(), "cuda")
         dtype = self._grad_code(grads, dtype)
         mtdao_step(self.h, self._ptr(grads), dtype, lr, sync_mask)
         return sync_mask
