@@ -24,7 +24,7 @@ namespace mtdao {
 //   M = 8       : two groups (half-warps) of R = 4, V = 4: replicas 0..3 and
 //                 4..7 are the two parts of the compensated mean of
 //                 replica_mean.cuh, combined by shuffles.
-// M = 6 to 8 on large states (fused_tile_from) and M from 9 to 256 take the tiled kernel of
+// M = 3 to 8 on large states (fused_tile_from) and M from 9 to 256 take the tiled kernel of
 // step_sync_wide.cuh (lane groups went further before: M = 16 as four groups
 // of four replicas, the compensated sums handed from group to group by
 // shuffles, ran at 4.9-5.3 TB/s against 6.7-6.9); above 256, the plain step
@@ -151,25 +151,34 @@ template <int BASE, int N, int M>
 constexpr int kFusedBlocksPerSm = M == 5 || (M == 6 && BASE == MTDAO_BASE_ADOPT && N <= 2) ? 3 : 2;
 constexpr int64_t kFusedThreeFrom = int64_t{1} << 16;
 
-// Smallest n that the tiled kernel of step_sync_wide.cuh takes for M = 6, 7
-// and 8 (0: none).  us here -> tiled, every state due, flat vectors:
-//   M = 8, n = 20M: Adam N = 1 to 4 695 -> 643, 877 -> 832, 1070 -> 1015, 1272
-//   -> 1201, ADOPT 701 -> 648, 882 -> 846, 1084 -> 1023, 1285 -> 1228, SGDM N =
-//   1, 4 497 -> 455, 1085 -> 1012; n = 2M Adam N = 2 95 -> 91, N = 4 133 -> 131;
-//   n = 1M 51 -> 49, 69 -> 71; n = 400k (in L2) 18 -> 21.
-//   M = 7, n = 20M: Adam 639 -> 568, 785 -> 736, 984 -> 891, 1140 -> 1053, ADOPT
-//   641 -> 605, 800 -> 783, 995 -> 909, 1181 -> 1085, SGDM 432 -> 400; n = 2M 86
-//   -> 84, 121 -> 116; n = 1M 47 -> 47; n = 400k 18 -> 21.
-//   M = 6, n = 20M: Adam 571 -> 514, 689 -> 687 (bf16 680 -> 659), 873 -> 794,
-//   989 -> 948, SGDM N = 1, 2, 4 363 -> 343, 506 -> 451, 814 -> 769, ADOPT N =
-//   3, 4 847 -> 830, 1007 -> 994 (N = 1, 2 529 -> 549, 680 -> 739); n = 4M Adam
-//   N = 2, 4 149 -> 152, 210 -> 207; n = 2M 76 -> 80, 107 -> 106.
-// M = 5 stays here (n = 20M, Adam N = 2 554 -> 600, ADOPT 552 -> 649), M = 4 too
-// (Adam N = 3 524 -> 598).
-template <int BASE, int N, int GDT>
+// Smallest n that the tiled kernel of step_sync_wide.cuh takes for M = 3 to 8
+// (0: none).  us here -> tiled, every state due, flat vectors, n = 24M (M = 7
+// and 8 20M):
+//   M = 8: Adam N = 1 to 4 695 -> 643, 877 -> 827, 1070 -> 1012, 1272 -> 1201,
+//   ADOPT 701 -> 648, 882 -> 846, 1084 -> 1023, 1285 -> 1228, SGDM 497 -> 455.
+//   M = 7: Adam 639 -> 568, 785 -> 726, 984 -> 891, 1140 -> 1053, ADOPT 641 ->
+//   605, 800 -> 783, 995 -> 909, 1181 -> 1085, SGDM 432 -> 400.
+//   M = 6: Adam N = 1, 3, 4 686 -> 578, 1051 -> 908, 1176 -> 1036, ADOPT N = 1,
+//   2, 4 635 -> 590, 779 -> 712, 1210 -> 1076, SGDM 435 -> 409.
+//     n = 1M: M = 8 51 -> 49 (SGDM 37 -> 35, Adam N = 4 69 -> 71), M = 6 41 ->
+//     38, SGDM 25 -> 23; n = 300k (in L2) 12 -> 16.
+//   M = 5: Adam 512 -> 499, 815 -> 766, 948 -> 866, ADOPT N = 1, 2, 4 522 -> 543,
+//   629 -> 603, 982 -> 902, SGDM N = 1, 2 347 -> 345, 484 -> 452; n = 2M Adam 62
+//   -> 62, ADOPT 59 -> 61; n = 4M 121 -> 117, 115 -> 113.
+//   M = 4: Adam 413 -> 407, 634 -> 612, 706 -> 696, ADOPT 416 -> 434, 512 -> 489,
+//   736 -> 738, SGDM N = 1, 2 278 -> 280, 372 -> 368; n = 2M Adam N = 2, 4 51 ->
+//   49, 68 -> 70, ADOPT N = 2 51 -> 49; n = 1M 23 -> 25.
+//   M = 3: Adam N = 1, 3, 4 359 -> 366, 549 -> 510, 607 -> 554, ADOPT N = 1, 2, 4
+//   310 -> 400, 448 -> 439, 626 -> 602, SGDM 209 -> 230, 324 -> 314.
+//   M = 2: Adam N = 1, 3 208 -> 268, 319 -> 373.
+template <int BASE, int N>
 constexpr int64_t fused_tile_from(int M) {
-    constexpr bool not6 = BASE == MTDAO_BASE_ADOPT ? N <= 2 : BASE == MTDAO_BASE_ADAM && N == 2 && GDT == MTDAO_F32;
-    return M >= 7 ? int64_t{1} << 21 : (M == 6 && !not6) ? int64_t{1} << 22 : 0;
+    constexpr bool adam = BASE == MTDAO_BASE_ADAM, adopt = BASE == MTDAO_BASE_ADOPT;
+    if (M >= 6) return int64_t{1} << 20;
+    if (M == 5 && !(adopt && N == 1)) return int64_t{1} << (adopt ? 22 : 21);
+    if (M == 4 && (adam ? N <= 3 : adopt ? N == 2 || N == 3 : N >= 2)) return int64_t{1} << 21;
+    if (M == 3 && N >= (adam ? 3 : 2)) return int64_t{1} << 22;
+    return 0;
 }
 
 template <int BASE, int N, int GDT, bool CLIP, int M, int BLOCKS>
@@ -318,7 +327,7 @@ cudaError_t launch_step_sync_t(const StepArgs &a, int num_sms, cudaStream_t stre
 
 template <int BASE, int N, int GDT, bool CLIP>
 cudaError_t launch_step_sync_m(const StepArgs &a, int num_sms, cudaStream_t st) {
-    const int64_t from = fused_tile_from<BASE, N, GDT>(a.M);
+    const int64_t from = fused_tile_from<BASE, N>(a.M);
     if (from > 0 && a.n_padded >= from) return launch_step_sync_tile<BASE, N, GDT, CLIP>(a, num_sms, st);
     switch (a.M) {
         case 2: return launch_step_sync_t<BASE, N, GDT, CLIP, 2>(a, num_sms, st);

@@ -1,6 +1,6 @@
 // step_sync_wide.cuh -- the local step with the replica average fused in,
-// for replica counts above what a lane holds (M = 6 to 8 on large states, 9
-// to kTileMaxM).
+// for replica counts above what a lane holds (M = 9 to kTileMaxM) and for most
+// of M = 3 to 8 on large states.
 //
 // A block owns a tile: S consecutive columns of all M replicas, of every
 // state and of the gradient, copied to shared memory (cp.async) at once.
@@ -192,8 +192,14 @@ cudaError_t launch_step_sync_tile(const StepArgs &a, int num_sms, cudaStream_t s
     });
     int log2_p = 0;
     while ((4 << log2_p) < w.S) ++log2_p;
-    auto kernel = a.M < kSplitMeansM ? step_sync_tile_kernel<BASE, N, GDT, CLIP, 1>
-                                     : step_sync_tile_kernel<BASE, N, GDT, CLIP, 0>;
+    // Means (see tile_means): four columns a lane where that still gives every
+    // lane one (us, one column -> four: M = 4, n = 20M, Adam N = 3 599 -> 514,
+    // ADOPT N = 2 488 -> 409; M = 6, ADOPT N = 2 741 -> 628; M = 12, n = 2^23 511
+    // -> 496; but M = 8, ADOPT N = 2, three states due 785 -> 793, M = 16 659 ->
+    // 671).
+    auto kernel = a.M >= kSplitMeansM              ? step_sync_tile_kernel<BASE, N, GDT, CLIP, 0>
+                  : n_due * w.S >= 4 * w.threads ? step_sync_tile_kernel<BASE, N, GDT, CLIP, 4>
+                                                 : step_sync_tile_kernel<BASE, N, GDT, CLIP, 1>;
     if (const cudaError_t e = allow_shared(kernel, w.smem); e != cudaSuccess) return e;
     kernel<<<static_cast<unsigned>(a.n_padded / w.S), w.threads, w.smem, stream>>>(a, log2_p);
     return cudaGetLastError();

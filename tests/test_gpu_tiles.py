@@ -46,14 +46,15 @@ def _same(a, b):
         assert torch.equal(torch.where(nan, 0.0, x), torch.where(nan, 0.0, y)), s
 
 
-# (M, numel): one tile, an SM's worth of tiles, tiles of every width; M = 7 and 8
-# from 2^21 elements on, 6 from 2^22; the largest tile set that fits (M = 256, N = 4, f32); above it
+# (M, numel): one tile, an SM's worth of tiles, tiles of every width; M = 6 to 8
+# from 2^20 elements on, most of 5 and 4 from 2^21, of 3 from 2^22; the largest tile set that fits (M = 256, N = 4, f32); above it
 CASES = [("adam", 4, "f32", 256, 30000), ("adam", 1, "f32", 256, 512), ("sgdm", 1, "bf16", 256, 1),
-         ("adopt", 2, "bf16", 255, 5000), ("adopt", 2, "bf16", 8, 1 << 21), ("sgdm", 3, "f32", 8, (1 << 21) - 256),
+         ("adopt", 2, "bf16", 255, 5000), ("adopt", 2, "bf16", 8, 1 << 20), ("sgdm", 3, "f32", 8, (1 << 20) - 256),
          ("adam", 2, "f32", 9, 150000), ("adopt", 1, "f32", 16, 20000), ("sgdm", 2, "bf16", 17, 10001),
          ("adam", 3, "f32", 48, 9999), ("adam", 4, "f32", 64, 9999), ("adopt", 2, "bf16", 64, 9999),
          ("sgdm", 4, "f32", 65, 4999), ("adam", 2, "bf16", 100, 4999), ("adam", 3, "f32", 129, 4999),
-         ("adam", 1, "bf16", 257, 3000), ("sgdm", 2, "f32", 6, 1 << 22), ("adopt", 4, "bf16", 7, (1 << 21) + 7),
+         ("adam", 1, "bf16", 257, 3000), ("sgdm", 2, "f32", 6, 1 << 20), ("adopt", 4, "bf16", 7, (1 << 20) + 7),
+         ("adam", 3, "f32", 5, (1 << 21) + 3), ("adopt", 2, "bf16", 4, 1 << 21), ("adam", 4, "f32", 3, 1 << 22),
          ("adam", 3, "f32", 5, 7000), ("adopt", 2, "bf16", 6, 7000)]
 
 
