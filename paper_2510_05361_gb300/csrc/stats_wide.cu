@@ -8,8 +8,8 @@
 // replicas (the average itself).  Every replica value is read from HBM once.
 // What overlaps the copies of a block is the work of the others on its SM.
 //
-// Sums are bit-reproducible: a thread's elements of a tile are summed in fp32,
-// each thread accumulates its tiles with Kahan compensation, the L lanes of a
+// Sums are bit-reproducible: a position's four elements are summed in fp32,
+// each thread accumulates its positions with Kahan compensation, the L lanes of a
 // replica combine their compensated sums by a fixed shuffle pattern, the block
 // writes one compensated sum per quantity, and launch_stats_finalize adds the
 // blocks' in fp64 in a fixed order.
@@ -104,8 +104,8 @@ __global__ void __launch_bounds__(kStatsTileThreads) stats_tile_kernel(const __g
         for (int j = 0; j < R; ++j) {
             const int r = row0 + j * row_step;
             if (r >= M) break;
-            float p0 = 0.0f, p1 = 0.0f, p2 = 0.0f, p3 = 0.0f;
             for (int c = 4 * lane; c < S; c += 4 * L) {
+                float p0 = 0.0f, p1 = 0.0f, p2 = 0.0f, p3 = 0.0f;     // this position's four elements
                 float x[4], mb[4];
                 to_array(*reinterpret_cast<const float4 *>(tile + r * S + c), x);
                 to_array(*reinterpret_cast<const float4 *>(mean + c), mb);
@@ -130,11 +130,11 @@ __global__ void __launch_bounds__(kStatsTileThreads) stats_tile_kernel(const __g
                         p3 = fmaf(mb[q], mb[q], p3);
                     }
                 }
+                own[j].add(p0);
+                cross[j].add(p1);
+                if (!CHANGE || r == 0) all.add(p2);
+                if (r == 0) ref.add(p3);
             }
-            own[j].add(p0);
-            cross[j].add(p1);
-            if (!CHANGE || r == 0) all.add(p2);
-            if (r == 0) ref.add(p3);
         }
         if constexpr (!CHANGE) {
             for (int i = t; i < items; i += static_cast<int>(blockDim.x)) {

@@ -154,7 +154,7 @@ def test_diagnostics_on_tiles(P, M, numel):
     assert float(a.pseudo_grad_stats(0)[: 2 * M + 1].abs().max()) == 0.0
 
     def close(got, want, scale=None):
-        # fp32 sums of at most 64 elements, then compensated: a few 2^-24 of the sum of magnitudes
+        # fp32 sums of four elements, then compensated: a few 2^-24 of the sum of magnitudes
         assert bool(((got - want).abs() <= 2e-6 * (want.abs() if scale is None else scale) + 1e-300).all())
 
     x, anchor = keep[0].double(), x0.double()
