@@ -87,7 +87,8 @@ cudaError_t launch_step(int base, int n_mom, int grad_dtype, bool clip, const St
 
 // Local step with the replica average of the states in a.sync_mask fused
 // into the same pass.  For 2 <= M <= 256; returns cudaErrorNotSupported
-// otherwise (the caller then runs launch_step followed by launch_sync).
+// otherwise, and where the two apart are faster (the caller then runs
+// launch_step followed by launch_sync).
 cudaError_t launch_step_sync(int base, int n_mom, int grad_dtype, bool clip, const StepArgs &a,
                              int num_sms, cudaStream_t stream);
 

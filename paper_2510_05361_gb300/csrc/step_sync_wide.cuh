@@ -190,6 +190,12 @@ cudaError_t launch_step_sync_tile(const StepArgs &a, int num_sms, cudaStream_t s
         return (static_cast<size_t>(tile_set_floats<BASE, N, GDT>(a.M, S)) + static_cast<size_t>(n_due) * S) *
                sizeof(float);
     });
+    // One tile an SM and one or two states due: the step and their average
+    // apart (us, tiled / apart: M = 181, n = 300k, Adam N = 3, bf16, one state
+    // due 469 / 395, three 503 / 520, five 581 / 645; M = 256, n = 150k, Adam N =
+    // 4 364 / 338, 440 / 427, 496 / 515; with two tiles an SM M = 128, n = 500k,
+    // Adam N = 2, one state due 381 / 404, M = 256 SGDM 340 / 417).
+    if (tile_blocks_fit(w.smem) == 1 && n_due <= 2) return cudaErrorNotSupported;
     int log2_p = 0;
     while ((4 << log2_p) < w.S) ++log2_p;
     // Means (see tile_means): four columns a lane where that still gives every
