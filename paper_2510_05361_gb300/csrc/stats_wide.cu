@@ -180,9 +180,9 @@ struct StatsTileShape {
 // round's end -- change of x, then the average of every state with its sums --
 // in us; the previous kernels, one-pass in rows of 128 to 256 bytes with
 // persistent blocks up to M = 64 and two passes above, first).
-//   Columns: 256 up to M = 12 (M = 9, Adam N = 1, n = 8M: 534 -> 380), 128 up
-//   to 16 (M = 16, Adam N = 2, n = 8M: 942 -> 747), else 64 (M = 32, n = 4M: 781
-//   -> 607; M = 64, n = 2M: 709 -> 616; M = 128, n = 600k: 1102 -> 496; M = 256, n = 400k: 1073 -> 598), fewer
+//   Columns: 256 up to M = 12 (M = 9, Adam N = 1, n = 8M: 534 -> 427), 128 up
+//   to 16 (M = 16, Adam N = 2, n = 8M: 942 -> 758), else 64 (M = 32, n = 4M: 781
+//   -> 612; M = 64, n = 2M: 709 -> 617; M = 128, n = 600k: 1102 -> 497; M = 256, n = 400k: 1073 -> 635), fewer
 //   where two tiles would not fit an SM or the SMs would not have one each.
 //   Lanes and threads: the fewer, the more rows a thread takes and the less
 //   there is to combine at a run's end (M = 64, means by lane pairs: 2 lanes and
@@ -231,8 +231,9 @@ cudaError_t launch_stats_tile(StatsTileArgs &a, int n_sel, int num_sms, size_t p
     a.log2_l = w.log2_l;
     a.tiles = w.tiles;
     cudaError_t e;
-    // R = 1 is M <= 64 (tile_means: M = 9 380 us with two columns a lane, 402
-    // with one, 392 with four; M = 64 616 with one, 651 with two)
+    // R = 1 is M <= 64 (tile_means, with the rows' sums compensated once a tile:
+    // M = 9 380 us with two columns a lane, 402 with one, 392 with four; M = 64
+    // 616 with one, 651 with two)
     switch (w.R) {
         case 1:
             e = a.M <= 16 ? launch_stats_tile_t<CHANGE, 1, 2>(a, w, n_sel, stream)

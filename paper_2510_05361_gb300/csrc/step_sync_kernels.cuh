@@ -24,8 +24,8 @@ namespace mtdao {
 //   M = 8       : two groups (half-warps) of R = 4, V = 4: replicas 0..3 and
 //                 4..7 are the two parts of the compensated mean of
 //                 replica_mean.cuh, combined by shuffles.
-// M = 3 to 8 on large states (fused_tile_from) and M from 9 to 256 take the tiled kernel of
-// step_sync_wide.cuh (lane groups went further before: M = 16 as four groups
+// M = 3 to 8 on large states (fused_tile_from) and M from 9 to 256 take the
+// tiled kernel of step_sync_wide.cuh (lane groups went further before: M = 16 as four groups
 // of four replicas, the compensated sums handed from group to group by
 // shuffles, ran at 4.9-5.3 TB/s against 6.7-6.9); above 256, the plain step
 // followed by the standalone average.
