@@ -12,7 +12,7 @@
 // each thread accumulates its positions with Kahan compensation, the L lanes of a
 // replica combine their compensated sums by a fixed shuffle pattern, the block
 // writes one compensated sum per quantity, and launch_stats_finalize adds the
-// blocks' in fp64 in a fixed order.
+// blocks' the same way, in a fixed order.
 #include <cuda_runtime.h>
 #include <cstdint>
 
@@ -182,7 +182,8 @@ struct StatsTileShape {
 // persistent blocks up to M = 64 and two passes above, first).
 //   Columns: 256 up to M = 12 (M = 9, Adam N = 1, n = 8M: 534 -> 427), 128 up
 //   to 16 (M = 16, Adam N = 2, n = 8M: 942 -> 758), else 64 (M = 32, n = 4M: 781
-//   -> 612; M = 64, n = 2M: 709 -> 617; M = 128, n = 600k: 1102 -> 497; M = 256, n = 400k: 1073 -> 635), fewer
+//   -> 612; M = 64, n = 2M: 709 -> 617; M = 128, n = 600k: 1102 -> 497; M =
+//   256, n = 400k: 1073 -> 635), fewer
 //   where two tiles would not fit an SM or the SMs would not have one each.
 //   Lanes and threads: the fewer, the more rows a thread takes and the less
 //   there is to combine at a run's end (M = 64, means by lane pairs: 2 lanes and
