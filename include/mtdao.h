@@ -319,8 +319,9 @@ int mtdao_sync(mtdao_handle h, uint32_t mask);
  * averaging pass itself (the sync's traffic, 8 M bytes per element and
  * state; from M = 9 a block stages a tile of all replicas in shared memory).
  * Every path forms (s_m - s_bar) against the fp32 mean it stores, sums a
- * thread's elements in fp32 with Kahan compensation and adds the partial
- * sums as compensated pairs.  The workspace is allocated on the first call.
+ * thread's elements in fp32 with Kahan compensation, a warp's sums as
+ * compensated pairs (in fp64 where they pass fp32's range) and those of warps
+ * and blocks in fp64.  The workspace is allocated on the first call.
  */
 int mtdao_sync_stats(mtdao_handle h, uint32_t mask, double *stats_dev);
 

@@ -124,9 +124,9 @@ cudaError_t launch_pseudo_grad_stats_tile(const float *x, const float *anchor, i
                                           cudaStream_t stream);
 
 // stats[row * Q + q] = the sum over blocks, in a fixed order, of
-// partial[(row * Q + q) * blocks + b] (Kahan sums, x - y); q = 0 divided by
-// divide_first when that is > 0.
-cudaError_t launch_stats_finalize(const float2 *partial, int64_t blocks, int Q, int rows, int divide_first,
+// partial[(row * Q + q) * blocks + b]; q = 0 divided by divide_first when that
+// is > 0.
+cudaError_t launch_stats_finalize(const double *partial, int64_t blocks, int Q, int rows, int divide_first,
                                   double *stats, cudaStream_t stream);
 
 // Per-replica sum of squares of the gradient: partial sums into

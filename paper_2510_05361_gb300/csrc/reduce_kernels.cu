@@ -287,19 +287,17 @@ __global__ void __launch_bounds__(kNormThreads) sqnorm_finalize_kernel(const dou
 
 // The block's sums of Q values per thread, value j to out[j * gridDim.x].
 template <int Q>
-__device__ __forceinline__ void block_sums(const Kahan (&acc)[Q], float2 *out) {
-    __shared__ float2 part[Q][kThreads / 32];
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-#pragma unroll
-    for (int j = 0; j < Q; ++j) {
-        const Kahan v = lanes_sum(acc[j], 32);
-        if (l == 0) part[j][w] = make_float2(v.s, v.c);
-    }
+__device__ __forceinline__ void block_sums(const Kahan (&acc)[Q], double *out) {
+    __shared__ double part[Q][kThreads / 32];
+    int j;
+    bool one;
+    const double sum = warp_sums_wide<Q>(acc, j, one);
+    if (one) part[j][threadIdx.x >> 5] = sum;
     __syncthreads();
     if (threadIdx.x < Q) {
-        Kahan total;
-        for (int i = 0; i < kThreads / 32; ++i) total = total + Kahan{part[threadIdx.x][i].x, part[threadIdx.x][i].y};
-        out[static_cast<int64_t>(threadIdx.x) * gridDim.x] = make_float2(total.s, total.c);
+        double total = 0.0;
+        for (int i = 0; i < kThreads / 32; ++i) total += part[threadIdx.x][i];
+        out[static_cast<int64_t>(threadIdx.x) * gridDim.x] = total;
     }
 }
 
@@ -312,10 +310,10 @@ __device__ __forceinline__ void block_sums(const Kahan (&acc)[Q], float2 *out) {
 // written to partial[(sel * Q + q) * gridDim.x + block], Q = 2 + 2M.  s_bar
 // is the fp32 mean that is stored, to the state's anchor too where it has one
 // (a copy of replica 0 after the pass took 176 us of the ~124M list's 2942 at
-// a round's end).  The sums travel as compensated fp32 pairs.  With M = 1 nothing is stored (there is nothing to average)
+// a round's end).  With M = 1 nothing is stored (there is nothing to average)
 // but the sums are still formed.
 template <int M>
-__global__ void __launch_bounds__(kThreads) sync_stats_kernel(const __grid_constant__ SyncArgs a, int tile, float2 *partial) {
+__global__ void __launch_bounds__(kThreads) sync_stats_kernel(const __grid_constant__ SyncArgs a, int tile, double *partial) {
     constexpr int Q = 2 + 2 * M;
     float *base = a.arena + static_cast<int64_t>(a.sel[blockIdx.y]) * a.stride;
     const int64_t n = a.n_padded;
@@ -359,29 +357,18 @@ __global__ void __launch_bounds__(kThreads) sync_stats_kernel(const __grid_const
 }
 
 // stats[row * Q + q] = the sum over blocks of partial[(row * Q + q) * blocks + b]
-// (Kahan sums): thread t of block (q, row) adds blocks t, t + 256, ... in
-// order, then lanes and warps combine in a fixed order.  q = 0 is divided by
+// in fp64: thread t of block (q, row) adds blocks t, t + 256, ... in order, then
+// block_sum adds the threads' sums in a fixed order.  q = 0 is divided by
 // divide_first (M for the variance, a mean over workers; 0 leaves it).
-__global__ void __launch_bounds__(kNormThreads) stats_finalize_kernel(const float2 *partial, int64_t blocks, int Q,
+__global__ void __launch_bounds__(kNormThreads) stats_finalize_kernel(const double *partial, int64_t blocks, int Q,
                                                                       int divide_first, double *stats) {
     const int q = blockIdx.x, row = blockIdx.y;
-    const float2 *p = partial + (static_cast<int64_t>(row) * Q + q) * blocks;
-    Kahan acc;
+    const double *p = partial + (static_cast<int64_t>(row) * Q + q) * blocks;
+    double acc = 0.0;
 #pragma unroll 4
-    for (int64_t b = threadIdx.x; b < blocks; b += kNormThreads) {
-        const float2 v = p[b];
-        acc = acc + Kahan{v.x, v.y};
-    }
-    __shared__ float2 part[kNormThreads / 32];
-    acc = lanes_sum(acc, 32);
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = make_float2(acc.s, acc.c);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double total = 0.0;
-        for (int i = 0; i < kNormThreads / 32; ++i)
-            total += static_cast<double>(part[i].x) - static_cast<double>(part[i].y);
-        stats[row * Q + q] = (q == 0 && divide_first > 0) ? total / divide_first : total;
-    }
+    for (int64_t b = threadIdx.x; b < blocks; b += kNormThreads) acc += p[b];
+    const double total = block_sum(acc);
+    if (threadIdx.x == 0) stats[row * Q + q] = (q == 0 && divide_first > 0) ? total / divide_first : total;
 }
 
 int64_t stats_blocks(int64_t n_padded, int tile) {
@@ -396,15 +383,16 @@ int64_t stats_blocks(int64_t n_padded, int tile) {
 // state.  One block per tile, started in index order as earlier blocks retire;
 // every block leaves one row of sums for stats_finalize_kernel, so the sums
 // do not depend on the SM count.  A short tile keeps the addresses under way
-// close together; what it pays for is the row at its end (2M + 2 block
-// reductions, as compensated fp32 pairs: in fp64, at 16 issue cycles an
-// instruction, only tiles of 128 and more paid).  The average of 4 states with
-// its sums, us, with tiles of 128 and fp64 rows -> of 16, here (in brackets 4,
-// 8, 32, 128): M = 2, n = 60M 716 -> 611 (639, 612, 615, 656); M = 4, n = 60M
-// 1291 -> 1173 (1156, 1172, 1179, 1232; 6.57 TB/s); M = 8, n = 30M 1311 -> 1164
-// (1190, 1166, 1173, 1266); M = 1 401 -> 388 (494, 414, 375, 387).  Smaller
-// states take shorter tiles, down to two positions, for 256 blocks: M = 4,
-// n = 1M 89 -> 25, n = 100k 61 -> 14 (tiles of 16 19).
+// close together; what it pays for is the row at its end (2M + 2 sums over the
+// block: as pairs within a warp, in fp64 from there on).  The average of 4
+// states with its sums, us, tiles of 128 with every sum in fp64 -> of 16, here
+// (in brackets 4, 8, 32, 128): M = 1, n = 60M 340 -> 312 (361, 327, 303, 326);
+// M = 2 803 -> 610 (627, 610, 613, 654); M = 4 1362 -> 1168 (1155, 1169, 1178,
+// 1234; 6.6 TB/s); M = 8, n = 30M 1307 -> 1159 (1167, 1169, 1186, 1213).  The
+// warps' sums in fp64 too took 1178 (M = 4), 661 where this takes 614 (M = 6,
+// n = 20M) and 48 where this takes 20 (M = 4, n = 1M).  Smaller states take
+// shorter tiles, down to two positions, for 256 blocks: M = 4, n = 1M 98 -> 20,
+// n = 100k 66 -> 6.5.
 int sync_stats_tile(int64_t n_padded) {
     int tile = 16;
     while (tile > 2 && stats_blocks(n_padded, tile) < 256) tile /= 2;
@@ -419,11 +407,10 @@ cudaError_t launch_sync_stats_t(const SyncArgs &a, double *partial, size_t parti
     const int64_t gx = stats_blocks(a.n_padded, tile);
     if (static_cast<size_t>(gx) * a.n_sel * Q > partial_cap || gx > 0x7fffffff) return cudaErrorInvalidValue;
     dim3 grid(static_cast<unsigned>(gx), static_cast<unsigned>(a.n_sel));
-    float2 *sums = reinterpret_cast<float2 *>(partial);
-    sync_stats_kernel<M><<<grid, kThreads, 0, stream>>>(a, tile, sums);
+    sync_stats_kernel<M><<<grid, kThreads, 0, stream>>>(a, tile, partial);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    stats_finalize_kernel<<<dim3(Q, a.n_sel), kNormThreads, 0, stream>>>(sums, gx, Q, M, stats);
+    stats_finalize_kernel<<<dim3(Q, a.n_sel), kNormThreads, 0, stream>>>(partial, gx, Q, M, stats);
     return cudaGetLastError();
 }
 
@@ -440,7 +427,7 @@ cudaError_t launch_sync_stats_t(const SyncArgs &a, double *partial, size_t parti
 // TB/s; 197 with fp64 rows).
 template <int M>
 __global__ void __launch_bounds__(kThreads) pseudo_grad_stats_kernel(const float *x, const float *anchor,
-                                                                     int64_t n, float2 *partial) {
+                                                                     int64_t n, double *partial) {
     constexpr int Q = 2 * M + 2;
     const int64_t nv = n / 4;
     Kahan acc[Q];
@@ -484,12 +471,11 @@ cudaError_t launch_pseudo_grad_stats_t(const float *x, const float *anchor, int6
     if (gx > need) gx = need;
     if (gx < 1) gx = 1;
     if (static_cast<size_t>(gx) * Q > partial_cap) return cudaErrorInvalidValue;
-    float2 *sums = reinterpret_cast<float2 *>(partial);
-    pseudo_grad_stats_kernel<M><<<static_cast<unsigned>(gx), kThreads, 0, stream>>>(x, anchor, n, sums);
+    pseudo_grad_stats_kernel<M><<<static_cast<unsigned>(gx), kThreads, 0, stream>>>(x, anchor, n, partial);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     // the same fixed-order finalisation as the sync diagnostics, with no division
-    stats_finalize_kernel<<<dim3(Q, 1), kNormThreads, 0, stream>>>(sums, gx, Q, 0, stats);
+    stats_finalize_kernel<<<dim3(Q, 1), kNormThreads, 0, stream>>>(partial, gx, Q, 0, stats);
     return cudaGetLastError();
 }
 
@@ -589,7 +575,7 @@ cudaError_t launch_grad_sqnorm(const void *grads, int grad_dtype, int32_t M, int
 }
 
 
-cudaError_t launch_stats_finalize(const float2 *partial, int64_t blocks, int Q, int rows, int divide_first,
+cudaError_t launch_stats_finalize(const double *partial, int64_t blocks, int Q, int rows, int divide_first,
                                   double *stats, cudaStream_t stream) {
     stats_finalize_kernel<<<dim3(Q, rows), kNormThreads, 0, stream>>>(partial, blocks, Q, divide_first, stats);
     return cudaGetLastError();

@@ -10,9 +10,8 @@
 //
 // Sums are bit-reproducible: a position's four elements are summed in fp32,
 // each thread accumulates its positions with Kahan compensation, the L lanes of a
-// replica combine their compensated sums by a fixed shuffle pattern, the block
-// writes one compensated sum per quantity, and launch_stats_finalize adds the
-// blocks' the same way, in a fixed order.
+// replica combine theirs by a fixed shuffle pattern (kahan.cuh), the block writes
+// one row in fp64, and launch_stats_finalize adds the rows in a fixed order.
 #include <cuda_runtime.h>
 #include <cstdint>
 
@@ -31,30 +30,13 @@ struct StatsTileArgs {
     float *arena;                    // state sel[blockIdx.y] at arena + sel * stride, [M][n]
     const float *anchor;             // change diagnostics: [n]
     float *new_anchor[2 + MTDAO_MAX_MOM];    // sync diagnostics: [n] copy of the mean, or nullptr
-    float2 *partial;                 // [state][Q][gridDim.x]: Kahan sums
+    double *partial;                 // [state][Q][gridDim.x]
     int64_t n, stride;
     int32_t sel[2 + MTDAO_MAX_MOM];
     int32_t M;
     int32_t tiles;                   // tiles of a run
     int32_t log2_s, log2_l;          // columns of a tile, lanes of a replica
 };
-
-// Sum over the block, valid in thread 0 (fixed order).
-__device__ Kahan block_total(Kahan v) {
-    __shared__ float2 part[kStatsTileThreads / 32];
-    v = lanes_sum(v, 32);
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = make_float2(v.s, v.c);
-    __syncthreads();
-    if (threadIdx.x == 0)
-        for (int i = 1; i < static_cast<int>(blockDim.x >> 5); ++i) {
-            Kahan o;
-            o.s = part[i].x;
-            o.c = part[i].y;
-            v = v + o;
-        }
-    __syncthreads();
-    return v;
-}
 
 // CHANGE = false, sync diagnostics (Q = 2 + 2M):
 //   q = 0          sum_m sum_i (s_m - s_bar)^2
@@ -149,24 +131,32 @@ __global__ void __launch_bounds__(kStatsTileThreads) stats_tile_kernel(const __g
     }
 
     const int Q = 2 + 2 * M;
-    float2 *out = a.partial + static_cast<int64_t>(blockIdx.y) * Q * gridDim.x + blockIdx.x;
-    auto put = [&](int q, const Kahan &v) { out[static_cast<int64_t>(q) * gridDim.x] = make_float2(v.s, v.c); };
+    double *out = a.partial + static_cast<int64_t>(blockIdx.y) * Q * gridDim.x + blockIdx.x;
+    auto put = [&](int q, double v) { out[static_cast<int64_t>(q) * gridDim.x] = v; };
     const int own_at = CHANGE ? 0 : 2;
 #pragma unroll
     for (int j = 0; j < R; ++j) {
         const int r = row0 + j * row_step;
-        const Kahan v0 = lanes_sum(own[j], L);
-        const Kahan v1 = lanes_sum(cross[j], L);
-        if (r < M && lane == 0) {
-            put(own_at + r, v0);
-            put(own_at + M + r, v1);
-        }
+        const double v = lanes_sum2_wide(own[j], cross[j], L);
+        if (r < M && lane < 2) put(own_at + lane * M + r, v);
     }
-    const Kahan all_sum = block_total(all);
-    const Kahan ref_sum = block_total(ref);
-    if (t == 0) {
-        put(CHANGE ? 2 * M : 0, all_sum);
-        put(CHANGE ? 2 * M + 1 : 1, ref_sum);
+    if constexpr (CHANGE) {                      // both in the lanes of replica 0
+        if (t < 32) {
+            const double v = lanes_sum2_wide(all, ref, L);
+            if (t < 2) put(2 * M + t, v);
+        }
+    } else {
+        __shared__ double part[kStatsTileThreads / 32];
+        // s_bar^2 lies in the lanes of replica 0, in the first warp
+        const double v = lanes_sum2_wide(all, ref, 32);
+        if ((t & 31) == 0) part[t >> 5] = v;
+        __syncthreads();
+        if (t == 0) {
+            double total = 0.0;
+            for (int i = 0; i < static_cast<int>(blockDim.x >> 5); ++i) total += part[i];
+            put(0, total);
+        }
+        if (t == 1) put(1, v);
     }
 }
 
@@ -264,7 +254,7 @@ cudaError_t launch_sync_stats_tile(const SyncArgs &s, int num_sms, double *parti
     if (s.n_sel <= 0) return cudaSuccess;
     StatsTileArgs a = {};
     a.arena = s.arena;
-    a.partial = reinterpret_cast<float2 *>(partial);
+    a.partial = partial;
     a.n = s.n_padded;
     a.stride = s.stride;
     a.M = s.M;
@@ -281,7 +271,7 @@ cudaError_t launch_pseudo_grad_stats_tile(const float *x, const float *anchor, i
     StatsTileArgs a = {};
     a.arena = const_cast<float *>(x);            // not written
     a.anchor = anchor;
-    a.partial = reinterpret_cast<float2 *>(partial);
+    a.partial = partial;
     a.n = n;
     a.M = M;
     return launch_stats_tile<true>(a, 1, num_sms, partial_cap, stats, stream);

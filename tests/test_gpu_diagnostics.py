@@ -229,3 +229,39 @@ def test_anchors_follow_every_average(P, M, how):
     with pytest.raises(P.MTDAOError):
         eng.pseudo_grad_stats(2)
     eng.close()
+
+
+@pytest.mark.parametrize("M,numel", [(1, 3000000), (2, 3000000), (4, 3000000), (8, 2000000), (9, 1000000), (16, 1000000),
+                                     (64, 400000), (100, 400000), (257, 100000), (1024, 60000)])
+def test_sums_beyond_the_range_of_fp32(P, M, numel):
+    """Values of rms 2e17: what one thread sums fits in fp32 (a square is 4e34), the
+    sums over a block or a state pass 3.4e38, and come out finite in the fp64
+    results."""
+    w = workload_dict([numel], M, base="sgdm", betas=(0.9,))
+    eng = P.MTDAO(w["opt"], M, w["shapes"])
+    gen = torch.Generator(device="cuda").manual_seed(M)
+    x0 = torch.randn(eng.n_padded, device="cuda", generator=gen) * 2e17
+    x = torch.randn((M, eng.n_padded), device="cuda", generator=gen) * 2e17
+    eng.set_params(x0)
+    eng.track_anchor(1)
+    eng.state_view(0).copy_(x)
+    change = eng.pseudo_grad_stats(0)
+    stats = eng.sync_stats(1)[0]
+    x, anchor = x.double(), x0.double()
+    mean = x.mean(0)
+    loc, glob = x - anchor, mean - anchor
+
+    def close(got, want, scale=None):
+        # four elements in fp32: at most 2^-22 of the sum of magnitudes, and as much from the fp32 mean and differences
+        assert bool(torch.isfinite(got).all())
+        assert bool(((got - want).abs() <= 2.0 ** -21 * (want.abs() if scale is None else scale)).all())
+
+    close(change[:M], loc.square().sum(1))
+    close(change[M:2 * M], (loc * glob).sum(1), (loc * glob).abs().sum(1))
+    close(change[2 * M], glob.square().sum())
+    close(change[2 * M + 1], anchor.square().sum())
+    close(stats[0], (x - mean).square().sum() / M)
+    close(stats[1], mean.square().sum())
+    close(stats[2:2 + M], x.square().sum(1))
+    close(stats[2 + M:], (x * mean).sum(1), (x * mean).abs().sum(1))
+    eng.close()
