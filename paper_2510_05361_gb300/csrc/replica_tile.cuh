@@ -149,11 +149,15 @@ inline int64_t tile_blocks_fit(size_t smem) {
     return fit < 1 ? 1 : fit;
 }
 
-// Opts a kernel in to more than the default 48 KB of dynamic shared memory.
+// Opts a kernel in to more than the default 48 KB of dynamic shared memory: to
+// the most that any tile takes, whatever this launch needs.  The limit belongs
+// to the kernel, not to the launch, so a limit of this launch's size would
+// refuse a larger tile that another thread is about to launch.
 template <typename Kernel>
 inline cudaError_t allow_shared(Kernel kernel, size_t smem) {
     if (smem <= 48 * 1024) return cudaSuccess;
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                static_cast<int>(kSharedPerSm - kSharedReserved));
 }
 
 }  // namespace mtdao

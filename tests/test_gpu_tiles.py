@@ -179,3 +179,46 @@ def test_diagnostics_on_tiles(P, M, numel):
 def test_register_diagnostics_tiles(P, M, numel):
     """Tiles of 2 to 16 positions per thread, the last one partly filled."""
     test_diagnostics_on_tiles(P, M, numel)
+
+
+@pytest.mark.parametrize("kind,sizes", [("fused", ((256, 512), (200, 60000))), ("sync", ((1024, 3000), (600, 9000))),
+                                        ("stats", ((1024, 3000), (600, 9000)))])
+def test_tiles_of_different_sizes_from_two_threads(P, kind, sizes):
+    """Two threads, a handle and a stream each, launch the same kernel with tiles of
+    different sizes (both above the default limit of shared memory)."""
+    import threading
+    jobs, errors = [], []
+    for M, numel in sizes:
+        stream = torch.cuda.Stream()
+        w = workload_dict([numel], M, base="adam", betas=(0.9, 0.999, 0.5, 0.99), px=1, pu=1, pv=1)
+        e = P.MTDAO(w["opt"], M, w["shapes"], stream.cuda_stream)
+        g = torch.zeros((M, e.n_padded), device="cuda")
+        out = torch.zeros((e.n_states, 2 + 2 * M), dtype=torch.float64, device="cuda")
+        every = (1 << e.n_states) - 1
+        run = {"fused": lambda e=e, g=g, every=every: e.step(g, 1e-3, every),
+               "sync": lambda e=e, every=every: e.sync(every),
+               "stats": lambda e=e, out=out, every=every: P.mtdao_sync_stats(e.h, every, out.data_ptr())}[kind]
+        run()
+        jobs.append((e, run, stream, g, out))
+    torch.cuda.synchronize()
+    start = threading.Barrier(len(jobs))
+
+    def work(run, stream):
+        try:
+            start.wait()
+            for k in range(4000):
+                run()
+                if k % 200 == 199:
+                    stream.synchronize()
+        except Exception as ex:
+            errors.append(ex)
+
+    threads = [threading.Thread(target=work, args=(run, stream)) for _, run, stream, _, _ in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not errors, errors
+    for e, *_ in jobs:
+        e.close()
