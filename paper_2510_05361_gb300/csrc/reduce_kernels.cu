@@ -64,15 +64,15 @@ constexpr int kSyncTileThreads = 128;
 
 // The average on one tile of S = 4 * 2^log2_p columns of all replicas per
 // block: copied to shared memory, the means formed there, stored to every
-// replica; the blocks start in index order.  Takes M > 14, where a thread
-// that streams the replicas of its position (four loads in flight, persistent
-// grid) has one long chain of loads behind its sums.  That one -> this, us:
+// replica; the blocks start in index order.  Takes M > 14 (but for what
+// stream_replicas names), where a thread that streams the replicas of its
+// position (four loads in flight, persistent grid) has one long chain of loads
+// behind its sums.  That one -> this, us:
 // M = 16, n = 8M, one state 179 -> 152, n = 20k 8.2 -> 4.1; M = 32, n = 5M, 3
 // states 620 -> 552 (6.96 TB/s), n = 200k 14.4 -> 8.2; M = 64, n = 2M 504 ->
-// 448; M = 256, n = 400k 423 -> 366; M = 1024, n = 100k, 2 states 520 -> 378; M
-// = 256, n = 1000 65.5 -> 6.2.  Bound by
-// HBM; above M = 256 by the tiles of 16 to 32 columns (64 to 128 bytes a row)
-// that two of them fit on an SM with.
+// 448; M = 256, n = 400k 423 -> 366, n = 1000 65.5 -> 6.2; M = 1024, n = 20k 258
+// -> 45.  Bound by HBM; from M = 450 on by the rows of 128 and 64 bytes of the
+// tiles that two of them fit on an SM with.
 template <int V>
 __global__ void __launch_bounds__(kSyncTileThreads) sync_tile_kernel(const __grid_constant__ SyncArgs a, int log2_p) {
     extern __shared__ __align__(16) float smem[];
@@ -99,17 +99,23 @@ __global__ void __launch_bounds__(kSyncTileThreads) sync_tile_kernel(const __gri
                  *reinterpret_cast<const float4 *>(mean + 4 * threadIdx.x));
 }
 
+size_t sync_tile_bytes(int M, int log2_p) { return (static_cast<size_t>(M + 1) * 4 * sizeof(float)) << log2_p; }
+
+// Columns of a tile (4 * 2^log2_p) of large states: 128 up to M = 32 (M = 16:
+// 152 us, 64 columns 195), 64 above (M = 64: 448, 128 columns 451), fewer where
+// two tiles would not fit an SM (32 from M = 450, 16 from M = 900).
+int sync_tile_log2_p(int M) {
+    int log2_p = M <= 32 ? 5 : 4;
+    while (log2_p > 1 && 2 * (sync_tile_bytes(M, log2_p) + kSharedReserved) > kSharedPerSm) --log2_p;
+    return log2_p;
+}
+
 cudaError_t launch_sync_tile(const SyncArgs &a, int num_sms, cudaStream_t stream) {
-    auto bytes = [&](int log2_p) { return (static_cast<size_t>(a.M + 1) * 4 * sizeof(float)) << log2_p; };
-    // Columns: 128 up to M = 32 (M = 16: 152 us, 64 columns 195), 64 above (M =
-    // 64: 448, 128 columns 451), fewer where two tiles would not fit an SM or
-    // the SMs would not have one each.  128 threads: M = 32 552 us, 256 560-580,
-    // 512 824-863.
-    int log2_p = a.M <= 32 ? 5 : 4;
-    while (log2_p > 1 && (2 * (bytes(log2_p) + kSharedReserved) > kSharedPerSm ||
-                          (a.n_padded >> (log2_p + 2)) * a.n_sel < num_sms))
-        --log2_p;
-    const size_t smem = bytes(log2_p);
+    // Fewer columns where the SMs would not have a tile each.  128 threads: M =
+    // 32 552 us, 256 560-580, 512 824-863.
+    int log2_p = sync_tile_log2_p(a.M);
+    while (log2_p > 1 && (a.n_padded >> (log2_p + 2)) * a.n_sel < num_sms) --log2_p;
+    const size_t smem = sync_tile_bytes(a.M, log2_p);
     auto kernel = a.M < kSplitMeansM ? sync_tile_kernel<1> : sync_tile_kernel<0>;
     if (const cudaError_t e = allow_shared(kernel, smem); e != cudaSuccess) return e;
     const int64_t gx = a.n_padded >> (log2_p + 2);
@@ -117,6 +123,87 @@ cudaError_t launch_sync_tile(const SyncArgs &a, int num_sms, cudaStream_t stream
     kernel<<<dim3(static_cast<unsigned>(gx), static_cast<unsigned>(a.n_sel)), kSyncTileThreads, smem, stream>>>(
         a, log2_p);
     return cudaGetLastError();
+}
+
+// Mean of the M replicas at float4 position e of state s: replica_mean.cuh's
+// operations in its order, four replicas' loads in flight.
+__device__ __forceinline__ float4 replica_mean4(const float *s, int64_t n, int M, int64_t e) {
+    float s0[4];
+    to_array(ld_state(s + e), s0);
+    DiffSum pa[4] = {DiffSum(s0[0]), DiffSum(s0[1]), DiffSum(s0[2]), DiffSum(s0[3])};
+    DiffSum pb[4] = {DiffSum(s0[0]), DiffSum(s0[1]), DiffSum(s0[2]), DiffSum(s0[3])};
+    float plain[4] = {s0[0], s0[1], s0[2], s0[3]};
+    const int h = M / 2;
+    for (int m = 1; m < M; m += 4) {
+        float r[4][4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (m + u < M) to_array(ld_state(s + (m + u) * n + e), r[u]);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (m + u >= M) break;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                if (m + u < h) pa[k].add(r[u][k]);
+                else pb[k].add(r[u][k]);
+                plain[k] += r[u][k];
+            }
+        }
+    }
+    float mean[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        mean[k] = mean_or_plain(
+            replica_mean_from_parts(s0[k], pa[k].partial(), pb[k].partial(), static_cast<float>(M)), plain[k],
+            static_cast<float>(M));
+    return from_array(mean);
+}
+
+// The average of many replicas of large states (stream_replicas): a thread
+// streams the replicas of its float4 position, on a persistent grid.
+__global__ void __launch_bounds__(kThreads) sync_stream_kernel(const __grid_constant__ SyncArgs a) {
+    float *base = a.arena + static_cast<int64_t>(a.sel[blockIdx.y]) * a.stride;
+    const int64_t n = a.n_padded;
+    const int64_t nv = n / 4;
+    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < nv;
+         i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+        const int64_t e = 4 * i;
+        const float4 mv = replica_mean4(base, n, a.M, e);
+        for (int m = 0; m < a.M; ++m) st_state(base + m * n + e, mv);
+        if (a.anchor[blockIdx.y] != nullptr) st_state(a.anchor[blockIdx.y] + e, mv);
+    }
+}
+
+cudaError_t launch_sync_stream(const SyncArgs &a, int num_sms, cudaStream_t stream) {
+    static const int per_sm = blocks_per_sm(sync_stream_kernel);
+    const int64_t need = (a.n_padded / 4 + kThreads - 1) / kThreads;
+    int64_t gx = static_cast<int64_t>(per_sm) * num_sms / a.n_sel;
+    if (gx > need) gx = need;
+    if (gx < 1) gx = 1;
+    sync_stream_kernel<<<dim3(static_cast<unsigned>(gx), static_cast<unsigned>(a.n_sel)), kThreads, 0, stream>>>(a);
+    return cudaGetLastError();
+}
+
+// Whether n_sel states of n elements are averaged by threads that stream the
+// replicas (rows of 512 bytes a warp, but a chain of loads as long as M) instead
+// of by tiles of all of them.  Where tiles have 64 columns or more, never; below,
+// once there are columns enough for every thread of the streaming grid.  us,
+// tiles / streamed, three states, by columns (n * 3):
+//   16 columns: M = 1024 60k 116 / 269, 176k 329 / 378, 351k 652 / 510, 586k
+//   1139 / 737, 1.2M 2556 / 1520 (one state 117k 227 / 273, 195k 388 / 379).
+//   32 columns, two tiles an SM: M = 768 78k 103 / 206, 234k 290 / 287, 469k 564
+//   / 451, 1.6M 1925 / 1530; M = 896 200k 285 / 331, 402k 552 / 462; M = 640 281k
+//   297 / 253, 560k 583 / 453.
+//   32 columns, three (M < 600): M = 512 1.2M 764 / 772, 2.3M 1614 / 1493; M = 576
+//   1.0M 743 / 773, 2.1M 1601 / 1509; M = 460 1.3M 767 / 832, 2.6M 1618 / 1524
+//   (one state 1.7M 1138 / 1000); M = 597 1.0M 609 / 732.
+//   64 columns: M = 440 2.7M 1418 / 1506; M = 257 4.7M 1399 / 1510.
+bool stream_replicas(int M, int64_t n, int n_sel) {
+    const int log2_p = sync_tile_log2_p(M);
+    const int64_t columns = n * n_sel;
+    if (log2_p >= 4) return false;
+    if (log2_p <= 2) return columns >= 200000;
+    return columns >= (M < 600 ? 1400000 : 300000);
 }
 
 // Deterministic block sum of one double per thread; result valid in thread 0.
@@ -537,7 +624,9 @@ cudaError_t launch_sync(const SyncArgs &a, int num_sms, cudaStream_t stream) {
         case 12: return launch_sync_t<12>(a, stream);
         case 13: return launch_sync_t<13>(a, stream);
         case 14: return launch_sync_t<14>(a, stream);
-        default: return launch_sync_tile(a, num_sms, stream);
+        default:
+            return stream_replicas(a.M, a.n_padded, a.n_sel) ? launch_sync_stream(a, num_sms, stream)
+                                                             : launch_sync_tile(a, num_sms, stream);
     }
 }
 

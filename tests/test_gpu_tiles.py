@@ -130,6 +130,26 @@ def test_average_on_tiles(P, M, numel):
     b.close()
 
 
+@pytest.mark.parametrize("M,numel", [(450, 800001), (600, 200001), (899, 160000), (900, 150001), (1024, 110000)])
+def test_streamed_average_equals_tiles(P, M, numel):
+    """Many replicas: two states together have columns enough to be streamed, each
+    alone is averaged on tiles; the anchor follows."""
+    w = workload_dict([numel], M, base="sgdm", betas=(0.9,), px=1, pu=1, pv=0)
+    (a, b), _ = _pair(P, w, M, "f32", seed=M, plant=True)
+    a.track_anchor(0b10)
+    a.sync(0b11)
+    b.sync(0b01)
+    b.sync(0b10)
+    _same(a, b)
+    for st in range(2):                                # the anchor is the average
+        a.state_view(st).normal_()
+    a.sync(0b11)
+    change = a.pseudo_grad_stats(1)
+    assert float(change[:2 * M + 1].abs().max()) == 0.0 and float(change[2 * M + 1]) > 0.0
+    a.close()
+    b.close()
+
+
 @pytest.mark.parametrize("M,numel", [(9, 256), (9, 700001), (12, 200000), (13, 400001), (16, 100), (17, 200001),
                                      (64, 200001), (65, 200001), (128, 5000), (129, 90000), (257, 20000),
                                      (513, 9000), (1024, 8000)])
