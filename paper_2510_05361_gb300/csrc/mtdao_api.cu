@@ -98,6 +98,7 @@ struct mtdao_ctx {
     int norm_blocks = 1;
     double *stats_partial = nullptr;  // diagnostics workspace (allocated on first use)
     size_t stats_cap = 0;
+    float *stats_mean = nullptr;      // [n_padded] replica mean of streamed diagnostics (likewise)
     float *anchor[2 + MTDAO_MAX_MOM] = {};  // per state: its value at the last average
     // host-gradient staging (mtdao_step_host)
     void *staging[2] = {nullptr, nullptr};
@@ -277,6 +278,7 @@ void release(mtdao_ctx *h) {
     if (h->norm_out) cudaFree(h->norm_out);
     if (h->norm_partial) cudaFree(h->norm_partial);
     if (h->stats_partial) cudaFree(h->stats_partial);
+    if (h->stats_mean) cudaFree(h->stats_mean);
     for (float *a : h->anchor)
         if (a) cudaFree(a);
 }
@@ -523,14 +525,26 @@ static int refresh_anchor(mtdao_ctx *h, uint32_t mask) {
 }
 
 // Diagnostics kernels hold M replicas in registers up to this M; above it
-// they stage them in shared memory (stats_wide.cu).
+// they stage them in shared memory (stats_wide.cu), or stream them twice where
+// stream_stats says so.
 constexpr int kStatsRegisterM = 8;
 
+// The workspace serves both kinds of diagnostics, with any states.
 static int ensure_stats_workspace(mtdao_ctx *h) {
+    const bool streams = stream_stats(h->M, h->n_padded, false) || stream_stats(h->M, h->n_padded, true);
+    if (h->stats_partial != nullptr && (!streams || h->stats_mean != nullptr)) return MTDAO_OK;
+    if (streams && h->stats_mean == nullptr) {
+        cudaError_t e = cudaMalloc(reinterpret_cast<void **>(&h->stats_mean), h->n_padded * sizeof(float));
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            h->stats_mean = nullptr;
+            return set_error(h, MTDAO_ERR_OOM, "diagnostics scratch: %s", cudaGetErrorString(e));
+        }
+    }
     if (h->stats_partial != nullptr) return MTDAO_OK;
-    const size_t cap = h->M <= kStatsRegisterM
-                           ? sync_stats_partial_capacity(h->num_sms, h->n_padded, h->n_states, h->M)
-                           : tile_stats_partial_capacity(h->num_sms, h->n_padded, h->n_states, h->M);
+    size_t cap = h->M <= kStatsRegisterM ? sync_stats_partial_capacity(h->num_sms, h->n_padded, h->n_states, h->M)
+                                         : tile_stats_partial_capacity(h->num_sms, h->n_padded, h->n_states, h->M);
+    if (streams) cap = std::max(cap, stream_stats_partial_capacity(h->num_sms, h->n_padded, h->M));
     cudaError_t e = cudaMalloc(reinterpret_cast<void **>(&h->stats_partial), cap * sizeof(double));
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -785,6 +799,9 @@ extern "C" int mtdao_sync_stats(mtdao_handle h, uint32_t mask, double *stats_dev
     const SyncArgs a = sync_args(h, mask);
     cudaError_t e = h->M <= kStatsRegisterM
                         ? launch_sync_stats(a, h->num_sms, h->stats_partial, h->stats_cap, stats_dev, h->stream)
+                    : stream_stats(h->M, h->n_padded, false)
+                        ? launch_sync_stats_stream(a, h->num_sms, h->stats_mean, h->stats_partial, h->stats_cap,
+                                                   stats_dev, h->stream)
                         : launch_sync_stats_tile(a, h->num_sms, h->stats_partial, h->stats_cap, stats_dev, h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "sync with diagnostics launch");
     return h->M > 1 ? MTDAO_OK : refresh_anchor(h, mask);
@@ -835,6 +852,10 @@ extern "C" int mtdao_pseudo_grad_stats(mtdao_handle h, int32_t state, double *ou
     cudaError_t e = h->M <= kStatsRegisterM
                         ? launch_pseudo_grad_stats(x, h->anchor[state], h->n_padded, h->M, h->num_sms,
                                                    h->stats_partial, h->stats_cap, out_dev, h->stream)
+                    : stream_stats(h->M, h->n_padded, true)
+                        ? launch_pseudo_grad_stats_stream(x, h->anchor[state], h->n_padded, h->M, h->num_sms,
+                                                          h->stats_mean, h->stats_partial, h->stats_cap, out_dev,
+                                                          h->stream)
                         : launch_pseudo_grad_stats_tile(x, h->anchor[state], h->n_padded, h->M, h->num_sms,
                                                         h->stats_partial, h->stats_cap, out_dev, h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "change diagnostics launch");

@@ -123,6 +123,17 @@ cudaError_t launch_pseudo_grad_stats_tile(const float *x, const float *anchor, i
                                           double *partial, size_t partial_cap, double *stats,
                                           cudaStream_t stream);
 
+// The same for many replicas of large states (stream_stats): two passes per
+// state through a [n_padded] fp32 scratch that holds the replica mean.
+// Workspace: partial needs stream_stats_partial_capacity() doubles.
+bool stream_stats(int M, int64_t n, bool change);
+size_t stream_stats_partial_capacity(int num_sms, int64_t n_padded, int M);
+cudaError_t launch_sync_stats_stream(const SyncArgs &a, int num_sms, float *mean, double *partial, size_t partial_cap,
+                                     double *stats, cudaStream_t stream);
+cudaError_t launch_pseudo_grad_stats_stream(const float *x, const float *anchor, int64_t n, int M, int num_sms,
+                                            float *mean, double *partial, size_t partial_cap, double *stats,
+                                            cudaStream_t stream);
+
 // stats[row * Q + q] = the sum over blocks, in a fixed order, of
 // partial[(row * Q + q) * blocks + b]; q = 0 divided by divide_first when that
 // is > 0.

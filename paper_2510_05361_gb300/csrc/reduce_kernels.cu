@@ -372,9 +372,9 @@ __global__ void __launch_bounds__(kNormThreads) sqnorm_finalize_kernel(const dou
 
 // ---------------------------------------------------------------- sync + diagnostics
 
-// The block's sums of Q values per thread, value j to out[j * gridDim.x].
+// The block's sums of Q values per thread, value j to out[j * stride].
 template <int Q>
-__device__ __forceinline__ void block_sums(const Kahan (&acc)[Q], double *out) {
+__device__ __forceinline__ void block_sums(const Kahan (&acc)[Q], double *out, int64_t stride) {
     __shared__ double part[Q][kThreads / 32];
     int j;
     bool one;
@@ -384,7 +384,7 @@ __device__ __forceinline__ void block_sums(const Kahan (&acc)[Q], double *out) {
     if (threadIdx.x < Q) {
         double total = 0.0;
         for (int i = 0; i < kThreads / 32; ++i) total += part[threadIdx.x][i];
-        out[static_cast<int64_t>(threadIdx.x) * gridDim.x] = total;
+        out[threadIdx.x * stride] = total;
     }
 }
 
@@ -440,7 +440,7 @@ __global__ void __launch_bounds__(kThreads) sync_stats_kernel(const __grid_const
             if (a.anchor[blockIdx.y] != nullptr) st_state(a.anchor[blockIdx.y] + e, mv);
         }
     }
-    block_sums<Q>(acc, partial + static_cast<int64_t>(blockIdx.y) * Q * gridDim.x + blockIdx.x);
+    block_sums<Q>(acc, partial + static_cast<int64_t>(blockIdx.y) * Q * gridDim.x + blockIdx.x, gridDim.x);
 }
 
 // stats[row * Q + q] = the sum over blocks of partial[(row * Q + q) * blocks + b]
@@ -544,7 +544,7 @@ __global__ void __launch_bounds__(kThreads) pseudo_grad_stats_kernel(const float
 #pragma unroll
         for (int j = 0; j < Q; ++j) acc[j].add(q[j]);
     }
-    block_sums<Q>(acc, partial + blockIdx.x);
+    block_sums<Q>(acc, partial + blockIdx.x, gridDim.x);
 }
 
 template <int M>
@@ -566,7 +566,215 @@ cudaError_t launch_pseudo_grad_stats_t(const float *x, const float *anchor, int6
     return cudaGetLastError();
 }
 
+// ---------------------------------------------------------------- diagnostics, replicas streamed
+
+// For many replicas of large states (stream_stats) the diagnostics take two
+// passes over a state; a [n] fp32 scratch holds the mean between them:
+//   pass 1 (grid-stride over float4 positions): the replica mean of
+//     replica_mean.cuh, written to the scratch (and to the state's anchor),
+//     and the sums that need only the mean (and the anchor);
+//   pass 2 (grid (blocks, M)): per replica the sums against the scratch mean
+//     and, for an average, the mean written over the replica.
+// The sums go as in the one-pass kernels: four elements in fp32, a thread's
+// positions with Kahan compensation, warps, blocks and the finalize in fp64.
+
+// Positions a pass-2 thread loads before it accumulates them (i, i + T,
+// i + 2T, ...: the order of a plain grid-stride loop): four for the sync
+// diagnostics (two float4 loads per position), two for the change
+// diagnostics (three per position, within 64 registers).
+constexpr int kPass2Unroll = 4;
+constexpr int kPass2UnrollChange = 2;
+
+// Pass 1.  Per block s_bar^2, or with CHANGE (x_bar - a)^2 and a^2: value j at
+// partial[j * gridDim.x + block].
+template <bool CHANGE>
+__global__ void __launch_bounds__(kThreads, 4) stream_stats_pass1_kernel(const float *s, const float *anchor, int64_t n,
+                                                                         int M, float *mean_out, float *new_anchor,
+                                                                         double *partial) {
+    constexpr int K = CHANGE ? 2 : 1;
+    const int64_t nv = n / 4;
+    Kahan acc[K];
+    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < nv;
+         i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+        const int64_t e = 4 * i;
+        const float4 mv = replica_mean4(s, n, M, e);
+        *reinterpret_cast<float4 *>(mean_out + e) = mv;
+        if (new_anchor != nullptr) st_state(new_anchor + e, mv);
+        float mean[4], p0 = 0.0f;
+        to_array(mv, mean);
+        if constexpr (CHANGE) {
+            float a[4], p1 = 0.0f;
+            to_array(__ldcs(reinterpret_cast<const float4 *>(anchor + e)), a);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const float glob = mean[k] - a[k];
+                p0 = fmaf(glob, glob, p0);
+                p1 = fmaf(a[k], a[k], p1);
+            }
+            acc[K - 1].add(p1);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) p0 = fmaf(mean[k], mean[k], p0);
+        }
+        acc[0].add(p0);
+    }
+    block_sums<K>(acc, partial + blockIdx.x, gridDim.x);
+}
+
+// Pass 2 of the sync diagnostics, replica m = blockIdx.y: per block
+// (s_m - s_bar)^2, s_m^2 and s_m * s_bar, value j at
+// partial[(j * M + m) * gridDim.x + block]; the replica becomes the mean.
+__global__ void __launch_bounds__(kThreads, 4) stream_sync_stats_pass2_kernel(float *s, int64_t n, const float *mean,
+                                                                              double *partial) {
+    const int m = blockIdx.y;
+    const int64_t nv = n / 4;
+    const int64_t T = static_cast<int64_t>(gridDim.x) * blockDim.x;
+    float *rep = s + m * n;
+    Kahan acc[3];
+    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < nv; i += kPass2Unroll * T) {
+        float4 rv[kPass2Unroll], mv[kPass2Unroll];
+#pragma unroll
+        for (int u = 0; u < kPass2Unroll; ++u)
+            if (i + u * T < nv) {
+                rv[u] = ld_state(rep + 4 * (i + u * T));
+                mv[u] = *reinterpret_cast<const float4 *>(mean + 4 * (i + u * T));
+            }
+#pragma unroll
+        for (int u = 0; u < kPass2Unroll; ++u) {
+            if (i + u * T >= nv) break;
+            float r[4], mb[4];
+            to_array(rv[u], r);
+            to_array(mv[u], mb);
+            float p0 = 0.0f, p1 = 0.0f, p2 = 0.0f;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const float dv = r[k] - mb[k];
+                p0 = fmaf(dv, dv, p0);
+                p1 = fmaf(r[k], r[k], p1);
+                p2 = fmaf(r[k], mb[k], p2);
+            }
+            acc[0].add(p0);
+            acc[1].add(p1);
+            acc[2].add(p2);
+            st_state(rep + 4 * (i + u * T), mv[u]);
+        }
+    }
+    block_sums<3>(acc, partial + static_cast<int64_t>(m) * gridDim.x + blockIdx.x,
+                  static_cast<int64_t>(gridDim.y) * gridDim.x);
+}
+
+// Pass 2 of the change diagnostics, replica m = blockIdx.y: per block
+// (x_m - a)^2 and (x_m - a)(x_bar - a), laid out as above.  Read-only.
+__global__ void __launch_bounds__(kThreads, 4) stream_change_pass2_kernel(const float *x, const float *anchor, int64_t n,
+                                                                          const float *mean, double *partial) {
+    const int m = blockIdx.y;
+    const int64_t nv = n / 4;
+    const int64_t T = static_cast<int64_t>(gridDim.x) * blockDim.x;
+    const float *rep = x + m * n;
+    Kahan acc[2];
+    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < nv; i += kPass2UnrollChange * T) {
+        float4 rv[kPass2UnrollChange], mv[kPass2UnrollChange], av[kPass2UnrollChange];
+#pragma unroll
+        for (int u = 0; u < kPass2UnrollChange; ++u)
+            if (i + u * T < nv) {
+                const int64_t e = 4 * (i + u * T);
+                rv[u] = ld_state(rep + e);
+                mv[u] = *reinterpret_cast<const float4 *>(mean + e);
+                av[u] = *reinterpret_cast<const float4 *>(anchor + e);
+            }
+#pragma unroll
+        for (int u = 0; u < kPass2UnrollChange; ++u) {
+            if (i + u * T >= nv) break;
+            float r[4], mb[4], a[4];
+            to_array(rv[u], r);
+            to_array(mv[u], mb);
+            to_array(av[u], a);
+            float p0 = 0.0f, p1 = 0.0f;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const float loc = r[k] - a[k];
+                const float glob = mb[k] - a[k];
+                p0 = fmaf(loc, loc, p0);
+                p1 = fmaf(loc, glob, p1);
+            }
+            acc[0].add(p0);
+            acc[1].add(p1);
+        }
+    }
+    block_sums<2>(acc, partial + static_cast<int64_t>(m) * gridDim.x + blockIdx.x,
+                  static_cast<int64_t>(gridDim.y) * gridDim.x);
+}
+
+struct StreamGrid {
+    int b1, b2;                      // blocks of pass 1, and of a replica in pass 2
+};
+
+StreamGrid stream_grid2(int num_sms, int M, int64_t n) {
+    const int64_t need = (n / 4 + kThreads - 1) / kThreads;
+    int64_t b1 = 4 * static_cast<int64_t>(num_sms), b2 = b1 / M;
+    if (b1 > need) b1 = need;
+    if (b2 > need) b2 = need;
+    return {static_cast<int>(b1 < 1 ? 1 : b1), static_cast<int>(b2 < 1 ? 1 : b2)};
+}
+
 }  // namespace
+
+// Two passes with rows of 512 bytes a warp against one pass on tiles of 32 or 16
+// columns.  us, tiles / streamed:
+//   16 columns (M > 898): M = 1024, average with sums of one state n = 59k 257 /
+//   316, 117k 471 / 404, 391k 1514 / 848; change n = 59k 226 / 279, 117k 409 /
+//   326, 781k 2413 / 1159.
+//   32 columns: change M = 512 234k 206 / 220, 391k 325 / 294, 1.6M 1162 / 1060; M
+//   = 768 260k 399 / 382, 1.0M 1384 / 1230; average with sums M = 896 223k 490 /
+//   518, 446k 1025 / 854; M = 768 521k 994 / 862; M = 640 312k 532 / 482, three
+//   states 1472 / 1441.  Up to M = 598 three tiles fit an SM: M = 512 781k 821 /
+//   921.
+//   M < 450 (32 columns from M = 257, 64 below): M = 440 change 1.8M 996 / 1102.
+bool stream_stats(int M, int64_t n, bool change) {
+    if (M < 450) return false;
+    if (M > 898) return n >= (change ? 81920 : 98304);
+    return change ? n >= 262144 : M >= 599 && n >= 393216;
+}
+
+size_t stream_stats_partial_capacity(int num_sms, int64_t n_padded, int M) {
+    const StreamGrid g = stream_grid2(num_sms, M, n_padded);
+    return 2 * static_cast<size_t>(g.b1) + 3 * static_cast<size_t>(g.b2) * static_cast<size_t>(M);
+}
+
+cudaError_t launch_sync_stats_stream(const SyncArgs &a, int num_sms, float *mean, double *partial, size_t partial_cap,
+                                     double *stats, cudaStream_t stream) {
+    const int M = a.M;
+    const StreamGrid g = stream_grid2(num_sms, M, a.n_padded);
+    if (stream_stats_partial_capacity(num_sms, a.n_padded, M) > partial_cap) return cudaErrorInvalidValue;
+    double *p1 = partial, *p2 = partial + g.b1;
+    const int64_t per_sum = static_cast<int64_t>(M) * g.b2;
+    for (int k = 0; k < a.n_sel; ++k, stats += 2 + 2 * M) {
+        float *s = a.arena + static_cast<int64_t>(a.sel[k]) * a.stride;
+        stream_stats_pass1_kernel<false><<<g.b1, kThreads, 0, stream>>>(s, nullptr, a.n_padded, M, mean, a.anchor[k], p1);
+        stream_sync_stats_pass2_kernel<<<dim3(g.b2, M), kThreads, 0, stream>>>(s, a.n_padded, mean, p2);
+        // stats row: [0] variance (over all replicas' blocks), [1] s_bar^2, [2 + m] s_m^2, [2 + M + m] s_m s_bar
+        stats_finalize_kernel<<<1, kNormThreads, 0, stream>>>(p2, per_sum, 1, M, stats);
+        stats_finalize_kernel<<<1, kNormThreads, 0, stream>>>(p1, g.b1, 1, 0, stats + 1);
+        stats_finalize_kernel<<<2 * M, kNormThreads, 0, stream>>>(p2 + per_sum, g.b2, 2 * M, 0, stats + 2);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+cudaError_t launch_pseudo_grad_stats_stream(const float *x, const float *anchor, int64_t n, int M, int num_sms,
+                                            float *mean, double *partial, size_t partial_cap, double *stats,
+                                            cudaStream_t stream) {
+    const StreamGrid g = stream_grid2(num_sms, M, n);
+    if (stream_stats_partial_capacity(num_sms, n, M) > partial_cap) return cudaErrorInvalidValue;
+    double *p1 = partial, *p2 = partial + 2 * g.b1;
+    stream_stats_pass1_kernel<true><<<g.b1, kThreads, 0, stream>>>(x, anchor, n, M, mean, nullptr, p1);
+    stream_change_pass2_kernel<<<dim3(g.b2, M), kThreads, 0, stream>>>(x, anchor, n, mean, p2);
+    // [m] (x_m - a)^2, [M + m] (x_m - a)(x_bar - a), [2M] (x_bar - a)^2, [2M + 1] a^2
+    stats_finalize_kernel<<<2 * M, kNormThreads, 0, stream>>>(p2, g.b2, 2 * M, 0, stats);
+    stats_finalize_kernel<<<2, kNormThreads, 0, stream>>>(p1, g.b1, 2, 0, stats + 2 * M);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_pseudo_grad_stats(const float *x, const float *anchor, int64_t n, int M, int num_sms,
                                      double *partial, size_t partial_cap, double *stats,

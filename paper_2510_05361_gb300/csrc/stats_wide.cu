@@ -171,9 +171,11 @@ struct StatsTileShape {
 // in us; the previous kernels, one-pass in rows of 128 to 256 bytes with
 // persistent blocks up to M = 64 and two passes above, first).
 //   Columns: 256 up to M = 12 (M = 9, Adam N = 1, n = 8M: 534 -> 427), 128 up
-//   to 16 (M = 16, Adam N = 2, n = 8M: 942 -> 758), else 64 (M = 32, n = 4M: 781
-//   -> 612; M = 64, n = 2M: 709 -> 617; M = 128, n = 600k: 1102 -> 497; M =
-//   256, n = 400k: 1073 -> 635), fewer
+//   to 16 (M = 16, Adam N = 2, n = 8M: 942 -> 758), 64 up to 256 (M = 32, n =
+//   4M: 781 -> 612; M = 64, n = 2M: 709 -> 617; M = 128, n = 600k: 1102 -> 497; M
+//   = 256, n = 400k: 1073 -> 635), 32 above, where 64 leave an SM two or three
+//   small blocks (change, M = 320, n = 1.25M 911 -> 553, M = 257, n = 3.1M 1339
+//   -> 1022; average with sums, M = 384, n = 521k, 3 states 1457 -> 1044); fewer
 //   where two tiles would not fit an SM or the SMs would not have one each.
 //   Lanes and threads: the fewer, the more rows a thread takes and the less
 //   there is to combine at a run's end (M = 64, means by lane pairs: 2 lanes and
@@ -186,7 +188,7 @@ struct StatsTileShape {
 StatsTileShape stats_tile_shape(int num_sms, int64_t n, int n_sel, int M) {
     StatsTileShape w;
     auto bytes = [&](int log2_s) { return static_cast<size_t>(M + 2) * sizeof(float) << log2_s; };
-    w.log2_s = M <= 12 ? 8 : (M <= 16 ? 7 : 6);
+    w.log2_s = M <= 12 ? 8 : (M <= 16 ? 7 : (M <= 256 ? 6 : 5));
     while (w.log2_s > 3 &&
            (2 * (bytes(w.log2_s) + kSharedReserved) > kSharedPerSm || (n >> w.log2_s) * n_sel < num_sms))
         --w.log2_s;

@@ -232,7 +232,8 @@ def test_anchors_follow_every_average(P, M, how):
 
 
 @pytest.mark.parametrize("M,numel", [(1, 3000000), (2, 3000000), (4, 3000000), (8, 2000000), (9, 1000000), (16, 1000000),
-                                     (64, 400000), (100, 400000), (257, 100000), (1024, 60000)])
+                                     (64, 400000), (100, 400000), (257, 100000), (1024, 60000), (600, 400001),
+                                     (1024, 90001)])
 def test_sums_beyond_the_range_of_fp32(P, M, numel):
     """Values of rms 2e17: what one thread sums fits in fp32 (a square is 4e34), the
     sums over a block or a state pass 3.4e38, and come out finite in the fp64

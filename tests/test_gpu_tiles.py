@@ -195,6 +195,14 @@ def test_diagnostics_on_tiles(P, M, numel):
     b.close()
 
 
+@pytest.mark.parametrize("M,numel", [(449, 270001), (450, 262000), (450, 262145), (599, 393217), (898, 270000),
+                                     (899, 81900), (899, 82001), (1024, 98305)])
+def test_streamed_diagnostics(P, M, numel):
+    """Both sides of the limits above which many replicas are streamed in two passes
+    (M = 450 to 599: the change alone)."""
+    test_diagnostics_on_tiles(P, M, numel)
+
+
 @pytest.mark.parametrize("M,numel", [(1, 5), (2, 1024), (3, 2049), (4, 600000), (5, 1100001), (8, 2200003), (7, 4200000)])
 def test_register_diagnostics_tiles(P, M, numel):
     """Tiles of 2 to 16 positions per thread, the last one partly filled."""
