@@ -139,17 +139,26 @@ __device__ __forceinline__ void load_replicas(const float *state, int64_t n_padd
     for (int r = 0; r < S::R; ++r) ld_v<S::V>(state + (grp * S::R + r) * n_padded + e, val[r]);
 }
 
-// Blocks of an SM that the registers are cut for: two (128 registers), three
-// (80) where that ran faster on flat 20M vectors with every state due (us, two
-// -> three): M = 5 Adam N = 1 to 4 500 -> 428, 604 -> 552, 754 -> 680, 865 ->
-// 835, ADOPT 499 -> 437, 621 -> 551, 879 -> 822, bf16 ADOPT N = 3 770 -> 651;
-// M = 6 ADOPT N = 1, 2 569 -> 527, 709 -> 681 (N = 4 1008 -> 1050, Adam N = 3
-// 874 -> 894); M = 4 Adam N = 3 783 -> 820, M = 7 Adam N = 2 785 -> 925.
-// Below kFusedThreeFrom elements the SMs have no third block to take (M = 5,
-// ADOPT N = 4, n = 20k, where 80 registers spill: 8.5 us with two, 10.3).
+// Blocks of an SM that the registers are cut for: two (128 registers), or three
+// (80) for M = 5 and ADOPT's M = 6 with N <= 2, which on a persistent grid take
+// them where the third block saves a round of the grid.  us, two / three blocks,
+// every state due (152 SMs: a round is 155,648 elements with two blocks, 233,472
+// with three):
+//             M = 5 Adam N = 1, N = 3  ADOPT N = 4    SGDM N = 2, N = 4   M = 6 ADOPT N = 2
+//   n = 100k  3.9 / 3.8, 4.9 / 5.3     5.7 / 6.3      3.1 / 3.1, 4.1 / 4.6    5.2 / 5.8
+//       200k  6.2 / 4.6, 8.2 / 6.7     9.7 / 8.2      4.7 / 4.2, 6.5 / 6.1    8.6 / 7.2
+//       300k  6.7 / 6.9, 9.2 / 10.4    11.1 / 12.6    5.3 / 5.2, 7.4 / 8.8    9.6 / 10.9
+//       400k  9.3 / 7.9, 12.5 / 12.1   15.9 / 15.0    7.1 / 6.4, 10.5 / 10.5  13.2 / 12.7
+//       700k  16.7 / 13.3, 28.5 / 23.1 36.5 / 31.8    9.9 / 9.3, 22.7 / 21.5  27.5 / 23.7
+//   ADOPT M = 5, N = 1, n = 4.2M (which the tiles do not take): 118 / 101.
 template <int BASE, int N, int M>
 constexpr int kFusedBlocksPerSm = M == 5 || (M == 6 && BASE == MTDAO_BASE_ADOPT && N <= 2) ? 3 : 2;
-constexpr int64_t kFusedThreeFrom = int64_t{1} << 16;
+
+// Rounds of a persistent grid of that many blocks an SM over the warps' items.
+inline int64_t grid_rounds(int blocks, int num_sms, int64_t n_warp_items) {
+    const int64_t warps = static_cast<int64_t>(blocks) * num_sms * (kThreads / 32);
+    return (n_warp_items + warps - 1) / warps;
+}
 
 // Smallest n that the tiled kernel of step_sync_wide.cuh takes for M = 3 to 8
 // (0: none).  us here -> tiled, every state due, flat vectors, n = 24M (M = 7
@@ -303,11 +312,11 @@ cudaError_t launch_step_sync_b(const StepArgs &a, int num_sms, cudaStream_t stre
     // M = 4 N = 2..4 6.6 -> 6.9-7.0 TB/s, SGDM N = 1 6487 -> 7061, but Adam
     // N = 1 6713 -> 6460 (M = 2), 6725 -> 6120 (M = 4), 6108 -> 5346 (M = 3)
     // and ADOPT N = 1 6447 -> 6248.  The 64-element chunks of M >= 5 keep
-    // the persistent grid (M = 8, ~350M workload: 6504 -> 6409), but for M =
-    // 5's SGDM (n = 20M, N = 1, 4: 310 -> 288, 693 -> 666 us).
+    // the persistent grid (M = 8, ~350M workload: 6504 -> 6409; M = 5, SGDM N = 2,
+    // n = 480k, two blocks 8.1 us, one chunk per warp 8.7, n = 1M 16.5, 18.3).
     auto kernel = step_sync_kernel<BASE, N, GDT, CLIP, M, BLOCKS>;
     int grid;
-    if constexpr (M <= 5 && (BASE == MTDAO_BASE_SGDM || (N >= 2 && M <= 4))) {
+    if constexpr (M <= 4 && (BASE == MTDAO_BASE_SGDM || N >= 2)) {
         grid = stream_grid(a.n_padded / FusedShape<M>::kChunk);
     } else {
         static const int per_sm = blocks_per_sm(kernel);
@@ -320,7 +329,8 @@ cudaError_t launch_step_sync_b(const StepArgs &a, int num_sms, cudaStream_t stre
 template <int BASE, int N, int GDT, bool CLIP, int M>
 cudaError_t launch_step_sync_t(const StepArgs &a, int num_sms, cudaStream_t stream) {
     constexpr int kBlocks = kFusedBlocksPerSm<BASE, N, M>;
-    if (kBlocks > 2 && a.n_padded >= kFusedThreeFrom)
+    const int64_t chunks = a.n_padded / FusedShape<M>::kChunk;
+    if (kBlocks > 2 && grid_rounds(kBlocks, num_sms, chunks) < grid_rounds(2, num_sms, chunks))
         return launch_step_sync_b<BASE, N, GDT, CLIP, M, kBlocks>(a, num_sms, stream);
     return launch_step_sync_b<BASE, N, GDT, CLIP, M, 2>(a, num_sms, stream);
 }

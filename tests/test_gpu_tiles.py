@@ -56,6 +56,11 @@ CASES = [("adam", 4, "f32", 256, 30000), ("adam", 1, "f32", 256, 512), ("sgdm", 
          ("adam", 1, "bf16", 257, 3000), ("sgdm", 2, "f32", 6, 1 << 20), ("adopt", 4, "bf16", 7, (1 << 20) + 7),
          ("adam", 3, "f32", 5, (1 << 21) + 3), ("adopt", 2, "bf16", 4, 1 << 21), ("adam", 4, "f32", 3, 1 << 22),
          ("adam", 3, "f32", 5, 7000), ("adopt", 2, "bf16", 6, 7000)]
+# M = 5 and ADOPT's M = 6: two blocks an SM or three, by the rounds of the grid
+CASES += ([(base, N, gdt, 5, numel) for base, N, gdt in (("adam", 1, "f32"), ("adam", 4, "bf16"), ("adopt", 1, "bf16"),
+                                                         ("adopt", 3, "f32"), ("sgdm", 2, "f32"), ("sgdm", 3, "bf16"))
+           for numel in (150001, 200003, 300005, 700007)]
+          + [("adopt", 1, "f32", 6, 200003), ("adopt", 2, "bf16", 6, 700007), ("adopt", 1, "f32", 5, (1 << 21) + 300)])
 
 
 @pytest.mark.parametrize("base,N,gdt,M,numel,clip", [c + (clip,) for c in CASES for clip in (False, True)
