@@ -46,7 +46,8 @@ __device__ __forceinline__ void ld_shared_v(const float *p, float (&v)[V]) {
 // V = 0: a pair of half-warps takes a column a lane, one part each, joined by a
 // shuffle: twice the lanes on chains that are long and tiles that are narrow
 // (average, M = 256, n = 400k 370 -> 367 us, n = 1000 8.0 -> 6.2, M = 1024, n =
-// 100k 452 -> 378; fused, M = 100 359 -> 353).  kSplitMeansM: M from which.
+// 100k 452 -> 378; fused, M = 100 359 -> 353).  kSplitMeansM: M from which it is
+// always taken.
 constexpr int kSplitMeansM = 65;
 
 template <int V, typename TileOf>

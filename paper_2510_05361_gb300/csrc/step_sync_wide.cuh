@@ -135,38 +135,62 @@ __global__ void __launch_bounds__(kTileMaxThreads) step_sync_tile_kernel(const S
     }
 }
 
-// Columns of a tile and threads of its block.
+// Columns of a tile, threads of its block and the form of its means (tile_means'
+// V).
 struct TileShape {
-    int S, threads;
+    int S, threads, means;
     size_t smem;
 };
 
-// The shape for M replicas of n elements; bytes(S): the shared memory of a
-// tile of S columns.  Columns (fused step, GB/s): 128 up to M = 16 (M = 16,
-// Adam N = 3: 6915, 64 columns 5874, 256 5866), else 64 (M = 32: 6864, 128
-// columns 5970; M = 64, SGDM 6730, 128 columns 6541); 32 where two blocks of
-// 64 would not fit an SM (M = 64, Adam N = 4: 5928, 64 columns 4583; M = 100,
-// Adam N = 2: 5998, 16 columns 3711).  Small states, where rows count less (L2)
+// The shape for M replicas of n elements with n_due states due; bytes(S): the
+// shared memory of a tile of S columns; sgdm_n_mom: SGDM's N (its update has no
+// square root and division), else 0.
+// Columns (fused step, GB/s): 128 up to M = 16 (M = 16, Adam N = 3: 6915, 64
+// columns 5874, 256 5866), else 64 (M = 32: 6864, 128 columns 5970; M = 64, SGDM
+// 6730, 128 columns 6541); 32 where two blocks of 64 would not fit an SM (M = 64,
+// Adam N = 4: 5928, 64 columns 4583; M = 100, Adam N = 2: 5998, 16 columns
+// 3711).  Small states, where rows count less (L2)
 // and the SMs are to have tiles enough, take fewer: the half while an SM would
 // get fewer tiles than tile_min of them (us: M = 16, n = 200k, ADOPT N = 3 128
 // columns 27.8, 64 26.6; M = 47, n = 149k, ADOPT N = 2 64 columns 53.1, 32
 // 48.1, 16 48.0; M = 64, n = 60k, Adam N = 2 28.7, 23.0, 23.8; M = 24, n = 500k
 // 72.3, 71.8, 73.4; M = 44, n = 10k, ADOPT N = 3 11.3, 9.3, 8.2; M = 100, n =
 // 4k 32 columns 8.2, 16 6.2, 8 8.2; M = 256, n = 512 32 columns 12.3, 8 8.2;
-// M = 11, n = 111k, SGDM N = 4 128 columns 8.3, 32 11.8).
+// M = 11, n = 111k, SGDM N = 4 128 columns 8.3, 32 11.8; M = 64, n = 1500, SGDM N
+// = 1 and 3, ADOPT N = 4 16 columns 2.7, 3.1, 4.0, 8 2.9, 3.4, 4.3).
 // Threads: about 1024 per SM over the blocks that fit, with 2 to 4 items each
 // (M = 48, Adam N = 3: 3 items 6740, 2 items 6169; M = 9: 2 items 6508, 3
 // items 6126, 1 item 4803); two items where that deals them out evenly to 256
 // threads at most and the rule's count does not (M = 16, ADOPT, bf16: 2 items
 // 6659, 3 items 6067).
+// Means: four columns a lane where that still gives every lane one (us, one
+// column -> four: M = 4, n = 20M, Adam N = 3 599 -> 514, ADOPT N = 2 488 -> 409; M
+// = 6, ADOPT N = 2 741 -> 628; M = 12, n = 2^23 511 -> 496; but M = 8, ADOPT N =
+// 2, three states due 785 -> 793, M = 16 659 -> 671).
+// Up to 20 tiles an SM (states in L2) the other blocks do not hide a block's
+// means, and their form is chosen by the columns due against the threads (M = 9 to
+// 64; 19411 random steps of 250 elements to 30M over all replicas: 2.3 % faster in
+// the mean, up to 16 %, and 6 % slower at most):
+//   at most half as many columns, M >= 24 and tiles for few rounds (3 an SM, SGDM
+//   6): a pair of half-warps (M = 56, n = 1500, SGDM N = 1 3.4 -> 2.75; M = 64, n =
+//   5000 3.9 -> 3.15; but M = 32, n = 16k, Adam N = 2 4.55 -> 4.97);
+//   more columns than threads, and fewer items a thread (two or more) give every
+//   column a thread: those (M = 20, n = 130k, SGDM N = 1, 5 items 7.7, 3 7.1);
+//   else twice as many columns, 256 or more: four a lane (M = 15, n = 130k, SGDM N =
+//   3 12.7 -> 9.5; M = 17, n = 90k, 10.0 -> 8.6);
+//   else M <= 16, SGDM N = 1: four a lane and 96 threads (M = 9, n = 130k 5.1 ->
+//   4.4; M = 10, n = 180k 6.6 -> 5.9; with N >= 3 or more replicas it loses).
+constexpr int64_t kTilesInL2 = 20;
+
 template <typename Bytes>
-TileShape tile_shape(int M, int64_t n, int num_sms, Bytes bytes) {
+TileShape tile_shape(int M, int64_t n, int num_sms, int n_due, int sgdm_n_mom, Bytes bytes) {
     TileShape w;
     w.S = M <= 16 ? 128 : 64;
     while (w.S > 32 && 2 * (bytes(w.S) + kSharedReserved) > kSharedPerSm) w.S /= 2;
     auto tile_min = [&](int S) {
         if (M * (S / 8) >= 256 && S >= 64) return S == 128 ? 11 : 16;      // the half still has items enough
-        return S >= 32 ? 3 : 1;
+        if (S >= 32) return 3;
+        return S == 16 && M > 32 && M < kSplitMeansM ? 0 : 1;
     };
     while (w.S > 8 && (bytes(w.S) + kSharedReserved > kSharedPerSm || n / w.S < int64_t{num_sms} * tile_min(w.S)))
         w.S /= 2;
@@ -175,10 +199,33 @@ TileShape tile_shape(int M, int64_t n, int num_sms, Bytes bytes) {
     int64_t resident = (n / w.S + num_sms - 1) / num_sms;        // blocks of an SM
     if (resident > tile_blocks_fit(w.smem)) resident = tile_blocks_fit(w.smem);
     if (resident > 16) resident = 16;
+    auto threads_of = [&](int per) {
+        const int t = ((items + per - 1) / per + 31) / 32 * 32;
+        return t < kTileMaxThreads ? t : kTileMaxThreads;
+    };
     int per = static_cast<int>((items * resident + 1023) / 1024);    // items of a thread
     if (per > 2 && items % (32 * per) != 0 && items % 64 == 0 && items <= 512) per = 2;
-    w.threads = ((items + per - 1) / per + 31) / 32 * 32;
-    if (w.threads > kTileMaxThreads) w.threads = kTileMaxThreads;
+    const int columns = n_due * w.S;
+    const int64_t tiles = n / w.S;
+    w.means = M >= kSplitMeansM ? 0 : (columns >= 4 * threads_of(per) ? 4 : 1);
+    if (M >= 9 && M < kSplitMeansM && tiles < kTilesInL2 * num_sms) {
+        if (2 * columns <= threads_of(per) && M >= 24 && tiles <= int64_t{num_sms} * (sgdm_n_mom > 0 ? 6 : 3)) {
+            w.means = 0;
+        } else if (columns > threads_of(per)) {
+            int fewer = per - 1;
+            while (fewer >= 2 && threads_of(fewer) < columns) --fewer;
+            if (fewer >= 2) {
+                per = fewer;
+                w.means = 1;
+            } else if (columns >= 256 && columns >= 2 * threads_of(per)) {
+                w.means = 4;
+            } else if (sgdm_n_mom == 1 && M <= 16 && w.means == 1) {
+                if (per < (items + 95) / 96) per = (items + 95) / 96;
+                w.means = 4;
+            }
+        }
+    }
+    w.threads = threads_of(per);
     return w;
 }
 
@@ -186,7 +233,7 @@ template <int BASE, int N, int GDT, bool CLIP>
 cudaError_t launch_step_sync_tile(const StepArgs &a, int num_sms, cudaStream_t stream) {
     if (a.M > kTileMaxM) return cudaErrorNotSupported;
     const int n_due = __builtin_popcount(a.sync_mask);
-    const TileShape w = tile_shape(a.M, a.n_padded, num_sms, [&](int S) {
+    const TileShape w = tile_shape(a.M, a.n_padded, num_sms, n_due, BASE == MTDAO_BASE_SGDM ? N : 0, [&](int S) {
         return (static_cast<size_t>(tile_set_floats<BASE, N, GDT>(a.M, S)) + static_cast<size_t>(n_due) * S) *
                sizeof(float);
     });
@@ -198,14 +245,9 @@ cudaError_t launch_step_sync_tile(const StepArgs &a, int num_sms, cudaStream_t s
     if (tile_blocks_fit(w.smem) == 1 && n_due <= 2) return cudaErrorNotSupported;
     int log2_p = 0;
     while ((4 << log2_p) < w.S) ++log2_p;
-    // Means (see tile_means): four columns a lane where that still gives every
-    // lane one (us, one column -> four: M = 4, n = 20M, Adam N = 3 599 -> 514,
-    // ADOPT N = 2 488 -> 409; M = 6, ADOPT N = 2 741 -> 628; M = 12, n = 2^23 511
-    // -> 496; but M = 8, ADOPT N = 2, three states due 785 -> 793, M = 16 659 ->
-    // 671).
-    auto kernel = a.M >= kSplitMeansM              ? step_sync_tile_kernel<BASE, N, GDT, CLIP, 0>
-                  : n_due * w.S >= 4 * w.threads ? step_sync_tile_kernel<BASE, N, GDT, CLIP, 4>
-                                                 : step_sync_tile_kernel<BASE, N, GDT, CLIP, 1>;
+    auto kernel = w.means == 0   ? step_sync_tile_kernel<BASE, N, GDT, CLIP, 0>
+                  : w.means == 4 ? step_sync_tile_kernel<BASE, N, GDT, CLIP, 4>
+                                 : step_sync_tile_kernel<BASE, N, GDT, CLIP, 1>;
     if (const cudaError_t e = allow_shared(kernel, w.smem); e != cudaSuccess) return e;
     kernel<<<static_cast<unsigned>(a.n_padded / w.S), w.threads, w.smem, stream>>>(a, log2_p);
     return cudaGetLastError();

@@ -60,6 +60,11 @@ CASES = [("adam", 4, "f32", 256, 30000), ("adam", 1, "f32", 256, 512), ("sgdm", 
 CASES += ([(base, N, gdt, 5, numel) for base, N, gdt in (("adam", 1, "f32"), ("adam", 4, "bf16"), ("adopt", 1, "bf16"),
                                                          ("adopt", 3, "f32"), ("sgdm", 2, "f32"), ("sgdm", 3, "bf16"))
            for numel in (150001, 200003, 300005, 700007)]
+          # small and middle states: every form of the means, items dealt out for them
+          + [("sgdm", 1, "bf16", M, numel) for M, numel in ((9, 60001), (9, 130001), (10, 180001), (14, 90001), (20, 130001),
+                                                            (33, 200), (40, 1500), (64, 5000))]
+          + [("sgdm", 3, "f32", 15, 130001), ("sgdm", 3, "f32", 20, 60001), ("adopt", 2, "f32", 9, 60001),
+             ("adopt", 4, "bf16", 33, 250), ("adam", 3, "bf16", 24, 2000), ("adam", 1, "f32", 12, 60001)]
           + [("adopt", 1, "f32", 6, 200003), ("adopt", 2, "bf16", 6, 700007), ("adopt", 1, "f32", 5, (1 << 21) + 300)])
 
 
