@@ -32,6 +32,9 @@ def _pair(P, w, M, gdt, seed, plant=False):
         if plant:
             vals[M // 2, 5::97] = float("inf")
             vals[M - 1, 7::89] = float("nan")
+            vals[:, 11::83] *= 1e-37                   # differences and their M-th subnormal
+            vals[:, 13::79] = vals[M - 1, 13::79]      # equal replicas
+            vals[:, 17::73] = -0.0
         for e in engines:
             e.state_view(s).copy_(vals)
     g = torch.randn((M, n), device="cuda", generator=gen) * 0.01
@@ -43,7 +46,7 @@ def _same(a, b):
         x, y = a.state_view(s), b.state_view(s)
         nan = torch.isnan(x)
         assert torch.equal(nan, torch.isnan(y)), s
-        assert torch.equal(torch.where(nan, 0.0, x), torch.where(nan, 0.0, y)), s
+        assert torch.equal(x.view(torch.int32).masked_fill(nan, 0), y.view(torch.int32).masked_fill(nan, 0)), s
 
 
 # (M, numel): one tile, an SM's worth of tiles, tiles of every width; M = 6 to 8
@@ -134,8 +137,10 @@ def test_average_on_tiles(P, M, numel):
         got = a.state_view(s).cpu().numpy()
         nan = np.isnan(ref[s])
         assert np.array_equal(np.isnan(got), np.broadcast_to(nan, got.shape)), s
-        assert np.array_equal(got[:, ~nan], np.broadcast_to(ref[s][~nan], got[:, ~nan].shape)), s
-    assert torch.equal(torch.nan_to_num(a.state_view(1)), torch.nan_to_num(b.state_view(1)))
+        want = np.broadcast_to(ref[s][~nan], got[:, ~nan].shape)
+        assert np.array_equal(got[:, ~nan].view(np.uint32), np.ascontiguousarray(want).view(np.uint32)), s
+    x, y = a.state_view(1), b.state_view(1)
+    assert torch.equal(x.view(torch.int32).masked_fill(torch.isnan(x), 0), y.view(torch.int32).masked_fill(torch.isnan(y), 0))
     a.close()
     b.close()
 
