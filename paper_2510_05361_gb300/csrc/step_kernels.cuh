@@ -198,8 +198,17 @@ __global__ void __launch_bounds__(kThreads) step_kernel(const StepArgs a) {
 // -> this: Adam N = 2, M = 4, n = 5k 6.1 -> 5.0 us; ADOPT N = 4, n = 20k 6.2 ->
 // 4.8; Adam N = 3, n = 60k 6.1 -> 4.9; n = 200k (41 warps an SM) 6.2 -> 6.0.
 constexpr int kSmallThreads = 64;
-constexpr int64_t kSmallWarps = 64;      // warps an SM takes at once
 constexpr int kSmallChunk = 128;         // elements of one warp
+
+// Warps an SM up to which it is taken: all that it holds, fewer where there is so
+// little to load that step_kernel catches up before (device time alone, us,
+// step_kernel / this, at 28, 38, 54 and 64 warps an SM of 152): SGDM N = 1 2.09 /
+// 2.09, 2.44 / 2.51, 2.88 / 3.16, 2.90 / 3.57; SGDM N = 2 at 54 3.67 / 3.40, 64
+// 3.70 / 3.81; Adam N = 1 3.84 / 3.68, 3.91 / 4.08; Adam N = 2 4.34 / 4.33, 4.55 /
+// 4.70; Adam N = 3 at 64 5.33 / 5.36, ADOPT N = 1, 4 4.83 / 4.69, 6.90 / 6.35.
+template <int BASE, int N>
+constexpr int64_t kSmallWarps = BASE == MTDAO_BASE_SGDM && N == 1 ? 28
+                                : BASE != MTDAO_BASE_ADOPT && N <= 2 ? 54 : 64;
 
 template <int BASE, int N, int GDT, bool CLIP>
 __global__ void __launch_bounds__(kSmallThreads) step_small_kernel(const StepArgs a) {
@@ -261,7 +270,7 @@ inline int stream_grid(int64_t n_warp_items) {
 
 template <int BASE, int N, int GDT, bool CLIP>
 cudaError_t launch_step_t(const StepArgs &a, int num_sms, cudaStream_t stream) {
-    if (a.stride <= kSmallWarps * num_sms * kSmallChunk) {
+    if (a.stride <= kSmallWarps<BASE, N> * num_sms * kSmallChunk) {
         const int64_t threads = a.stride / kSmallChunk * 32;
         step_small_kernel<BASE, N, GDT, CLIP>
             <<<static_cast<unsigned>((threads + kSmallThreads - 1) / kSmallThreads), kSmallThreads, 0, stream>>>(a);
