@@ -444,18 +444,39 @@ __global__ void __launch_bounds__(kThreads) sync_stats_kernel(const __grid_const
 }
 
 // stats[row * Q + q] = the sum over blocks of partial[(row * Q + q) * blocks + b]
-// in fp64: thread t of block (q, row) adds blocks t, t + 256, ... in order, then
-// block_sum adds the threads' sums in a fixed order.  q = 0 is divided by
-// divide_first (M for the variance, a mean over workers; 0 leaves it).
+// in fp64, WARPS warps a sum: thread t of them adds blocks t, t + 32 WARPS, ... in
+// order, then the lanes and the warps are added in a fixed order.  q = 0 is divided
+// by divide_first (M for the variance, a mean over workers; 0 leaves it).
+template <int WARPS>
 __global__ void __launch_bounds__(kNormThreads) stats_finalize_kernel(const double *partial, int64_t blocks, int Q,
-                                                                      int divide_first, double *stats) {
-    const int q = blockIdx.x, row = blockIdx.y;
-    const double *p = partial + (static_cast<int64_t>(row) * Q + q) * blocks;
+                                                                      int n_sums, int divide_first, double *stats) {
+    const int sum = WARPS == 1 ? static_cast<int>((blockIdx.x * kNormThreads + threadIdx.x) >> 5) : blockIdx.x;
+    const int t = WARPS == 1 ? threadIdx.x & 31 : threadIdx.x;
+    if (sum >= n_sums) return;
+    const double *p = partial + static_cast<int64_t>(sum) * blocks;
     double acc = 0.0;
 #pragma unroll 4
-    for (int64_t b = threadIdx.x; b < blocks; b += kNormThreads) acc += p[b];
-    const double total = block_sum(acc);
-    if (threadIdx.x == 0) stats[row * Q + q] = (q == 0 && divide_first > 0) ? total / divide_first : total;
+    for (int64_t b = t; b < blocks; b += 32 * WARPS) acc += p[b];
+    const double total = WARPS == 1 ? warp_sum(acc) : block_sum(acc);
+    if (t == 0) stats[sum] = (divide_first > 0 && sum % Q == 0) ? total / divide_first : total;
+}
+
+// A block for each sum, or a warp where there are many sums of few blocks: adding
+// the lanes and warps of a block is 48 fp64 instructions, 16 cycles of the SM each,
+// against blocks / 32 (average with sums, us, a block / a warp each, in brackets
+// sums and blocks: M = 1024, n = 1219, 5 states (10250, 160) 73 / 46; M = 200, n =
+// 30k, 3 states (1206, 473) 40.6 / 37.7; M = 64, n = 300, 5 states (650, 40) 7.6 /
+// 6.3; but n = 286k, 4 states (520, 559) 112 / 114).
+cudaError_t launch_finalize(const double *partial, int64_t blocks, int Q, int rows, int divide_first, double *stats,
+                            cudaStream_t stream) {
+    const int n_sums = Q * rows;
+    if (n_sums >= 256 && blocks <= (n_sums >= 1024 ? 1024 : 256))
+        stats_finalize_kernel<1><<<(n_sums + 7) / 8, kNormThreads, 0, stream>>>(partial, blocks, Q, n_sums,
+                                                                               divide_first, stats);
+    else
+        stats_finalize_kernel<kNormThreads / 32><<<n_sums, kNormThreads, 0, stream>>>(partial, blocks, Q, n_sums,
+                                                                                     divide_first, stats);
+    return cudaGetLastError();
 }
 
 int64_t stats_blocks(int64_t n_padded, int tile) {
@@ -497,8 +518,7 @@ cudaError_t launch_sync_stats_t(const SyncArgs &a, double *partial, size_t parti
     sync_stats_kernel<M><<<grid, kThreads, 0, stream>>>(a, tile, partial);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    stats_finalize_kernel<<<dim3(Q, a.n_sel), kNormThreads, 0, stream>>>(partial, gx, Q, M, stats);
-    return cudaGetLastError();
+    return launch_finalize(partial, gx, Q, a.n_sel, M, stats, stream);
 }
 
 // Pseudo-gradient diagnostics of the parameters x[M][n] against the anchor
@@ -562,8 +582,7 @@ cudaError_t launch_pseudo_grad_stats_t(const float *x, const float *anchor, int6
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     // the same fixed-order finalisation as the sync diagnostics, with no division
-    stats_finalize_kernel<<<dim3(Q, 1), kNormThreads, 0, stream>>>(partial, gx, Q, 0, stats);
-    return cudaGetLastError();
+    return launch_finalize(partial, gx, Q, 1, 0, stats, stream);
 }
 
 // ---------------------------------------------------------------- diagnostics, replicas streamed
@@ -753,10 +772,10 @@ cudaError_t launch_sync_stats_stream(const SyncArgs &a, int num_sms, float *mean
         stream_stats_pass1_kernel<false><<<g.b1, kThreads, 0, stream>>>(s, nullptr, a.n_padded, M, mean, a.anchor[k], p1);
         stream_sync_stats_pass2_kernel<<<dim3(g.b2, M), kThreads, 0, stream>>>(s, a.n_padded, mean, p2);
         // stats row: [0] variance (over all replicas' blocks), [1] s_bar^2, [2 + m] s_m^2, [2 + M + m] s_m s_bar
-        stats_finalize_kernel<<<1, kNormThreads, 0, stream>>>(p2, per_sum, 1, M, stats);
-        stats_finalize_kernel<<<1, kNormThreads, 0, stream>>>(p1, g.b1, 1, 0, stats + 1);
-        stats_finalize_kernel<<<2 * M, kNormThreads, 0, stream>>>(p2 + per_sum, g.b2, 2 * M, 0, stats + 2);
-        const cudaError_t e = cudaGetLastError();
+        cudaError_t e = cudaGetLastError();
+        if (e == cudaSuccess) e = launch_finalize(p2, per_sum, 1, 1, M, stats, stream);
+        if (e == cudaSuccess) e = launch_finalize(p1, g.b1, 1, 1, 0, stats + 1, stream);
+        if (e == cudaSuccess) e = launch_finalize(p2 + per_sum, g.b2, 2 * M, 1, 0, stats + 2, stream);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -771,9 +790,10 @@ cudaError_t launch_pseudo_grad_stats_stream(const float *x, const float *anchor,
     stream_stats_pass1_kernel<true><<<g.b1, kThreads, 0, stream>>>(x, anchor, n, M, mean, nullptr, p1);
     stream_change_pass2_kernel<<<dim3(g.b2, M), kThreads, 0, stream>>>(x, anchor, n, mean, p2);
     // [m] (x_m - a)^2, [M + m] (x_m - a)(x_bar - a), [2M] (x_bar - a)^2, [2M + 1] a^2
-    stats_finalize_kernel<<<2 * M, kNormThreads, 0, stream>>>(p2, g.b2, 2 * M, 0, stats);
-    stats_finalize_kernel<<<2, kNormThreads, 0, stream>>>(p1, g.b1, 2, 0, stats + 2 * M);
-    return cudaGetLastError();
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = launch_finalize(p2, g.b2, 2 * M, 1, 0, stats, stream);
+    if (e == cudaSuccess) e = launch_finalize(p1, g.b1, 2, 1, 0, stats + 2 * M, stream);
+    return e;
 }
 
 cudaError_t launch_pseudo_grad_stats(const float *x, const float *anchor, int64_t n, int M, int num_sms,
@@ -874,8 +894,7 @@ cudaError_t launch_grad_sqnorm(const void *grads, int grad_dtype, int32_t M, int
 
 cudaError_t launch_stats_finalize(const double *partial, int64_t blocks, int Q, int rows, int divide_first,
                                   double *stats, cudaStream_t stream) {
-    stats_finalize_kernel<<<dim3(Q, rows), kNormThreads, 0, stream>>>(partial, blocks, Q, divide_first, stats);
-    return cudaGetLastError();
+    return launch_finalize(partial, blocks, Q, rows, divide_first, stats, stream);
 }
 
 }  // namespace mtdao
