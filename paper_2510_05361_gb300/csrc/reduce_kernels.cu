@@ -744,7 +744,7 @@ StreamGrid stream_grid2(int num_sms, int M, int64_t n) {
 //   316, 117k 471 / 404, 391k 1514 / 848; change n = 59k 226 / 279, 117k 409 /
 //   326, 781k 2413 / 1159.
 //   32 columns: change M = 512 234k 206 / 220, 391k 325 / 294, 1.6M 1162 / 1060; M
-//   = 768 260k 399 / 382, 1.0M 1384 / 1230; average with sums M = 896 223k 490 /
+//   = 600 267k 349 / 260, M = 768 156k 268 / 297, 260k 399 / 382, 1.0M 1384 / 1230; average with sums M = 896 223k 490 /
 //   518, 446k 1025 / 854; M = 768 521k 994 / 862; M = 640 312k 532 / 482, three
 //   states 1472 / 1441.  Up to M = 598 three tiles fit an SM: M = 512 781k 821 /
 //   921.
@@ -752,7 +752,7 @@ StreamGrid stream_grid2(int num_sms, int M, int64_t n) {
 bool stream_stats(int M, int64_t n, bool change) {
     if (M < 450) return false;
     if (M > 898) return n >= (change ? 81920 : 98304);
-    return change ? n >= 262144 : M >= 599 && n >= 393216;
+    return change ? n >= (M < 599 ? 262144 : 196608) : M >= 599 && n >= 393216;
 }
 
 size_t stream_stats_partial_capacity(int num_sms, int64_t n_padded, int M) {

@@ -175,7 +175,8 @@ struct StatsTileShape {
 //   4M: 781 -> 612; M = 64, n = 2M: 709 -> 617; M = 128, n = 600k: 1102 -> 497; M
 //   = 256, n = 400k: 1073 -> 635), 32 above, where 64 leave an SM two or three
 //   small blocks (change, M = 320, n = 1.25M 911 -> 553, M = 257, n = 3.1M 1339
-//   -> 1022; average with sums, M = 384, n = 521k, 3 states 1457 -> 1044); fewer
+//   -> 1022; average with sums, M = 384, n = 521k, 3 states 1457 -> 1044) but
+//   for small states (change, M = 257, n = 29k 64 columns 19, 32 24); fewer
 //   where two tiles would not fit an SM or the SMs would not have one each.
 //   Lanes and threads: the fewer, the more rows a thread takes and the less
 //   there is to combine at a run's end (M = 64, means by lane pairs: 2 lanes and
@@ -188,7 +189,7 @@ struct StatsTileShape {
 StatsTileShape stats_tile_shape(int num_sms, int64_t n, int n_sel, int M) {
     StatsTileShape w;
     auto bytes = [&](int log2_s) { return static_cast<size_t>(M + 2) * sizeof(float) << log2_s; };
-    w.log2_s = M <= 12 ? 8 : (M <= 16 ? 7 : (M <= 256 ? 6 : 5));
+    w.log2_s = M <= 12 ? 8 : (M <= 16 ? 7 : (M <= 256 || (n >> 6) * n_sel < 4 * num_sms ? 6 : 5));
     while (w.log2_s > 3 &&
            (2 * (bytes(w.log2_s) + kSharedReserved) > kSharedPerSm || (n >> w.log2_s) * n_sel < num_sms))
         --w.log2_s;

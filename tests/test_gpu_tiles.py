@@ -210,7 +210,7 @@ def test_diagnostics_on_tiles(P, M, numel):
     b.close()
 
 
-@pytest.mark.parametrize("M,numel", [(449, 270001), (450, 262000), (450, 262145), (599, 393217), (898, 270000),
+@pytest.mark.parametrize("M,numel", [(449, 270001), (450, 262000), (450, 262145), (599, 196607), (599, 393217), (898, 270000),
                                      (899, 81900), (899, 82001), (1024, 98305)])
 def test_streamed_diagnostics(P, M, numel):
     """Both sides of the limits above which many replicas are streamed in two passes
