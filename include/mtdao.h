@@ -245,8 +245,9 @@ int mtdao_set_params(mtdao_handle h, const float *x0_dev);
  *   step (E_m[.] of Algorithm 1); usually the value of mtdao_sync_due.  The
  *   average is fused into the step's pass: it costs no extra HBM traffic for
  *   2 <= M <= 256 (from M = 9, and on most large states, a block stages a
- *   tile of all replicas in shared memory); larger M, and a few states due
- *   where one tile fills an SM, take a separate averaging pass.
+ *   tile of all replicas in shared memory), but for the copy of a tracked
+ *   anchor (8 bytes per element); larger M, and a few states due where one
+ *   tile fills an SM, take a separate averaging pass.
  * With MTDAO_CLIP_GLOBAL_NORM a reduction pass over grads precedes the step.
  * With adopt_prev_v (the original ADOPT order) step 0 runs a separate pass
  * that writes v = g_0^2 and reads or writes nothing else, so u and x keep
@@ -317,11 +318,17 @@ int mtdao_sync(mtdao_handle h, uint32_t mask);
  * fixed-order (bit-reproducible).  With M = 1 the states are left as they
  * are and only the diagnostics are written.  The sums are formed in the
  * averaging pass itself (the sync's traffic, 8 M bytes per element and
- * state; from M = 9 a block stages a tile of all replicas in shared memory).
+ * state; from M = 9 a block stages a tile of all replicas in shared memory);
+ * large states of some 600 replicas and more (900 and more: from 100k
+ * elements) take two passes through a library-owned [n_padded] fp32 scratch
+ * that holds the mean (12 M bytes), and so does the change diagnostics from
+ * 450 replicas.
  * Every path forms (s_m - s_bar) against the fp32 mean it stores, sums a
  * thread's elements in fp32 with Kahan compensation, a warp's sums as
  * compensated pairs (in fp64 where they pass fp32's range) and those of warps
- * and blocks in fp64.  The workspace is allocated on the first call.
+ * and blocks in fp64: a sum is finite as long as the squares of a thread's
+ * elements (some hundreds) add up to less than 3.4e38.  The workspace is
+ * allocated on the first call.
  */
 int mtdao_sync_stats(mtdao_handle h, uint32_t mask, double *stats_dev);
 
@@ -350,7 +357,7 @@ int mtdao_track_anchor(mtdao_handle h, uint32_t state_mask);
  * so cos(local, global) = [M+m] / sqrt([m] [2M]) and the relative change of
  * the averaged state over the round = sqrt([2M] / [2M+1]).  Call it before
  * the round's average of that state.  MTDAO_ERR_STATE if the state has no
- * anchor.  One read-only pass, with the workspace of mtdao_sync_stats.
+ * anchor.  Read-only, one pass or two, with the workspace of mtdao_sync_stats.
  */
 int mtdao_pseudo_grad_stats(mtdao_handle h, int32_t state, double *out_dev);
 

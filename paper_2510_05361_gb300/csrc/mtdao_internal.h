@@ -112,7 +112,7 @@ size_t sync_stats_partial_capacity(int num_sms, int64_t n_padded, int n_states, 
 cudaError_t launch_sync_stats(const SyncArgs &a, int num_sms, double *partial, size_t partial_cap,
                               double *stats, cudaStream_t stream);
 
-// The diagnostics for more replicas (9 to MTDAO_MAX_REPLICAS): same outputs as
+// The diagnostics for more replicas (9 to MTDAO_MAX_REPLICAS), on tiles: same outputs as
 // launch_sync_stats / launch_pseudo_grad_stats, the averaged states
 // bit-identical to launch_sync's.  Workspace: partial needs
 // tile_stats_partial_capacity() doubles.

@@ -73,19 +73,4 @@ __device__ __forceinline__ float replica_mean(Get get) {
     return plain / static_cast<float>(M);
 }
 
-// Same, for a replica count known only at run time.
-template <typename Get>
-__device__ __forceinline__ float replica_mean_rt(int M, Get get) {
-    const int h = M / 2;
-    const float s0 = get(0);
-    DiffSum a(s0), b(s0);
-    for (int m = 1; m < h; ++m) a.add(get(m));
-    for (int m = (h > 1 ? h : 1); m < M; ++m) b.add(get(m));
-    const float mean = replica_mean_from_parts(s0, a.partial(), b.partial(), static_cast<float>(M));
-    if (mean == mean) return mean;
-    float plain = s0;
-    for (int m = 1; m < M; ++m) plain += get(m);
-    return plain / static_cast<float>(M);
-}
-
 }  // namespace mtdao

@@ -1,5 +1,6 @@
 // stats_wide.cu -- the cross-worker diagnostics of section 4.1 for more
-// replicas than a thread holds (9 <= M <= 1024).
+// replicas than a thread holds (9 <= M <= 1024; large states of 450 replicas and
+// more are streamed, reduce_kernels.cu).
 //
 // A block takes a run of consecutive tiles, S columns of all M replicas each:
 // copies a tile to shared memory (cp.async), forms its replica means
@@ -183,9 +184,11 @@ struct StatsTileShape {
 //   128 threads 639, 8 lanes 683, 512 threads 1120).
 //   Tiles: runs enough for 8 blocks an SM, 8 at most, so that the tiles under
 //   way lie close together (M = 64: 640, runs of 32 675; M = 100, n = 75k, runs
-//   of 1 to 2: 231 -> 56, of 32 254); as many columns where the tiles are
-//   narrower, which keeps the workspace under 1 % of the states (M = 1024, n =
-//   100k: 1305 -> 998 in runs of 6, 1033 of 12).
+//   of 1 to 2: 231 -> 56, of 32 254); as many columns (512) where the tiles are
+//   narrower (M = 1024, n = 100k: 1305 -> 998 in runs of 6, 1033 of 12).
+//   Workspace: 16 bytes a run and replica, under 1 % of the states in runs of 512
+//   columns, more on small states (6 % at M = 100, n = 75k with runs of one tile of
+//   64 columns, half of them with tiles of 8).
 StatsTileShape stats_tile_shape(int num_sms, int64_t n, int n_sel, int M) {
     StatsTileShape w;
     auto bytes = [&](int log2_s) { return static_cast<size_t>(M + 2) * sizeof(float) << log2_s; };

@@ -20,6 +20,12 @@
 // here (5 blocks, one gradient ahead; 117-121 with 4 to 6 blocks and two to
 // four gradients ahead).  The averages in the same kernel (a block
 // of M warps, the due states meeting in shared memory) took 141 to 166.
+// 48 registers spill 44 to 84 bytes for Adam with N = 3 and 4, 16 to 32 for ADOPT,
+// which costs less than the fifth block brings on large states (M = 4, us, single
+// steps / 5 / 4 blocks: rounds of 16, n = 2^20 Adam N = 3 393 / 114 / 111, N = 4 532
+// / 129 / 124, ADOPT N = 3 408 / 124 / 125, N = 4 529 / 136 / 137, SGDM N = 4 364 /
+// 71 / 71; of 4, n = 30M Adam N = 3 3025 / 1533 / 1554, ADOPT N = 3 3053 / 1533 /
+// 1581).
 #pragma once
 
 #include "step_kernels.cuh"

@@ -141,7 +141,7 @@ WORKLOADS = {
         "name": "profile_small_m16",
         "desc": "flat fp32 vector n=2^23 with M=16 replicas and the ~1B workload's optimizer "
                 "(N=3 beta=(0.5,0.9,0.999), Adam, grads N(0,1e-3) with 1% outliers x100, "
-                "H=32): the block-staged fused step and one-pass diagnostics on ~3 GB of "
+                "H=32): the tiled fused step and one-pass diagnostics on ~3 GB of "
                 "device memory, for profiler captures",
         "shapes": [1 << 23],
         "M": 16,

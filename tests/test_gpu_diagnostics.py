@@ -35,10 +35,9 @@ def _fill(eng, rng, spread):
 
 @pytest.mark.parametrize("M", [1, 2, 3, 4, 8, 9, 16, 32, 33, 37, 64, 65, 100, 256, 300, 1024])
 def test_sync_stats_match_oracle_and_plain_sync(P, M):
-    """M <= 8: one pass with the replicas in registers; 9 <= M <= 64: one
-    pass with a span of all replicas staged in shared memory (four-column
-    means up to 32); M > 64: two passes through a scratch mean.  All match the oracle's definitions and
-    leave the states bit-identical to the plain average."""
+    """M <= 8: the replicas in registers; above: tiles of all replicas in shared
+    memory.  All match the oracle's definitions and leave the states bit-identical
+    to the plain average."""
     shapes = [70001, 999, 4096] if M <= 37 else [7001, 99, 1024]
     w = workload_dict(shapes, M, betas=(0.9, 0.99))
     a = P.MTDAO(w["opt"], M, shapes)
@@ -76,11 +75,9 @@ def test_sync_stats_match_oracle_and_plain_sync(P, M):
 
 @pytest.mark.parametrize("M", [4, 12, 40])
 def test_one_pass_diagnostics_over_many_spans(P, M):
-    """Large lists: the one-pass diagnostics for 9 <= M <= 64 run a
-    persistent grid whose blocks take many spans each (2^21 elements), the
-    next span's copy in flight while the current one is summed; for M = 4
-    the sync diagnostics run 264 tile blocks per state, so the finalize adds
-    runs of block rows per thread, and the pseudo-gradient pass runs its
+    """Large lists: for M = 12 and 40 every block takes a run of eight tiles (2^21
+    elements); for M = 4 the sync diagnostics leave 2112 rows per state, so the
+    finalize adds eight or nine a thread, and the pseudo-gradient pass runs its
     whole persistent grid.  Sums match the oracle's definitions, the averaged
     states equal the plain average bit for bit."""
     from oracle.oracle import pseudo_grad_stats

@@ -112,12 +112,11 @@ def test_fused_sync_is_bitwise_equal_to_separate_sync(P, M, gdt):
 
 @pytest.mark.parametrize("M", range(2, 71))
 def test_fused_equals_separate_for_every_replica_count(P, M):
-    """Every M from 2 to 70 crosses each switch between averaging paths:
-    lane groups (M <= 8), the block-staged fused step (9..64; one or two
-    float4 positions per thread at 16/17, four-column or one-column means at
-    32/33), step + average above 64, and the standalone average in registers
-    (M <= 14) or streamed.  Fused and separate averaging agree bit for bit,
-    and the averaged states equal the oracle within the tolerance."""
+    """Every M from 2 to 70 crosses the switches between averaging paths on small
+    states: lane groups (M <= 8) and tiles of all replicas in the fused step (the
+    means by pairs of half-warps from M = 24 on, always from 65), the standalone
+    average in registers (M <= 14) or on tiles.  Fused and separate averaging agree
+    bit for bit, and the averaged states equal the oracle within the tolerance."""
     w = workload_dict([700, 300, 24], M, base="adam", betas=(0.9, 0.99), px=2, pu=[3, 2], pv=3, gdt="f32")
     a = gpu_run(P, w, 6, fused=True)
     b = gpu_run(P, w, 6, fused=False)
@@ -506,7 +505,7 @@ def test_nonfinite_gradients_propagate_like_the_oracle(P, variant, gdt, sync, t_
     (step 0 only sets v = g_0^2, Algorithm 2 read as the original method)
     must leave u and x finite when step 0's gradient is not.  An infinite
     state stays infinite at the next steps (beta * inf = inf), M = 12 runs
-    the fused average of the block-staged kernel."""
+    the fused average on tiles."""
     period = {"plain": 0, "fused_every2": 2, "fused_every1": 1}[sync]
     kw = dict(NONFINITE_VARIANTS[variant])
     w = workload_dict([1000, 37], M, betas=(0.9, 0.99), px=period, pu=period, pv=period, gdt=gdt,

@@ -89,6 +89,6 @@ def test_random_configuration_parity(P, case):
 
 @pytest.mark.parametrize("case", range(96, 120))
 def test_random_configuration_parity_wide(P, case):
-    """The same draws with replica counts on both sides of the block-staged
-    fused step's layout switches (10, 24, 40, 64)."""
+    """The same draws with replica counts on both sides of the switches of the
+    tiled fused step's shape (10, 24, 40, 64)."""
     run_case(P, *draw(case, replica_counts=[10, 24, 40, 64]))

@@ -16,7 +16,7 @@ pytestmark = pytest.mark.gpu
 POINTS = ([(M, N, 8) for M in (1, 2, 4, 8) for N in (1, 2, 3, 4)]
           + [(M, 1, 1) for M in (1, 2, 4, 8)]
           + [(4, 2, 64), (8, 4, 64), (2, 3, 1)]
-          + [(12, 1, 8), (16, 3, 8), (32, 2, 8), (64, 4, 1)])   # the block-staged fused step
+          + [(12, 1, 8), (16, 3, 8), (32, 2, 8), (64, 4, 1)])   # the tiled fused step
 
 
 @pytest.fixture(scope="module")
@@ -37,10 +37,9 @@ def test_sweep_point_parity(P, M, N, H):
 
 
 @pytest.mark.parametrize("M,N,H,base", [(16, 2, 4, "adopt"), (24, 3, 4, "adam"), (40, 1, 2, "sgdm")])
-def test_block_staged_fused_step_bf16_many_spans(P, M, N, H, base):
-    """bf16 gradients through the block-staged fused step with 2^20 elements
-    per replica: every persistent block walks many spans, each span's
-    gradient tile copied 8 bytes at a time while the previous one is used."""
+def test_tiled_fused_step_bf16_many_tiles(P, M, N, H, base):
+    """bf16 gradients through the tiled fused step with 2^20 elements per replica:
+    8192 tiles of 128 columns or more, the gradient's copied 8 bytes at a time."""
     w = W.sweep_point(20, M, N, H, base=base)
     w["grad_dtype"] = "bf16"
     run_point(P, w, M, N, H)

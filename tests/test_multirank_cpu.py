@@ -142,7 +142,7 @@ def test_clock_sample_summary():
 def test_sweep_options(monkeypatch):
     """bench.py --sweep visits M in {1,2,4,8} and N in {1..4} unless told
     otherwise; --sweep-M / --sweep-N take other replica and momentum counts
-    (the block-staged fused step's range, for instance)."""
+    (those of the tiled fused step, for instance)."""
     sys.path.insert(0, ROOT)
     import bench
     monkeypatch.setattr("sys.argv", ["bench.py", "--sweep"])
